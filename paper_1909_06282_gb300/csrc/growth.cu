@@ -163,19 +163,47 @@ __host__ __device__ inline D2Geo d2_geo(int variant) {
   return g;
 }
 
-// GEO 0: r = 1, c = 0 (T1, Winther, GR): one extra chain, the T1 braces mu - B.
-// GEO 1: r = 1, c != 0: one extra chain (k1 = k2), full braces.
-// GEO 2: r != 1: chains at k1 and k2, full braces.
-template <int GEO> struct Layout {
-  static constexpr int NB = GEO == 2 ? 8 : 6;   // states per set: D1, D1s, Da, Das, (Db, Dbs,) D2, D2s
-  static constexpr int A = 2, B = GEO == 2 ? 4 : 2, D2 = GEO == 2 ? 6 : 4;
+// GEO 0: r = 1, c = 0 (T1, Winther, GR): the T1 braces mu - B.
+// GEO 1: r = 1, c != 0: k1 = k2, full braces.
+// GEO 2: r != 1: full braces at k1 and k2.
+//
+// The integration.  Per k there are eight second-order chains
+//   y_ss = -damp y_s + c(s) y + src(s):
+// D1(k), Da = D1(k1), Db = D1(k2) (no source); D2 (source: -W Pa Pb) and the ln|fR0| tangents
+// Z1, Za, Zb (source: T times the chain's own primal); Z2 (source: T2 D2 - W (Pat Pb + Pa Pbt)
+// - Wt Pa Pb).  One warp integrates four k, a lane per chain.
+//
+// What bounds it: an FP64 instruction occupies an SM sub-partition of this GPU for 64 cycles
+// whatever the active lanes (measured: 64.3 cycles per dependent or independent DFMA), so the
+// time is the number of FP64 instructions a warp issues per step.  A lane does only what
+// depends on its own state, 21 of them: the coefficients, which depend on (k, a) alone, and the
+// sources, which depend on chains integrated earlier, come from the block's other three warps
+// (one per remaining sub-partition) through shared memory.  The lanes of one warp are at
+// different times: a level (primal chains; D2 and the first tangents; Z2) runs two chunks of
+// GR_CH steps behind the one whose stage values its sources need, so in an iteration the chain
+// warp advances level l by chunk it - 2 l while the other warps fill the coefficients of chunk
+// it + 1, the level-1 sources of chunk it - 1 and the level-2 sources of chunk it - 3.
+// Measured (512 k, 1024 steps): 12.4 ms with a thread per k doing all of it, 0.87 ms now (the
+// chain warp alone would take 0.76 ms: 21 instructions x 64 cycles x 1056 steps).
+constexpr int GR_KPB = 4;            // k per block: 4 x 8 chains fill the chain warp
+constexpr int GR_CH = 8;             // RK4 steps per chunk
+constexpr int GR_HS = 2 * GR_CH + 1; // half steps of a chunk, both ends included
+constexpr int GR_THREADS = 128;      // the chain warp and three warps for coefficients and sources
+constexpr int GR_NC = 10;            // coefficients per (half step, k): c x 4, tangent x 4, W, Wt
+constexpr int GR_VRING = 4, GR_SRING = 2, GR_CRING = 6;   // chunks kept: stage values, sources, coefficients
+enum { CH_D1 = 0, CH_DA = 1, CH_DB = 2, CH_D2 = 3, CH_Z1 = 4, CH_ZA = 5, CH_ZB = 6, CH_Z2 = 7 };
+struct GrowthSmem {
+  double val[GR_VRING][GR_CH][4][32];             // y at the four stages of each step, per chain lane
+  double src[GR_SRING][GR_CH][4][32];             // h^2 src at the four stages
+  double coef[GR_CRING][GR_HS][GR_KPB][GR_NC];    // h^2 times the coefficients
+  double damp[GR_CRING][GR_HS];                   // -h damp
+  double red[8][4];                               // norm reduction
+  double out[32];
 };
 
-// right-hand side; y = [set] (+ [tangent set] when TAN)
-template <bool TAN, int GEO>
-__device__ __forceinline__ void rhs(const Bg& b, double k2, bool gr, const D2Geo& g, const double* y, double* dy) {
-  using L = Layout<GEO>;
-  constexpr int T = L::NB;
+// Coefficients of (k, half step), times h2: c of D1, Da, Db, D2; their tangents; W, Wt.
+template <int GEO>
+__device__ __forceinline__ void growth_coef(const Bg& b, double k2, bool gr, const D2Geo& g, double h2, double* o) {
   const double q = k2 * b.inv_a2, qa = q * g.fa, qb = q * g.fb;
   double mu_k = 1.0, mu_a = 1.0, mu_b = 1.0, mu_kt = 0.0, mu_at = 0.0, mu_bt = 0.0, br = 1.0, brt = 0.0;
   if (!gr) {
@@ -184,150 +212,232 @@ __device__ __forceinline__ void rhs(const Bg& b, double k2, bool gr, const D2Geo
     mu_k = 1.0 + q * rpk * (1.0 / 3.0);
     mu_a = 1.0 + qa * rpa * (1.0 / 3.0);
     mu_b = GEO == 2 ? 1.0 + qb * rpb * (1.0 / 3.0) : mu_a;
+    mu_kt = q * b.m2 * rpk * rpk * (1.0 / 3.0);
+    mu_at = qa * b.m2 * rpa * rpa * (1.0 / 3.0);
+    mu_bt = GEO == 2 ? qb * b.m2 * rpb * rpb * (1.0 / 3.0) : mu_at;
     const double B = b.bfac * q * rpk * rpa * rpb;
-    if (TAN) {
-      mu_kt = q * b.m2 * rpk * rpk * (1.0 / 3.0);
-      mu_at = qa * b.m2 * rpa * rpa * (1.0 / 3.0);
-      mu_bt = GEO == 2 ? qb * b.m2 * rpb * rpb * (1.0 / 3.0) : mu_at;
-    }
     if (g.gr2) {             // the GR D2 variant: mu = 1 in its chains and equation
       mu_a = mu_b = 1.0;
       mu_at = mu_bt = 0.0;
     } else if (GEO == 0) {
       br = mu_k - B;
-      if (TAN) brt = mu_kt - B * (-2.0 + b.m2 * rpk + 2.0 * b.m2 * rpa);
+      brt = mu_kt - B * (-2.0 + b.m2 * rpk + 2.0 * b.m2 * rpa);
     } else {
-      const double G = b.m2 * rpk;
+      const double G = b.m2 * rpk, Gt = -G * q * rpk;
       const double lin = 2.0 * g.c2 * (mu_a + mu_b - 2.0) + (g.c / g.r) * (mu_a - 1.0) + g.r * g.c * (mu_b - 1.0);
+      const double lint = 2.0 * g.c2 * (mu_at + mu_bt) + (g.c / g.r) * mu_at + g.r * g.c * mu_bt;
+      const double Bt = B * (-2.0 + b.m2 * rpk + b.m2 * rpa + b.m2 * rpb);
       br = (mu_k - g.c2 * (mu_a + mu_b - mu_k) + G * lin - B) * g.inv_s2;
-      if (TAN) {
-        const double Gt = -G * q * rpk;
-        const double lint = 2.0 * g.c2 * (mu_at + mu_bt) + (g.c / g.r) * mu_at + g.r * g.c * mu_bt;
-        const double Bt = B * (-2.0 + b.m2 * rpk + b.m2 * rpa + b.m2 * rpb);
-        brt = (mu_kt - g.c2 * (mu_at + mu_bt - mu_kt) + Gt * lin + G * lint - Bt) * g.inv_s2;
-      }
+      brt = (mu_kt - g.c2 * (mu_at + mu_bt - mu_kt) + Gt * lin + G * lint - Bt) * g.inv_s2;
     }
   }
-  const double mu_2 = g.gr2 ? 1.0 : mu_k, mu_2t = g.gr2 ? 0.0 : mu_kt;
-  // D1(k1) D1(k2) of the source (Winther: D1(k)^2)
-  const double Pa = g.winther ? y[0] : y[L::A], Pb = g.winther ? y[0] : y[L::B];
-  dy[0] = y[1];
-  dy[1] = -b.damp * y[1] + b.cc * mu_k * y[0];
-  dy[L::A] = y[L::A + 1];
-  dy[L::A + 1] = -b.damp * y[L::A + 1] + b.cc * mu_a * y[L::A];
-  if (GEO == 2) {
-    dy[L::B] = y[L::B + 1];
-    dy[L::B + 1] = -b.damp * y[L::B + 1] + b.cc * mu_b * y[L::B];
-  }
-  dy[L::D2] = y[L::D2 + 1];
-  dy[L::D2 + 1] = -b.damp * y[L::D2 + 1] + b.cc * mu_2 * y[L::D2] - b.cc * Pa * Pb * br;
-  if (TAN) {
-    const double Pat = g.winther ? y[T] : y[T + L::A], Pbt = g.winther ? y[T] : y[T + L::B];
-    dy[T] = y[T + 1];
-    dy[T + 1] = -b.damp * y[T + 1] + b.cc * (mu_k * y[T] + mu_kt * y[0]);
-    dy[T + L::A] = y[T + L::A + 1];
-    dy[T + L::A + 1] = -b.damp * y[T + L::A + 1] + b.cc * (mu_a * y[T + L::A] + mu_at * y[L::A]);
-    if (GEO == 2) {
-      dy[T + L::B] = y[T + L::B + 1];
-      dy[T + L::B + 1] = -b.damp * y[T + L::B + 1] + b.cc * (mu_b * y[T + L::B] + mu_bt * y[L::B]);
+  const double w = h2 * b.cc;
+  o[CH_D1] = w * mu_k;
+  o[CH_DA] = w * mu_a;
+  o[CH_DB] = w * mu_b;
+  o[CH_D2] = g.gr2 ? w : w * mu_k;
+  o[CH_Z1] = w * mu_kt;
+  o[CH_ZA] = w * mu_at;
+  o[CH_ZB] = w * mu_bt;
+  o[CH_Z2] = g.gr2 ? 0.0 : w * mu_kt;
+  o[8] = w * br;
+  o[9] = w * brt;
+}
+
+// s = ln a at half step j of steps of size h from s0
+__device__ __forceinline__ double half_step_s(double s0, double h, int j) {
+  const int i = j >> 1;
+  return (j & 1) ? (s0 + i * h) + 0.5 * h : s0 + i * h;
+}
+
+// One RK4 step of (y, u = h y_s): coefficients C and damping D (scaled) at the step's ends and
+// middle, stage sources s0..s3; the stage values of y go to st.
+struct Rk4Stage { double y0, y1, y2, y3; };
+__device__ __forceinline__ Rk4Stage rk4_step(double& y, double& u, double D0, double Dm, double D1, double C0, double Cm,
+                                             double C1, double s0, double s1, double s2, double s3) {
+  Rk4Stage r;
+  r.y0 = y;
+  const double f0 = fma(D0, u, fma(C0, y, s0));
+  r.y1 = fma(0.5, u, y);
+  const double u1 = fma(0.5, f0, u);
+  const double f1 = fma(Dm, u1, fma(Cm, r.y1, s1));
+  r.y2 = fma(0.5, u1, y);
+  const double u2 = fma(0.5, f1, u);
+  const double f2 = fma(Dm, u2, fma(Cm, r.y2, s2));
+  r.y3 = y + u2;
+  const double u3 = u + f2;
+  const double f3 = fma(D1, u3, fma(C1, r.y3, s3));
+  const double f12 = f1 + f2, f012 = f0 + f12;
+  y = fma(1.0 / 6.0, f012, y + u);
+  u = fma(1.0 / 6.0, (f012 + f12) + f3, u);
+  return r;
+}
+
+// D1 of GR at a = 1 from the Einstein-de Sitter mode at a_init, by the whole block: the RK4
+// step is a 2x2 matrix on (y, u), each thread multiplies those of its share of the steps, and
+// the shares are multiplied in order.
+__device__ double gr_norm(const GrowthParams& p, double s0, GrowthSmem& sm) {
+  const double h = (0.0 - s0) / p.n_steps;
+  const int per = (p.n_steps + GR_THREADS - 1) / GR_THREADS;
+  const int i0 = threadIdx.x * per, i1 = min(p.n_steps, i0 + per);
+  double a0 = 1.0, a1 = 0.0, b0 = 0.0, b1 = 1.0;   // columns: (y, u) images of (1, 0) and (0, 1)
+  if (i0 < i1) {
+    Bg e = background(p, half_step_s(s0, h, 2 * i0), true);
+    for (int i = i0; i < i1; ++i) {
+      const Bg m = background(p, half_step_s(s0, h, 2 * i + 1), true), f = background(p, half_step_s(s0, h, 2 * i + 2), true);
+      const double D0 = -h * e.damp, Dm = -h * m.damp, D1 = -h * f.damp;
+      const double C0 = h * h * e.cc, Cm = h * h * m.cc, C1 = h * h * f.cc;
+      rk4_step(a0, a1, D0, Dm, D1, C0, Cm, C1, 0.0, 0.0, 0.0, 0.0);
+      rk4_step(b0, b1, D0, Dm, D1, C0, Cm, C1, 0.0, 0.0, 0.0, 0.0);
+      e = f;
     }
-    dy[T + L::D2] = y[T + L::D2 + 1];
-    dy[T + L::D2 + 1] = -b.damp * y[T + L::D2 + 1] + b.cc * (mu_2 * y[T + L::D2] + mu_2t * y[L::D2]) -
-                        b.cc * ((Pat * Pb + Pa * Pbt) * br + Pa * Pb * brt);
   }
+  // lane l holds the product of the shares l .. l + 2^k - 1 after k rounds
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const double c0 = __shfl_down_sync(0xffffffffu, a0, o), c1 = __shfl_down_sync(0xffffffffu, a1, o);
+    const double d0 = __shfl_down_sync(0xffffffffu, b0, o), d1 = __shfl_down_sync(0xffffffffu, b1, o);
+    const double n0 = fma(c0, a0, d0 * a1), n1 = fma(c1, a0, d1 * a1);
+    const double m0 = fma(c0, b0, d0 * b1), m1 = fma(c1, b0, d1 * b1);
+    a0 = n0; a1 = n1; b0 = m0; b1 = m1;
+  }
+  const int warp = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0) {
+    sm.red[warp][0] = a0;
+    sm.red[warp][1] = a1;
+    sm.red[warp][2] = b0;
+    sm.red[warp][3] = b1;
+  }
+  __syncthreads();
+  double y = p.a_init, u = h * p.a_init;   // EdS growing mode: D = a, dD/ds = a
+  for (int w = 0; w < GR_THREADS / 32; ++w) {
+    const double ny = fma(sm.red[w][0], y, sm.red[w][2] * u);
+    u = fma(sm.red[w][1], y, sm.red[w][3] * u);
+    y = ny;
+  }
+  return y;
 }
 
-template <int NY, bool TAN, int GEO>
-__device__ void rk4(const Bg* tab, int n_steps, double h, double k2, bool gr, const D2Geo& g, double* y) {
-  double k1[NY], k2v[NY], k3[NY], k4[NY], t[NY];
-  for (int i = 0; i < n_steps; ++i) {
-    const Bg& b0 = tab[2 * i];
-    const Bg& bm = tab[2 * i + 1];
-    const Bg& b1 = tab[2 * i + 2];
-    rhs<TAN, GEO>(b0, k2, gr, g, y, k1);
-#pragma unroll
-    for (int j = 0; j < NY; ++j) t[j] = y[j] + 0.5 * h * k1[j];
-    rhs<TAN, GEO>(bm, k2, gr, g, t, k2v);
-#pragma unroll
-    for (int j = 0; j < NY; ++j) t[j] = y[j] + 0.5 * h * k2v[j];
-    rhs<TAN, GEO>(bm, k2, gr, g, t, k3);
-#pragma unroll
-    for (int j = 0; j < NY; ++j) t[j] = y[j] + h * k3[j];
-    rhs<TAN, GEO>(b1, k2, gr, g, t, k4);
-#pragma unroll
-    for (int j = 0; j < NY; ++j) y[j] = y[j] + (h / 6.0) * (k1[j] + 2.0 * k2v[j] + 2.0 * k3[j] + k4[j]);
-  }
-}
-
-__device__ void fill_bg(Bg* tab, const GrowthParams& p, double s0, double h, int n_steps, bool gr) {
-  for (int j = threadIdx.x; j <= 2 * n_steps; j += blockDim.x) {
-    const int i = j >> 1;
-    const double s = (j & 1) ? (s0 + i * h) + 0.5 * h : s0 + i * h;
-    tab[j] = background(p, s, gr);
-  }
-}
-
-template <bool TAN, int GEO>
-__global__ void k_growth(GrowthParams p, double* tab, float* tabf) {
-  using L = Layout<GEO>;
-  extern __shared__ Bg s_bg[];
+template <int GEO>
+__global__ void __launch_bounds__(GR_THREADS) k_growth(GrowthParams p, double* tab, float* tabf) {
+  extern __shared__ __align__(16) unsigned char s_raw[];
+  GrowthSmem& sm = *reinterpret_cast<GrowthSmem*>(s_raw);
   if (p.fr0s) p.fr0_abs = p.fr0s[blockIdx.y];     // instance blockIdx.y
   tab += (size_t)blockIdx.y * 4 * p.nk;
   tabf += (size_t)blockIdx.y * 4 * p.nk;
   const bool gr = (p.fr0_abs == 0.0);
   const D2Geo geo = d2_geo(p.d2_variant);
   const double s0 = log(p.a_init);
-  // GR normalisation D1_GR(a = 1)
-  const double hg = (0.0 - s0) / p.n_steps;
-  fill_bg(s_bg, p, s0, hg, p.n_steps, true);
+  const double norm = gr_norm(p, s0, sm);
+  const double h = (log(p.a_out) - s0) / p.n_steps, h2 = h * h;
+  const int k0 = blockIdx.x * GR_KPB;
+  const int n_half = 2 * p.n_steps;
+  const int nch = (p.n_steps + GR_CH - 1) / GR_CH;
+  // coefficients of chunk c: threads t, t + stride, ... of a group of `stride` threads, t and
+  // stride congruent to threadIdx.x and 0 mod GR_KPB, so a thread keeps to one k
+  const int kf = threadIdx.x % GR_KPB;
+  const double k = p.k_min * pow(p.k_max / p.k_min, (double)min(k0 + kf, p.nk - 1) / (double)(p.nk - 1));
+  auto fill_coef = [&](int c, int t, int stride) {
+    for (; t < GR_HS * GR_KPB; t += stride) {
+      const int j = t / GR_KPB;
+      const Bg b = background(p, half_step_s(s0, h, min(c * 2 * GR_CH + j, n_half)), gr);
+      growth_coef<GEO>(b, k * k, gr, geo, h2, sm.coef[c % GR_CRING][j][kf]);
+      if (kf == 0) sm.damp[c % GR_CRING][j] = -h * b.damp;
+    }
+  };
+  fill_coef(0, threadIdx.x, GR_THREADS);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // chain lane: k = lane / 8, chain = lane % 8
+  const int chain = lane & 7, kk = lane >> 3;
+  const int level = chain < CH_D2 ? 0 : (chain == CH_Z2 ? 2 : 1);
+  double y = chain < CH_D2 ? p.a_init : (chain == CH_D2 ? -3.0 / 7.0 * p.a_init * p.a_init : 0.0);
+  double u = h * (chain < CH_D2 ? p.a_init : (chain == CH_D2 ? -6.0 / 7.0 * p.a_init * p.a_init : 0.0));
   __syncthreads();
-  double g[6] = {p.a_init, p.a_init, p.a_init, p.a_init, 0.0, 0.0};
-  rk4<6, false, 0>(s_bg, p.n_steps, hg, 1.0, true, d2_geo(0), g);
-  const double norm = g[0];
-  __syncthreads();
-  const double h = (log(p.a_out) - s0) / p.n_steps;
-  fill_bg(s_bg, p, s0, h, p.n_steps, gr);
-  __syncthreads();
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= p.nk) return;
-  const double k = p.k_min * pow(p.k_max / p.k_min, (double)t / (double)(p.nk - 1));
-  constexpr int NY = TAN ? 2 * L::NB : L::NB;
-  double y[NY];
+  for (int it = 0; it < nch + 4; ++it) {
+    if (warp == 0) {
+      const int c = it - 2 * level;
+      if (c >= 0 && c < nch) {
+        const double* cf = &sm.coef[c % GR_CRING][0][kk][chain & 3];
+        const double* dm = sm.damp[c % GR_CRING];
+        double* va = &sm.val[c % GR_VRING][0][0][lane];
+        const double* sr = &sm.src[c % GR_SRING][0][0][lane];
+        double D0 = dm[0], C0 = cf[0];
+#pragma unroll 2
+        for (int i = 0; i < GR_CH; ++i) {
+          const double Dm = dm[2 * i + 1], D1 = dm[2 * i + 2];
+          const double Cm = cf[(2 * i + 1) * GR_KPB * GR_NC], C1 = cf[(2 * i + 2) * GR_KPB * GR_NC];
+          double s[4] = {0.0, 0.0, 0.0, 0.0};
+          if (level > 0) {
 #pragma unroll
-  for (int j = 0; j < NY; ++j) y[j] = 0.0;
-#pragma unroll
-  for (int j = 0; j < L::D2; ++j) y[j] = p.a_init;
-  y[L::D2] = -3.0 / 7.0 * p.a_init * p.a_init;
-  y[L::D2 + 1] = -6.0 / 7.0 * p.a_init * p.a_init;
-  rk4<NY, TAN, GEO>(s_bg, p.n_steps, h, k * k, gr, geo, y);
+            for (int q = 0; q < 4; ++q) s[q] = sr[(i * 4 + q) * 32];
+          }
+          double ny = y, nu = u;
+          const Rk4Stage r = rk4_step(ny, nu, D0, Dm, D1, C0, Cm, C1, s[0], s[1], s[2], s[3]);
+          va[(i * 4 + 0) * 32] = r.y0;
+          va[(i * 4 + 1) * 32] = r.y1;
+          va[(i * 4 + 2) * 32] = r.y2;
+          va[(i * 4 + 3) * 32] = r.y3;
+          if (c * GR_CH + i < p.n_steps) {   // the last chunk may be partial
+            y = ny;
+            u = nu;
+          }
+          D0 = D1;
+          C0 = C1;
+        }
+      }
+    } else {
+      const int t0 = threadIdx.x - 32, stride = GR_THREADS - 32;
+      if (it + 1 < nch) fill_coef(it + 1, t0, stride);
+      // sources: task (step, stage, k); the half step of stages 0, 1, 2, 3 is 2 i + {0, 1, 1, 2}
+      for (int lev = 1; lev <= 2; ++lev) {
+        const int c = it + 1 - 2 * lev;
+        if (c < 0 || c >= nch) continue;
+        for (int t = t0; t < GR_CH * 4 * GR_KPB; t += stride) {
+          const int kt = t % GR_KPB, q = (t / GR_KPB) & 3, i = t / (4 * GR_KPB);
+          const int j = 2 * i + ((q + 1) >> 1);
+          const double* cf = sm.coef[c % GR_CRING][j][kt];
+          const double* v = &sm.val[c % GR_VRING][i][q][kt * 8];
+          double* o = &sm.src[c % GR_SRING][i][q][kt * 8];
+          const double Pa = v[geo.winther ? CH_D1 : CH_DA], Pb = v[geo.winther ? CH_D1 : CH_DB];
+          if (lev == 1) {
+            o[CH_D2] = -cf[8] * (Pa * Pb);
+            o[CH_Z1] = cf[4] * v[CH_D1];
+            o[CH_ZA] = cf[5] * v[CH_DA];
+            o[CH_ZB] = cf[6] * v[CH_DB];
+          } else {
+            const double Pat = v[geo.winther ? CH_Z1 : CH_ZA], Pbt = v[geo.winther ? CH_Z1 : CH_ZB];
+            o[CH_Z2] = fma(cf[7], v[CH_D2], -fma(cf[8], fma(Pat, Pb, Pa * Pbt), cf[9] * (Pa * Pb)));
+          }
+        }
+      }
+    }
+    __syncthreads();
+  }
+  if (warp == 0) sm.out[lane] = y;
+  __syncthreads();
+  const int t = k0 + threadIdx.x;
+  if (threadIdx.x >= GR_KPB || t >= p.nk) return;
+  const double* o = sm.out + threadIdx.x * 8;
   const int nk = p.nk;
-  const int T = L::NB;
-  tab[t] = y[0] / norm;
-  tab[nk + t] = y[L::D2] / (norm * norm);
-  tab[2 * nk + t] = TAN ? y[T] / norm : 0.0;
-  tab[3 * nk + t] = TAN ? y[T + L::D2] / (norm * norm) : 0.0;
+  tab[t] = o[CH_D1] / norm;
+  tab[nk + t] = o[CH_D2] / (norm * norm);
+  tab[2 * nk + t] = o[CH_Z1] / norm;
+  tab[3 * nk + t] = o[CH_Z2] / (norm * norm);
   if (geo.fit) {   // D2 = -(3/7) D1^2 Omega_m(a)^(-1/143), tangent -(6/7) D1 dD1 Omega_m(a)^(-1/143)
     const double a3 = 1.0 / (p.a_out * p.a_out * p.a_out);
     const double f = pow(p.omega_m * a3 / (p.omega_m * a3 + p.omega_l), -1.0 / 143.0);
     tab[nk + t] = -3.0 / 7.0 * tab[t] * tab[t] * f;
     tab[3 * nk + t] = -6.0 / 7.0 * tab[t] * tab[2 * nk + t] * f;
   }
-  tabf[t] = (float)(y[0] / norm);
-  tabf[nk + t] = (float)tab[nk + t];
-  tabf[2 * nk + t] = (float)tab[2 * nk + t];
-  tabf[3 * nk + t] = (float)tab[3 * nk + t];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) tabf[i * nk + t] = (float)tab[i * nk + t];
 }
 
-#ifndef LPT2_GROWTH_THREADS
-#define LPT2_GROWTH_THREADS 32   // k nodes per block (measured best: the RK4 chains are FP64-latency bound)
-#endif
 template <int GEO>
 static cudaError_t launch_growth_geo(const GrowthParams& p, double* tab, float* tabf, cudaStream_t s) {
-  const int threads = LPT2_GROWTH_THREADS;
-  const int blocks = (p.nk + threads - 1) / threads;
-  const size_t smem = (size_t)(2 * p.n_steps + 1) * sizeof(Bg);
-  cudaFuncSetAttribute(k_growth<true, GEO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_growth<true, GEO><<<dim3(blocks, p.n_inst > 0 ? p.n_inst : 1), threads, smem, s>>>(p, tab, tabf);
+  const int blocks = (p.nk + GR_KPB - 1) / GR_KPB;
+  cudaFuncSetAttribute(k_growth<GEO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GrowthSmem));
+  k_growth<GEO><<<dim3(blocks, p.n_inst > 0 ? p.n_inst : 1), GR_THREADS, sizeof(GrowthSmem), s>>>(p, tab, tabf);
   return cudaGetLastError();
 }
 
