@@ -77,7 +77,7 @@ struct Group {
   double box;
   int count;
   int inst0;       // index of the group's first instance in the plan
-  float2* tw;      // twiddles exp(-2 pi i m / n)
+  float2* tw;      // twiddles, in the stages' order (twiddle_exponent)
   size_t off;      // floats before the group's first instance in per-instance real fields
   float4* mt0;     // per-|n|^2 multiplier tables [count][mode_table_len(n)]
   float2* mt1;
@@ -218,6 +218,20 @@ int x_blocks(int n) {
     case 256: return x_blocks_256();
     case 512: return x_blocks_512();
     default: return x_blocks_1024();
+  }
+}
+
+int twiddle_exponent(int n, int i) {
+  switch (n) {
+    case 16: return twiddle_exponent_16(i);
+    case 32: return twiddle_exponent_32(i);
+    case 64: return twiddle_exponent_64(i);
+    case 96: return twiddle_exponent_96(i);
+    case 128: return twiddle_exponent_128(i);
+    case 192: return twiddle_exponent_192(i);
+    case 256: return twiddle_exponent_256(i);
+    case 512: return twiddle_exponent_512(i);
+    default: return twiddle_exponent_1024(i);
   }
 }
 
@@ -788,11 +802,11 @@ int lpt2_plan(lpt2_plan_t* out, const lpt2_instance* inst, int n_inst, int n_k, 
     return fail(e == cudaErrorMemoryAllocation ? LPT2_ENOMEM : LPT2_ECUDA, "plan allocation failed: %s",
                 cudaGetErrorString(e));
   }
-  // twiddles exp(-2 pi i m / N), FP64 then rounded once
+  // twiddles exp(-2 pi i m / N) in the stages' order, FP64 then rounded once
   for (Group& g : p->groups) {
     std::vector<float2> tw(g.n);
     for (int m = 0; m < g.n; ++m) {
-      const double ang = 2.0 * M_PI * (double)m / (double)g.n;
+      const double ang = 2.0 * M_PI * (double)twiddle_exponent(g.n, m) / (double)g.n;
       tw[m] = make_float2((float)cos(ang), (float)(-sin(ang)));
     }
     e = cudaMemcpy(g.tw, tw.data(), g.n * sizeof(float2), cudaMemcpyHostToDevice);

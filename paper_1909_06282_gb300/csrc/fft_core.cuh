@@ -9,7 +9,8 @@
 // butterflies on inputs b + r N/R, twiddle W_{Ns R}^{r (b mod Ns)}, outputs at
 // (b / Ns) Ns R + b mod Ns + r Ns) with one shared-memory exchange between
 // consecutive stages.  Twiddles come from a table exp(-2 pi i m / N) computed in
-// FP64 on the host and rounded once to FP32.
+// FP64 on the host and rounded once to FP32, stored per stage in the order the lanes of a
+// pencil read them (twiddle_exponent).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -21,6 +22,31 @@ __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
+}
+// cadd and csub as one packed instruction (add / sub.rn.f32x2: the same roundings).  The packed
+// form has the arithmetic rate of two scalar adds but takes one issue slot instead of two
+// (measured: 0.53 against 1.04 instructions per cycle and scheduler), and the passes with
+// several transforms per field are bound by issue and shared-memory slots: z_source at 512^3
+// 1141 -> 1071 us, z_final 636 -> 617 us, x_pkadj 367 -> 341 us.  Products stay scalar: a packed
+// complex product needs swapped or doubled operands, whose moves cost what it saves.
+__device__ __forceinline__ float2 padd(float2 a, float2 b) {
+#ifdef __CUDA_ARCH__
+  return __fadd2_rn(a, b);
+#else
+  return cadd(a, b);
+#endif
+}
+__device__ __forceinline__ float2 psub(float2 a, float2 b) {
+#ifdef __CUDA_ARCH__
+  float2 o;
+  asm("{\n\t.reg .b64 p, q, r;\n\tmov.b64 p, {%2, %3};\n\tmov.b64 q, {%4, %5};\n\tsub.rn.f32x2 r, p, q;\n\t"
+      "mov.b64 {%0, %1}, r;\n\t}"
+      : "=f"(o.x), "=f"(o.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return o;
+#else
+  return csub(a, b);
+#endif
 }
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
 __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
@@ -60,6 +86,20 @@ template <int N> __host__ __device__ constexpr int ns_before(int s) {
   int p = 1;
   for (int i = 0; i < s; ++i) p *= Cfg<N>::rad(i);
   return p;
+}
+
+// Twiddle table: entry i, NS <= i < NS R of a stage with radix R after NS = ns_before points,
+// is exp(-2 pi i r j / (NS R)) for r = i / NS, j = i mod NS (a thread's butterfly b reads j = b
+// mod NS): the lanes of a pencil, whose b are consecutive, read consecutive entries.  The
+// stages' ranges tile [ns_before(1), N).  A table in the order of the exponent puts the lanes
+// r entries apart, up to 16 to a bank (512^3: z_source 1257 -> 1141 us, z_adj_source 2223 ->
+// 1907 us, x_pkadj 438 -> 367 us by this order).  Returns the exponent m of exp(-2 pi i m / N).
+template <int N> __host__ __device__ constexpr int twiddle_exponent(int i) {
+  for (int s = 1; s < Cfg<N>::NS; ++s) {
+    const int ns = ns_before<N>(s), R = Cfg<N>::rad(s);
+    if (i >= ns && i < ns * R) return (i / ns) * (i % ns) * (N / (ns * R));
+  }
+  return 0;
 }
 
 // ------------------------------------------------------- in-register DFTs
@@ -103,8 +143,9 @@ template <bool INV> struct Dft<3, INV> {
 template <bool INV> struct Dft<2, INV> {
   static __device__ __forceinline__ void run(float2* v) {
     const float2 a = v[0];
-    v[0] = cadd(a, v[1]);
-    v[1] = csub(a, v[1]);
+    const float2 b = v[1];
+    v[0] = padd(a, b);
+    v[1] = psub(a, b);
   }
 };
 
@@ -123,8 +164,13 @@ template <int R, bool INV> struct Dft {   // even R: split into even and odd hal
       if (j == 0) t = o[k];
       else if (j == 12) t = INV ? mul_i(o[k]) : mul_mi(o[k]);
       else t = cmul(o[k], root48(j, INV));
-      v[k] = cadd(e[k], t);
-      v[k + R / 2] = csub(e[k], t);
+      if (j == 12) {   // t is o with its parts swapped: scalar adds read the swap in place
+        v[k] = cadd(e[k], t);
+        v[k + R / 2] = csub(e[k], t);
+      } else {
+        v[k] = padd(e[k], t);
+        v[k + R / 2] = psub(e[k], t);
+      }
     }
   }
 };
@@ -173,7 +219,7 @@ __device__ __forceinline__ void fft_stages(float2 (&v)[Cfg<N>::RMAX], int t, con
       const int j = b % NS;
 #pragma unroll
       for (int r = 1; r < R; ++r) {
-        float2 w = tw[(r * j) * (N / (NS * R))];
+        float2 w = tw[r * NS + j];
         if (INV) w.y = -w.y;
         v[q * R + r] = cmul(v[q * R + r], w);
       }

@@ -83,12 +83,21 @@ int fail(int code, const std::string& msg) {
   return code;
 }
 
-// Twiddles exp(-2 pi i m / n) in FP64, rounded once to FP32.
-__global__ void k_noalloc_twiddles(float2* tw, int n) {
-  for (int m = threadIdx.x; m < n; m += blockDim.x) {
+// Twiddles exp(-2 pi i m / N) in FP64, rounded once to FP32, in the order of the pass kernels'
+// table (twiddle_exponent).
+template <int N> __global__ void k_noalloc_twiddles(float2* tw) {
+  for (int i = threadIdx.x; i < N; i += blockDim.x) {
     double s, c;
-    sincospi(2.0 * (double)m / (double)n, &s, &c);
-    tw[m] = make_float2((float)c, (float)(-s));
+    sincospi(2.0 * (double)twiddle_exponent<N>(i) / (double)N, &s, &c);
+    tw[i] = make_float2((float)c, (float)(-s));
+  }
+}
+void noalloc_twiddles(int n, float2* tw, cudaStream_t s) {
+  switch (n) {
+    case 16: k_noalloc_twiddles<16><<<1, 128, 0, s>>>(tw); break;
+    case 32: k_noalloc_twiddles<32><<<1, 128, 0, s>>>(tw); break;
+    case 64: k_noalloc_twiddles<64><<<1, 128, 0, s>>>(tw); break;
+    default: k_noalloc_twiddles<128><<<1, 128, 0, s>>>(tw); break;
   }
 }
 
@@ -194,7 +203,7 @@ extern "C" int lpt2_cic_pk_noalloc(int n, double box, const float* pos, float* d
     if (e_ != cudaSuccess) return fail(LPT2_ECUDA, std::string(#expr ": ") + cudaGetErrorString(e_)); \
   } while (0)
 
-  k_noalloc_twiddles<<<1, 128, 0, s>>>(tw, n);
+  noalloc_twiddles(n, tw, s);
   NA_CHECK(cudaGetLastError());
   NA_CHECK(launch_fill0(rho, n3, s));               // the deposit accumulates: start from zero
   CicArgs c{g, pos, rho};

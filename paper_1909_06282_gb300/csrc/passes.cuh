@@ -1662,4 +1662,5 @@ template <int N> int x_blocks_t() { return (PassCfg<N>::H / PassCfg<N>::W) * N; 
   }                                                                                                  \
   cudaError_t launch_x_##N(const XArgs& a, cudaStream_t s) { return launch_x_t<N>(a, s); }           \
   int x_blocks_##N() { return x_blocks_t<N>(); }                                                     \
+  int twiddle_exponent_##N(int i) { return twiddle_exponent<N>(i); }                                 \
   }

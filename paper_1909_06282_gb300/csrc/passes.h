@@ -221,7 +221,8 @@ struct CicArgs {
   cudaError_t launch_y_##N(const YArgs&, cudaStream_t);                          \
   cudaError_t launch_z_adj_source_##N(const ZAdjSourceArgs&, cudaStream_t);      \
   cudaError_t launch_x_##N(const XArgs&, cudaStream_t);                          \
-  int x_blocks_##N();
+  int x_blocks_##N();                                                            \
+  int twiddle_exponent_##N(int i); /* order of the twiddle table (fft_core.cuh) */
 
 LPT2_DECLARE_LAUNCHERS(16)
 LPT2_DECLARE_LAUNCHERS(32)
