@@ -917,7 +917,7 @@ struct XSmemIn {
 // s_acc the per-warp accumulators (zeroed by the caller), blk the tile's linear index,
 // s_sc the tile of the scf field staged in shared memory (element (kx, w) at kx W + w), or
 // null to read a.scf from global memory.
-template <int N, int MODE>
+template <int N, int MODE, bool SPLIT>
 __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[PassCfg<N>::RMAX], int kzb, int ky, int inst,
                                        size_t blk, const SmemCol<PassCfg<N>::W>& sm, const float2* s_tw,
                                        double* s_acc, const float* s_sc = nullptr, XSmemIn si = {}) {
@@ -1145,8 +1145,8 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[PassCfg<N>::R
   // sqrt(P N^3/V) and 1/(k^2 N^3) only, the first comes from the scf field (coalesced, or
   // staged with the tile) and the second is computed.
   const size_t toff = (size_t)inst * mode_table_len(N);
-  const bool field = (MODE == X_DELTA && !a.split && (s_sc || a.scf)) || (MODE == X_ADJ_DELTA && a.scf);
-  float2 g[C::RMAX], hpot[C::RMAX];
+  constexpr bool field = (MODE == X_DELTA && !SPLIT) || MODE == X_ADJ_DELTA;
+  float2 g[C::RMAX], hpot[SPLIT && MODE == X_DELTA ? C::RMAX : 1];
   float theta = 0.f;
 #pragma unroll
   for (int r = 0; r < C::RMAX; ++r) {
@@ -1169,10 +1169,10 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[PassCfg<N>::R
       const float2 d = cscale(v[r], sc);
       if (a.delta_out) a.delta_out[e] = d;
       g[r] = cscale(d, inv);                                // phi1 = delta / k^2 (1/N^3 folded)
-      if (a.split) hpot[r] = cscale(g[r], d1);
+      if constexpr (SPLIT) hpot[r] = cscale(g[r], d1);
     } else if (MODE == X_SOURCE) {                        // v = S(k)
       float2 u = cscale(v[r], -d2 * inv);                   // phi2 = -S D2 / k^2
-      if (!a.split) {
+      if constexpr (!SPLIT) {
         const float2 dl = a.delta_in[e];
         u = cadd(u, cscale(dl, d1 * inv));                  // + phi1 D1 (total potential)
       }
@@ -1203,18 +1203,18 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[PassCfg<N>::R
   // x-inverse transforms with x-derivative orders (the exchange buffer may hold the
   // shared-memory inputs read above: every thread has read its own first)
   if (si.summed) __syncthreads();
-  int nout;
-  if (MODE == X_DELTA) nout = a.split ? 5 : 3;
-  else if (MODE == X_SOURCE) nout = 2;
-  else nout = 1;
+  constexpr int nout = MODE == X_DELTA ? (SPLIT ? 5 : 3) : (MODE == X_SOURCE ? 2 : 1);
+#pragma unroll 1
   for (int o = 0; o < nout; ++o) {
-    const bool fromh = (MODE == X_DELTA) && o >= 3;
+    const bool fromh = SPLIT && MODE == X_DELTA && o >= 3;
     const int m = MODE == X_DELTA ? (o < 3 ? o : o - 3) : (MODE == X_SOURCE ? o : 0);
     float2 u[C::RMAX];
 #pragma unroll
     for (int r = 0; r < C::RMAX; ++r) {
       const int kx = elem<N>(t, r);
-      u[r] = deriv(fromh ? hpot[r] : g[r], kf * (float)mode_of(kx, N), m);
+      float2 src = g[r];
+      if constexpr (SPLIT && MODE == X_DELTA) src = fromh ? hpot[r] : src;
+      u[r] = deriv(src, kf * (float)mode_of(kx, N), m);
     }
     fft<N, true>(u, t, sm, s_tw);
 #pragma unroll
@@ -1229,7 +1229,10 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[PassCfg<N>::R
 
 // Tile loads from global memory (one CTA per tile): the adjoint modes, whose tiles are sums
 // over several inputs, and any mode when the bulk-tensor path is off.
-template <int N, int MODE>
+// SPLIT (X_DELTA, X_SOURCE): separate Psi1 and Psi2 potentials.  A template parameter: as a run-time
+// flag the second potential array held its registers in the total form too (x_delta at 512^3 850 ->
+// 740 us, its split form at 256^3 124 -> 113 us).
+template <int N, int MODE, bool SPLIT>
 __global__ void __launch_bounds__(PassCfg<N>::XT, x_minb<N>(MODE)) k_x(XArgs a) {
   using C = PassCfg<N>;
   extern __shared__ float2 smem[];
@@ -1253,7 +1256,7 @@ __global__ void __launch_bounds__(PassCfg<N>::XT, x_minb<N>(MODE)) k_x(XArgs a) 
     for (int r = 0; r < C::RMAX; ++r) v[r] = a.in[base + (size_t)(elem<N>(t, r)) * ((size_t)N * C::H)];
   }
   const size_t blk = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-  x_tile<N, MODE>(a, v, blockIdx.x, blockIdx.y, blockIdx.z, blk, sm, s_tw, s_acc);
+  x_tile<N, MODE, SPLIT>(a, v, blockIdx.x, blockIdx.y, blockIdx.z, blk, sm, s_tw, s_acc);
 }
 
 // Tile loads by the tensor-memory accelerator: a persistent CTA walks the tiles
@@ -1266,8 +1269,8 @@ __global__ void __launch_bounds__(PassCfg<N>::XT, x_minb<N>(MODE)) k_x(XArgs a) 
 #ifndef LPT2_X_TMA
 #define LPT2_X_TMA 1
 #endif
-// SC: each ring stage also holds the tile of the scf field (TILE floats after the TILE
-// float2 of the input).
+// SC (the total-potential form): each ring stage also holds the tile of the scf field (TILE
+// floats after the TILE float2 of the input); without it the pass is the split form.
 template <int N, bool SC = false> struct XTmaCfg {
   using C = PassCfg<N>;
   static constexpr int TILE = N * C::W;                 // float2 per tile
@@ -1343,7 +1346,7 @@ __global__ void __launch_bounds__(PassCfg<N>::XT, x_minb<N>(MODE)) k_x_tma(const
     const int kzb = tile % Q::KZB, ky = (tile / Q::KZB) % N, inst = tile / (Q::KZB * N);
     const SmemCol<C::W> sm{ring + st * Q::STAGE + w};
     const float* s_sc = SC ? reinterpret_cast<const float*>(ring + st * Q::STAGE + Q::TILE) : nullptr;
-    x_tile<N, MODE>(a, v, kzb, ky, inst, (size_t)tile, sm, s_tw, s_acc, s_sc);
+    x_tile<N, MODE, !SC>(a, v, kzb, ky, inst, (size_t)tile, sm, s_tw, s_acc, s_sc);
     __syncthreads();   // ring stage and accumulators free
     if (threadIdx.x == 0 && tile + 2 * gridDim.x < ntiles) {
       fence_proxy_async_smem();
@@ -1460,7 +1463,7 @@ __global__ void __launch_bounds__(PassCfg<N>::XT, x_minb<N>(MODE)) k_x_tma_adj(c
       si.s = ring + s1 * Q::TILE;
       ex = ring + s1 * Q::TILE;
     }
-    x_tile<N, MODE>(a, v, kzb, ky, inst, (size_t)tile, SmemCol<C::W>{ex + w}, s_tw, s_acc, nullptr, si);
+    x_tile<N, MODE, false>(a, v, kzb, ky, inst, (size_t)tile, SmemCol<C::W>{ex + w}, s_tw, s_acc, nullptr, si);
     __syncthreads();   // stages and accumulators free
     if (threadIdx.x == 0) {
       fence_proxy_async_smem();
@@ -1610,20 +1613,20 @@ template <int N, int MODE> cudaError_t launch_x_m(const XArgs& a, cudaStream_t s
   // the CTAs per SM, and the source multiplier, which also reads delta(k) per mode, measured
   // 0.73 -> 0.76 ms with bulk-tensor tiles.
   if (a.g.xtile < 0 || a.g.xtile > 2) return cudaErrorInvalidValue;
+  if (((MODE == X_DELTA && !a.split) || MODE == X_ADJ_DELTA) && !a.scf) return cudaErrorInvalidValue;
   if constexpr (MODE == X_ADJ_DELTA || MODE == X_ADJ_SOURCE) {
     if (a.g.xtile == 0 ? LPT2_X_TMA_ADJ != 0 : a.g.xtile == 1) return launch_x_tma_adj<N, MODE>(a, acc, s);
   }
   if constexpr (MODE == X_DELTA) {
     if (a.g.xtile == 0 ? LPT2_X_TMA != 0 : a.g.xtile == 1) {
-      if constexpr (MODE == X_DELTA) {
-        if (a.scf && !a.split) return launch_x_tma<N, MODE, true>(a, acc, s);
-      }
-      return launch_x_tma<N, MODE, false>(a, acc, s);
+      return a.split ? launch_x_tma<N, MODE, false>(a, acc, s) : launch_x_tma<N, MODE, true>(a, acc, s);
     }
   }
   const int smem = C::XSMEM + acc;
-  cudaFuncSetAttribute(k_x<N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  k_x<N, MODE><<<dim3(C::H / C::W, N, a.g.batch), C::XT, smem, s>>>(a);
+  constexpr bool has_split = MODE == X_DELTA || MODE == X_SOURCE;
+  auto k = has_split && a.split ? k_x<N, MODE, has_split> : k_x<N, MODE, false>;
+  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  k<<<dim3(C::H / C::W, N, a.g.batch), C::XT, smem, s>>>(a);
   return cudaGetLastError();
 }
 template <int N> cudaError_t launch_x_t(const XArgs& a, cudaStream_t s) {
