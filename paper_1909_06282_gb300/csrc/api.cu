@@ -406,7 +406,8 @@ int check_plan_ws(lpt2_plan_t p) {
 }
 
 // forward r2c of a real field (or the Philox noise) into `out`, z -> y -> x (plain)
-int forward_zy(lpt2_plan_t p, int src, const float* in, float2* out) {
+// (Z_DENSITY: in - 1, which also goes to `contrast` when that is not null)
+int forward_zy(lpt2_plan_t p, int src, const float* in, float2* out, float* contrast = nullptr) {
   ZR2CArgs z{};
   z.g = make_geo(p);
   z.tw = p->tw;
@@ -417,8 +418,9 @@ int forward_zy(lpt2_plan_t p, int src, const float* in, float2* out) {
   z.seeds = p->seeds_dev;
   z.bm = p->bm_tab;
   z.out = out;
+  z.contrast = contrast;
   LAUNCH(p, src == Z_NOISE ? "z_r2c_noise" : (src == Z_DENSITY ? "z_r2c_density" : "z_r2c"),
-         (src == Z_NOISE ? 4.0 : 8.0) * V3(p), z_r2c(p->n, z, p->stream));
+         ((src == Z_NOISE ? 4.0 : 8.0) + (contrast ? 4.0 : 0.0)) * V3(p), z_r2c(p->n, z, p->stream));
   YArgs y{};
   y.g = z.g;
   y.tw = p->tw;
@@ -518,9 +520,8 @@ int cic_pk_group(lpt2_plan_t p, int gi, const float* pos, float* density, double
     CicArgs c{g, pos, rho};
     LAUNCH(p, "cic", 20.0 * V3(p), launch_cic(c, p->stream));
   }
-  int rc = forward_zy(p, Z_DENSITY, rho, A);   // rho - 1 is formed in the z pass; rho is kept
+  int rc = forward_zy(p, Z_DENSITY, rho, A, density);   // rho - 1 is formed in the z pass; rho is kept
   if (rc) return rc;
-  if (density) LAUNCH(p, "contrast", 8.0 * V3(p), launch_contrast(rho, density, cells, p->stream));
   XArgs x{};
   x.g = g;
   x.tw = p->tw;
@@ -1086,7 +1087,6 @@ int displace_suffix(lpt2_plan_t p, const FwdSlots& f, bool split, float* psi1, f
   const int n = p->n;
   const Geo g = make_geo(p);
   float* rho = rho_group(p);
-  const size_t cells = (size_t)n * n * n * p->cur_batch;   // real elements of the group
 
   // 4. x pass: S(k) -> phi2 = -S D2/k^2 (+ D1 delta/k^2 when not split), x inverse
   XArgs xs{};
@@ -1096,6 +1096,7 @@ int displace_suffix(lpt2_plan_t p, const FwdSlots& f, bool split, float* psi1, f
   xs.split = split;
   xs.in = f.A;
   xs.s_out = s_keep;
+  xs.zero = rho;   // cleared for the deposit below
   xs.delta_out = nullptr;
   xs.delta_in = f.D;
   xs.out[0] = f.X[0];
@@ -1107,7 +1108,7 @@ int displace_suffix(lpt2_plan_t p, const FwdSlots& f, bool split, float* psi1, f
   xs.d2f = tabf + p->nk;
   xs.t1f = tabf + 2 * p->nk;
   xs.t2f = tabf + 3 * p->nk;
-  LAUNCH(p, "x_source", (split ? 12.0 : 16.0) * V3(p), x_pass(n, xs, p->stream));
+  LAUNCH(p, "x_source", (split ? 16.0 : 20.0) * V3(p), x_pass(n, xs, p->stream));   // + the cleared density
 
   // 5. y inverse: (x0 y0), (x0 y1), (x1 y0)
   YArgs y2{};
@@ -1126,8 +1127,7 @@ int displace_suffix(lpt2_plan_t p, const FwdSlots& f, bool split, float* psi1, f
   }
   LAUNCH(p, "y_psi", 20.0 * V3(p), y_pass(n, y2, p->stream));
 
-  // 6. z inverse, positions, CIC
-  LAUNCH(p, "fill0", 4.0 * V3(p), launch_fill0(rho, cells, p->stream));
+  // 6. z inverse, positions, CIC (the density was cleared by the x pass)
   ZFinalArgs zf{};
   zf.g = g;
   zf.tw = p->tw;
@@ -1526,9 +1526,7 @@ int lpt2_cic_pk_est(lpt2_plan_t p, const float* pos, float* density, double* pk,
       CicArgs c{g, gpos, rho, 0.f};
       LAUNCH(p, "cic", 20.0 * V3(p), launch_cic(c, p->stream));
     }
-    if ((rc = forward_zy(p, Z_DENSITY, rho, A))) return rc;
-    if (density)
-      LAUNCH(p, "contrast", 8.0 * V3(p), launch_contrast(rho, density + gr.off, cells, p->stream));
+    if ((rc = forward_zy(p, Z_DENSITY, rho, A, density ? density + gr.off : nullptr))) return rc;
     float2* B = slot(p, S_Y0);
     if (inter) {   // second grid: the particles shifted by +h/2 along every axis
       float* rho2 = reinterpret_cast<float*>(slot(p, S_X0));

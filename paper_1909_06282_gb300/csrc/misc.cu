@@ -277,17 +277,6 @@ cudaError_t launch_fill0(float* p, size_t n, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// density contrast delta = rho N^3 / N_p - 1 with one particle per cell
-__global__ void k_contrast(const float* __restrict__ rho, float* __restrict__ out, size_t n) {
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    out[i] = rho[i] - 1.0f;
-}
-
-cudaError_t launch_contrast(const float* rho, float* out, size_t n, cudaStream_t s) {
-  k_contrast<<<152 * 8, 256, 0, s>>>(rho, out, n);
-  return cudaGetLastError();
-}
-
 // One block per shell: fixed-order strided sums then a tree (deterministic).
 __global__ void k_pk_finalize(const double* part, int n_blocks, int ns, double* pk, double* kmean,
                               int64_t* nmodes) {

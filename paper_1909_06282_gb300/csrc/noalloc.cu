@@ -214,6 +214,7 @@ extern "C" int lpt2_cic_pk_noalloc(int n, double box, const float* pos, float* d
   z.src = Z_DENSITY;
   z.in = rho;
   z.out = spec;
+  z.contrast = density;
   NA_CHECK(z_r2c_n(n, z, s));
   YArgs y{};
   y.g = g;
@@ -234,7 +235,6 @@ extern "C" int lpt2_cic_pk_noalloc(int n, double box, const float* pos, float* d
   x.n_shells = n_shells;
   NA_CHECK(x_n(n, x, s));
   NA_CHECK(launch_pk_finalize(part, xblocks_n(n), n_shells, pk, k_mean, n_modes, s));
-  if (density) NA_CHECK(launch_contrast(rho, density, n3, s));
 #undef NA_CHECK
   return LPT2_OK;
 }

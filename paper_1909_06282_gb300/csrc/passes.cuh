@@ -179,6 +179,7 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, SRC == Z_NOISE ? LPT2_ZNOISE_M
   const size_t n3 = (size_t)N * N * N;                 // instance blockIdx.z of the batch
   if (SRC != Z_NOISE) a.in += blockIdx.z * n3;
   a.out += blockIdx.z * (n3 / 2);
+  if (SRC == Z_DENSITY && a.contrast) a.contrast += blockIdx.z * n3;
   if (SRC == Z_NOISE && a.seeds) {
     const uint64_t sd = a.seeds[a.g.inst0 + blockIdx.z];
     a.seed_lo = (uint32_t)sd;
@@ -196,7 +197,16 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, SRC == Z_NOISE ? LPT2_ZNOISE_M
     } else {
       fa = __ldg(a.in + (size_t)rowa * N + n);
       fb = __ldg(a.in + (size_t)rowb * N + n);
-      if (SRC == Z_DENSITY) { fa -= 1.0f; fb -= 1.0f; }
+      if (SRC == Z_DENSITY) {
+        // density contrast rho N^3 / N_p - 1 with one particle per cell.  Written from here it
+        // costs its own bytes only (a pass of its own re-read the density: 260 us at 512^3)
+        fa -= 1.0f;
+        fb -= 1.0f;
+        if (a.contrast) {
+          a.contrast[(size_t)rowa * N + n] = fa;
+          a.contrast[(size_t)rowb * N + n] = fb;
+        }
+      }
     }
     v[r] = make_float2(fa, fb);
   }
@@ -1256,6 +1266,13 @@ __global__ void __launch_bounds__(PassCfg<N>::XT, x_minb<N>(MODE)) k_x(XArgs a) 
     for (int r = 0; r < C::RMAX; ++r) v[r] = a.in[base + (size_t)(elem<N>(t, r)) * ((size_t)N * C::H)];
   }
   const size_t blk = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+  if (MODE == X_SOURCE && a.zero) {
+    // this tile's 2 N W floats of the density to clear: the pass leaves half of the bandwidth
+    // idle, so the stores ride along (a fill kernel took 84 us at 512^3 and a launch)
+    float4* z = reinterpret_cast<float4*>(a.zero) + blk * (N * C::W / 2);
+#pragma unroll
+    for (int i = 0; i < C::RMAX / 2; ++i) z[threadIdx.x + i * C::XT] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
   x_tile<N, MODE, SPLIT>(a, v, blockIdx.x, blockIdx.y, blockIdx.z, blk, sm, s_tw, s_acc);
 }
 

@@ -61,6 +61,7 @@ struct ZR2CArgs {      // forward z pass: real rows -> half-spectrum rows
   const uint64_t* seeds;  // per global instance (Z_NOISE), or null to use seed_lo/hi
   const float4* bm;       // Box-Muller tables (Z_NOISE; boxmuller.cuh)
   float2* out;         // [N*N][N/2]
+  float* contrast;     // Z_DENSITY: the contrast (in - 1) is also written here, or null
 };
 
 struct ZC2RArgs {      // inverse z pass of one field: half-spectrum rows -> real rows
@@ -154,6 +155,8 @@ struct XArgs {
   float2* delta_out;      // X_DELTA: delta(k)
   const float2* delta_in; // X_SOURCE total mode, X_ADJ_SOURCE: delta(k)
   float2* s_out;          // X_SOURCE: S(k), kept for the adjoint (or null)
+  float* zero;            // X_SOURCE: real field [batch][N^3] the pass also clears (the density that
+                          // the particles are deposited into afterwards), 16-byte aligned, or null
   const float2* s_in;     // X_ADJ_SOURCE: S(k)
   float2* hpsi_out;       // X_ADJ_SOURCE: h_Psi(k)
   const float2* hpsi_in;  // X_ADJ_DELTA: h_Psi(k)
