@@ -807,7 +807,12 @@ int lpt2_plan(lpt2_plan_t* out, const lpt2_instance* inst, int n_inst, int n_k, 
   for (Group& g : p->groups) {
     std::vector<float2> tw(g.n);
     for (int m = 0; m < g.n; ++m) {
-      const double ang = 2.0 * M_PI * (double)twiddle_exponent(g.n, m) / (double)g.n;
+      const int e = twiddle_exponent(g.n, m);
+      if (4 * e == g.n) {   // -i exactly (cos(pi/2) is not 0 in FP64), as the in-register radices have it
+        tw[m] = make_float2(0.f, -1.f);
+        continue;
+      }
+      const double ang = 2.0 * M_PI * (double)e / (double)g.n;
       tw[m] = make_float2((float)cos(ang), (float)(-sin(ang)));
     }
     e = cudaMemcpy(g.tw, tw.data(), g.n * sizeof(float2), cudaMemcpyHostToDevice);

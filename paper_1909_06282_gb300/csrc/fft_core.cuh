@@ -54,9 +54,13 @@ __device__ __forceinline__ float2 mul_i(float2 a) { return make_float2(-a.y, a.x
 __device__ __forceinline__ float2 mul_mi(float2 a) { return make_float2(a.y, -a.x); }   // -i a
 
 // ------------------------------------------------------------ radix schedules
-// Radix sequences with the same radix first and last (so that stage-0 input and
+// V = 0: radix sequences with the same radix first and last (so that stage-0 input and
 // last-stage output share one element pattern); every radix divides RMAX.
-template <int N> struct Cfg;
+// V = 1 (where it exists): twice the values per thread and two stages, so one shared-memory
+// exchange per transform instead of two, half the twiddle loads and half the threads per
+// pencil: for passes that hold one array of values (registers).  fft() brings the outputs
+// back into the input's pattern (a renaming of registers).
+template <int N, int V = 0> struct Cfg;
 template <> struct Cfg<96>   { static constexpr int NS = 3, RMAX = 12; static __host__ __device__ constexpr int rad(int s) { return s == 1 ? 6 : 4; } };
 template <> struct Cfg<192>  { static constexpr int NS = 3, RMAX = 12; static __host__ __device__ constexpr int rad(int s) { return s == 1 ? 12 : 4; } };
 template <> struct Cfg<16>   { static constexpr int NS = 2, RMAX = 4;  static __host__ __device__ constexpr int rad(int s) { return 4; } };
@@ -70,10 +74,11 @@ template <> struct Cfg<256>  { static constexpr int NS = 2, RMAX = 16; static __
 template <> struct Cfg<512>  { static constexpr int NS = 3, RMAX = LPT2_R512;
   static __host__ __device__ constexpr int rad(int s) { return LPT2_R512 == 8 ? 8 : (s == 1 ? 2 : 16); } };
 template <> struct Cfg<1024> { static constexpr int NS = 3, RMAX = 16; static __host__ __device__ constexpr int rad(int s) { return s == 1 ? 4 : 16; } };
+template <> struct Cfg<512, 1> { static constexpr int NS = 2, RMAX = 32; static __host__ __device__ constexpr int rad(int s) { return s == 0 ? 32 : 16; } };
 
-// element index held in register slot j by lane t (first-stage input = last-stage output)
-template <int N> __host__ __device__ __forceinline__ constexpr int elem(int t, int j) {
-  constexpr int R0 = Cfg<N>::rad(0), TPP = N / Cfg<N>::RMAX;
+// element index held in register slot j by lane t (first-stage input, and output of fft())
+template <int N, int V = 0> __host__ __device__ __forceinline__ constexpr int elem(int t, int j) {
+  constexpr int R0 = Cfg<N, V>::rad(0), TPP = N / Cfg<N, V>::RMAX;
   return t + (j / R0) * TPP + (j % R0) * (N / R0);
 }
 
@@ -82,9 +87,9 @@ template <int N> __host__ __device__ __forceinline__ constexpr int wrap_idx(int 
   return ((N & (N - 1)) == 0) ? (i & (N - 1)) : (i >= N ? i - N : i);
 }
 
-template <int N> __host__ __device__ constexpr int ns_before(int s) {
+template <int N, int V = 0> __host__ __device__ constexpr int ns_before(int s) {
   int p = 1;
-  for (int i = 0; i < s; ++i) p *= Cfg<N>::rad(i);
+  for (int i = 0; i < s; ++i) p *= Cfg<N, V>::rad(i);
   return p;
 }
 
@@ -94,6 +99,7 @@ template <int N> __host__ __device__ constexpr int ns_before(int s) {
 // stages' ranges tile [ns_before(1), N).  A table in the order of the exponent puts the lanes
 // r entries apart, up to 16 to a bank (512^3: z_source 1257 -> 1141 us, z_adj_source 2223 ->
 // 1907 us, x_pkadj 438 -> 367 us by this order).  Returns the exponent m of exp(-2 pi i m / N).
+// (V = 1 of N = 512 starts its one twiddled stage at the same 32 points as V = 0's last.)
 template <int N> __host__ __device__ constexpr int twiddle_exponent(int i) {
   for (int s = 1; s < Cfg<N>::NS; ++s) {
     const int ns = ns_before<N>(s), R = Cfg<N>::rad(s);
@@ -104,17 +110,22 @@ template <int N> __host__ __device__ constexpr int twiddle_exponent(int i) {
 
 // ------------------------------------------------------- in-register DFTs
 // Forward: X[k] = sum_n x[n] exp(-2 pi i n k / R); INV flips the sign.
-// Roots of unity of order 48 (covers R = 2, 3, 4, 6, 8, 12, 16): cos / sin of
-// 2 pi j / 48, from cos(j * 7.5 deg) for j = 0..12.
-__device__ __forceinline__ float2 root48(int j, bool inv) {
-  // j in [0, 48); value exp(-+ 2 pi i j / 48)
-  const float c[13] = {1.0f, 0.99144486137381038f, 0.96592582628906831f, 0.92387953251128674f,
-                       0.86602540378443865f, 0.79335334029123517f, 0.70710678118654752f,
-                       0.60876142900872066f, 0.5f, 0.38268343236508977f, 0.25881904510252074f,
-                       0.13052619222005159f, 0.0f};
+// Roots of unity of order 96 (covers R = 2, 3, 4, 6, 8, 12, 16, 32): cos / sin of
+// 2 pi j / 96, from cos(j * 3.75 deg) for j = 0..24.
+__device__ __forceinline__ float2 root96(int j, bool inv) {
+  // j in [0, 96); value exp(-+ 2 pi i j / 96)
+  const float c[25] = {1.0f, 0.99785892323860348f, 0.99144486137381038f,
+                       0.98078528040323043f, 0.96592582628906831f, 0.94693012949510569f,
+                       0.92387953251128674f, 0.89687274153268826f, 0.86602540378443871f,
+                       0.83146961230254524f, 0.79335334029123517f, 0.75183980747897738f,
+                       0.70710678118654757f, 0.65934581510006884f, 0.60876142900872066f,
+                       0.55557023301960229f, 0.5f, 0.44228869021900125f,
+                       0.38268343236508984f, 0.3214394653031617f, 0.25881904510252074f,
+                       0.19509032201612833f, 0.13052619222005171f, 0.065403129230143048f,
+                       0.0f};
   float cs, sn;
-  const int q = j % 12, quad = j / 12;
-  const float cq = c[q], sq = c[12 - q];
+  const int q = j % 24, quad = j / 24;
+  const float cq = c[q], sq = c[24 - q];
   switch (quad) {
     case 0: cs = cq; sn = sq; break;
     case 1: cs = -sq; sn = cq; break;
@@ -150,7 +161,7 @@ template <bool INV> struct Dft<2, INV> {
 };
 
 template <int R, bool INV> struct Dft {   // even R: split into even and odd halves
-  static_assert(R % 2 == 0 && 48 % R == 0, "radix must be 2, 4, 6, 8, 12 or 16 here");
+  static_assert(R % 2 == 0 && 96 % R == 0, "radix must be 2, 4, 6, 8, 12, 16, 24 or 32 here");
   static __device__ __forceinline__ void run(float2* v) {
     float2 e[R / 2], o[R / 2];
 #pragma unroll
@@ -159,12 +170,12 @@ template <int R, bool INV> struct Dft {   // even R: split into even and odd hal
     Dft<R / 2, INV>::run(o);
 #pragma unroll
     for (int k = 0; k < R / 2; ++k) {
-      const int j = k * (48 / R);   // exponent in units of 2 pi / 48
+      const int j = k * (96 / R);   // exponent in units of 2 pi / 96
       float2 t;
       if (j == 0) t = o[k];
-      else if (j == 12) t = INV ? mul_i(o[k]) : mul_mi(o[k]);
-      else t = cmul(o[k], root48(j, INV));
-      if (j == 12) {   // t is o with its parts swapped: scalar adds read the swap in place
+      else if (j == 24) t = INV ? mul_i(o[k]) : mul_mi(o[k]);
+      else t = cmul(o[k], root96(j, INV));
+      if (j == 24) {   // t is o with its parts swapped: scalar adds read the swap in place
         v[k] = cadd(e[k], t);
         v[k + R / 2] = csub(e[k], t);
       } else {
@@ -204,13 +215,14 @@ template <int W> struct SmemCol {
 // Runs all stages on v (in: x[t + r TPP], out: X[t + r TPP]).  Every thread of
 // the CTA (of the warp, for a warp-private row layout) must call this the same number
 // of times (it contains the layout's barriers).
-template <int N, bool INV, int S, class SM>
-__device__ __forceinline__ void fft_stages(float2 (&v)[Cfg<N>::RMAX], int t, const SM& sm,
+template <int N, bool INV, int S, int V, class SM>
+__device__ __forceinline__ void fft_stages(float2 (&v)[Cfg<N, V>::RMAX], int t, const SM& sm,
                                            const float2* __restrict__ tw) {
-  constexpr int RMAX = Cfg<N>::RMAX;
+  using C = Cfg<N, V>;
+  constexpr int RMAX = C::RMAX;
   constexpr int TPP = N / RMAX;
-  constexpr int R = Cfg<N>::rad(S);
-  constexpr int NS = ns_before<N>(S);
+  constexpr int R = C::rad(S);
+  constexpr int NS = ns_before<N, V>(S);
   constexpr int NB = RMAX / R;
 #pragma unroll
   for (int q = 0; q < NB; ++q) {
@@ -226,7 +238,7 @@ __device__ __forceinline__ void fft_stages(float2 (&v)[Cfg<N>::RMAX], int t, con
     }
     Dft<R, INV>::run(&v[q * R]);
   }
-  if constexpr (S + 1 < Cfg<N>::NS) {
+  if constexpr (S + 1 < C::NS) {
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
       const int b = t + q * TPP;
@@ -235,7 +247,7 @@ __device__ __forceinline__ void fft_stages(float2 (&v)[Cfg<N>::RMAX], int t, con
       for (int r = 0; r < R; ++r) sm.st(d + r * NS, v[q * R + r]);
     }
     sm.sync();
-    constexpr int R2 = Cfg<N>::rad(S + 1);
+    constexpr int R2 = C::rad(S + 1);
 #pragma unroll
     for (int q = 0; q < RMAX / R2; ++q) {
       const int b = t + q * TPP;
@@ -243,14 +255,25 @@ __device__ __forceinline__ void fft_stages(float2 (&v)[Cfg<N>::RMAX], int t, con
       for (int r = 0; r < R2; ++r) v[q * R2 + r] = sm.ld(b + r * (N / R2));
     }
     sm.sync();
-    fft_stages<N, INV, S + 1, SM>(v, t, sm, tw);
+    fft_stages<N, INV, S + 1, V, SM>(v, t, sm, tw);
+  } else if constexpr (R != C::rad(0)) {
+    // output (q, r) is element t + q TPP + r NS: back into the order of elem()
+    constexpr int R0 = C::rad(0);
+    float2 o[RMAX];
+#pragma unroll
+    for (int i = 0; i < RMAX; ++i) {
+      const int m = i / R + (i % R) * (NS / TPP);          // element t + m TPP
+      o[(m % (N / R0 / TPP)) * R0 + m / (N / R0 / TPP)] = v[i];
+    }
+#pragma unroll
+    for (int i = 0; i < RMAX; ++i) v[i] = o[i];
   }
 }
 
-template <int N, bool INV, class SM>
-__device__ __forceinline__ void fft(float2 (&v)[Cfg<N>::RMAX], int t, const SM& sm,
+template <int N, bool INV, int V = 0, class SM>
+__device__ __forceinline__ void fft(float2 (&v)[Cfg<N, V>::RMAX], int t, const SM& sm,
                                     const float2* __restrict__ tw) {
-  fft_stages<N, INV, 0, SM>(v, t, sm, tw);
+  fft_stages<N, INV, 0, V, SM>(v, t, sm, tw);
 }
 
 // Copy the N-entry twiddle table to shared memory (all threads participate).

@@ -51,15 +51,22 @@ template <int N> struct PassCfg {
 // whole (ky, kz) plane apart, and the two passes hold different working sets).  WY = 0 is
 // the build default; the launcher also has WY = 8 and 16 compiled, which a plan's tile
 // schedule (Geo::ytile) selects per grid-size group.
-#ifndef LPT2_WY512
-#define LPT2_WY512 LPT2_W512
-#endif
-template <int N, int WY = 0> struct YCfg {
-  static constexpr int RMAX = Cfg<N>::RMAX;
-  static constexpr int TPP = N / RMAX;
+//
+// N = 512, one array of values (Y_ONE, Y_MULTI): bound by DRAM, whose rows want 128-byte
+// segments, so 16 kz per CTA; with 16 values per thread that CTA has 512 threads that
+// wait for one another (y_phi 1399 us), with 32 values 256 threads and one exchange instead
+// of two: y_phi 1067 -> 930 us, y_psi 537 -> 463, y_fwd 215 -> 184 against 8 kz and 16
+// values.  Two CTAs per SM: a third fits in registers (80), but its tile takes the L1 the loads in
+// flight need (y_phi 1098 us).  Y_SUM keeps an accumulator beside the values: 8 kz, 16 values.
+enum YKind { Y_MULTI = 0, Y_SUM = 1, Y_ONE = 2 };
+template <int N, int KIND, int WY = 0> struct YCfg {
   static constexpr int H = N / 2;
-  static constexpr int W = WY ? WY : (N == 512 ? LPT2_WY512 : PassCfg<N>::W);
+  static constexpr int W = WY ? WY : (N == 512 ? (KIND == Y_SUM ? 8 : 16) : PassCfg<N>::W);
+  static constexpr int V = N == 512 && W == 16 && KIND != Y_SUM ? 1 : 0;
+  static constexpr int RMAX = Cfg<N, V>::RMAX;
+  static constexpr int TPP = N / RMAX;
   static constexpr int XT = TPP * W;
+  static constexpr int MINB = V ? 2 : 0;   // resident CTAs asked of the compiler (0: none)
   static constexpr int XSMEM = (N + N * W) * 8;
   static_assert(H % W == 0, "a CTA's kz block must tile the half spectrum");
 };
@@ -802,11 +809,9 @@ __global__ void __launch_bounds__(ZAdjFpCfg<N>::THREADS, 2) k_z_adj_source_fp(ZA
 //                input copy stays in registers;
 //       Y_SUM    out[dst[i]] += conj((i k_y)^ord[i]) forward-transform(in[i]);
 //       Y_ONE    one input, one output, no derivative (forward or inverse).
-enum YKind { Y_MULTI = 0, Y_SUM = 1, Y_ONE = 2 };
-
 template <int N, int KIND, int WY>
-__global__ void __launch_bounds__(YCfg<N, WY>::XT) k_y(YArgs a) {
-  using C = YCfg<N, WY>;
+__global__ void __launch_bounds__(YCfg<N, KIND, WY>::XT, YCfg<N, KIND, WY>::MINB) k_y(YArgs a) {
+  using C = YCfg<N, KIND, WY>;
   extern __shared__ float2 smem[];
   float2* s_tw = smem;
   load_twiddles(s_tw, a.tw, N);
@@ -825,30 +830,30 @@ __global__ void __launch_bounds__(YCfg<N, WY>::XT) k_y(YArgs a) {
         if (a.job.dst[i] != o) continue;
         float2 v[C::RMAX];
 #pragma unroll
-        for (int r = 0; r < C::RMAX; ++r) v[r] = a.job.in[i][base + (size_t)(elem<N>(t, r)) * C::H];
-        fft<N, false>(v, t, sm, s_tw);
+        for (int r = 0; r < C::RMAX; ++r) v[r] = a.job.in[i][base + (size_t)(elem<N, C::V>(t, r)) * C::H];
+        fft<N, false, C::V>(v, t, sm, s_tw);
         const int zo = a.job.zord[i];
 #pragma unroll
         for (int r = 0; r < C::RMAX; ++r) {
-          const int n = elem<N>(t, r);
+          const int n = elem<N, C::V>(t, r);
           const float2 u = dconj(v[r], a.g.kf * (float)mode_of(n, N), a.job.ord[i]);
           acc[r] = cadd(acc[r], zo ? dconj(u, a.g.kf * (float)kz, zo) : u);
         }
       }
       float2* dst = a.job.out[o];
 #pragma unroll
-      for (int r = 0; r < C::RMAX; ++r) dst[base + (size_t)(elem<N>(t, r)) * C::H] = acc[r];
+      for (int r = 0; r < C::RMAX; ++r) dst[base + (size_t)(elem<N, C::V>(t, r)) * C::H] = acc[r];
     }
     return;
   }
   if (KIND == Y_ONE) {
     float2 v[C::RMAX];
 #pragma unroll
-    for (int r = 0; r < C::RMAX; ++r) v[r] = a.job.in[0][base + (size_t)(elem<N>(t, r)) * C::H];
-    if (a.inverse) fft<N, true>(v, t, sm, s_tw);
-    else fft<N, false>(v, t, sm, s_tw);
+    for (int r = 0; r < C::RMAX; ++r) v[r] = a.job.in[0][base + (size_t)(elem<N, C::V>(t, r)) * C::H];
+    if (a.inverse) fft<N, true, C::V>(v, t, sm, s_tw);
+    else fft<N, false, C::V>(v, t, sm, s_tw);
 #pragma unroll
-    for (int r = 0; r < C::RMAX; ++r) a.job.out[0][base + (size_t)(elem<N>(t, r)) * C::H] = v[r];
+    for (int r = 0; r < C::RMAX; ++r) a.job.out[0][base + (size_t)(elem<N, C::V>(t, r)) * C::H] = v[r];
     return;
   }
   for (int o = 0; o < a.job.n_out; ++o) {
@@ -857,15 +862,15 @@ __global__ void __launch_bounds__(YCfg<N, WY>::XT) k_y(YArgs a) {
     float2 v[C::RMAX];
 #pragma unroll
     for (int r = 0; r < C::RMAX; ++r) {
-      const int n = elem<N>(t, r);
+      const int n = elem<N, C::V>(t, r);
       const float2 u = src[base + (size_t)n * C::H];
       v[r] = (m != 0 && n == C::H) ? make_float2(0.f, 0.f) : deriv(u, a.g.kf * (float)mode_of(n, N), m);
     }
-    if (a.inverse) fft<N, true>(v, t, sm, s_tw);
-    else fft<N, false>(v, t, sm, s_tw);
+    if (a.inverse) fft<N, true, C::V>(v, t, sm, s_tw);
+    else fft<N, false, C::V>(v, t, sm, s_tw);
     float2* dst = a.job.out[o];
 #pragma unroll
-    for (int r = 0; r < C::RMAX; ++r) dst[base + (size_t)(elem<N>(t, r)) * C::H] = v[r];
+    for (int r = 0; r < C::RMAX; ++r) dst[base + (size_t)(elem<N, C::V>(t, r)) * C::H] = v[r];
   }
 }
 
@@ -1549,8 +1554,9 @@ template <int N> cudaError_t launch_z_adj_source_t(const ZAdjSourceArgs& a, cuda
   k_z_adj_source<N><<<dim3(N * N / Q::ROWS, 1, a.g.batch), C::ZT, Q::SMEM, s>>>(a);
   return cudaGetLastError();
 }
-template <int N, int KIND, int WY> cudaError_t launch_y_k(const YArgs& a, cudaStream_t s) {
-  using C = YCfg<N, WY>;
+template <int N, int KIND, int WYA> cudaError_t launch_y_k(const YArgs& a, cudaStream_t s) {
+  constexpr int WY = WYA == YCfg<N, KIND>::W ? 0 : WYA;   // the default by its number: one instance
+  using C = YCfg<N, KIND, WY>;
   LPT2_CHECK_BATCH(a);
   cudaFuncSetAttribute(k_y<N, KIND, WY>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::XSMEM);
   k_y<N, KIND, WY><<<dim3(C::H / C::W, N, a.g.batch), C::XT, C::XSMEM, s>>>(a);
@@ -1564,13 +1570,11 @@ template <int N, int WY> cudaError_t launch_y_w(const YArgs& a, cudaStream_t s) 
 }
 // y pencils per CTA: Geo::ytile 0 (build default), 8 or 16 (where they tile N/2)
 template <int N> cudaError_t launch_y_t(const YArgs& a, cudaStream_t s) {
-  if constexpr (N >= 32 && YCfg<N>::W != 8) {
-    if (a.g.ytile == 8) return launch_y_w<N, 8>(a, s);
-  }
-  if constexpr (N >= 32 && YCfg<N>::W != 16) {
+  if (a.g.ytile == 8) return launch_y_w<N, 8>(a, s);
+  if constexpr (N >= 32) {
     if (a.g.ytile == 16) return launch_y_w<N, 16>(a, s);
   }
-  if (a.g.ytile != 0 && a.g.ytile != YCfg<N>::W) return cudaErrorInvalidValue;
+  if (a.g.ytile != 0) return cudaErrorInvalidValue;
   return launch_y_w<N, 0>(a, s);
 }
 // persistent bulk-tensor x pass: as many CTAs as fit on the GPU at once, or one per tile
