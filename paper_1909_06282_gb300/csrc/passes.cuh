@@ -179,6 +179,7 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, SRC == Z_NOISE ? LPT2_ZNOISE_M
     bm_load_table(s_bm, a.bm);
     __syncthreads();
   }
+  if (SRC != Z_NOISE) grid_sync_and_trigger();
   const int p = threadIdx.x / C::TPP, t = threadIdx.x % C::TPP;
   const SmemRowT<kRowWarp<N>> sm{smem + N + p * SmemRow::words(N)};
   const int pair = blockIdx.x * C::ZP + p;
@@ -217,6 +218,7 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, SRC == Z_NOISE ? LPT2_ZNOISE_M
     }
     v[r] = make_float2(fa, fb);
   }
+  if (SRC == Z_NOISE) grid_sync_and_trigger();   // the draws need nothing of the earlier kernels
   __syncthreads();   // twiddles visible
   fft<N, false>(v, t, sm, s_tw);
   z_store_pair<N>(v, t, sm, a.out + (size_t)rowa * C::H, a.out + (size_t)rowb * C::H);
@@ -228,6 +230,7 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_c2r(ZC2RArgs 
   extern __shared__ float2 smem[];
   float2* s_tw = smem;
   load_twiddles(s_tw, a.tw, N);
+  grid_sync_and_trigger();
   const int p = threadIdx.x / C::TPP, t = threadIdx.x % C::TPP;
   const SmemRowT<kRowWarp<N>> sm{smem + N + p * SmemRow::words(N)};
   const int pair = blockIdx.x * C::ZP + p;
@@ -310,6 +313,8 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_source(ZSourc
     for (int s = 0; s < Q::STAGES; ++s) mbar_init(&bar[s], 1);
     mbar_init_fence();
   }
+  load_twiddles(s_tw, a.tw, N);
+  grid_sync_and_trigger();
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int f = 0; f < Q::STAGES; ++f) {
@@ -317,7 +322,6 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_source(ZSourc
       bulk_load(ring + f * Q::STAGE_F2, a.in[f] + zoff + tile, Q::STAGE_BYTES, &bar[f]);
     }
   }
-  load_twiddles(s_tw, a.tw, N);
   // field f of the ring into v, then the copy of field f + STAGES; false if a wait ran out
   // (the CTA has then drained its copies and reported, and must return)
   auto fetch = [&](int f, float2 (&v)[C::RMAX]) -> bool {
@@ -460,6 +464,8 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_final(ZFinalA
     for (int st = 0; st < Q::STAGES; ++st) mbar_init(&bar[st], 1);
     mbar_init_fence();
   }
+  load_twiddles(s_tw, a.tw, N);
+  grid_sync_and_trigger();
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int q = 0; q < Q::STAGES && q < NQ; ++q) {
@@ -467,7 +473,6 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_final(ZFinalA
       bulk_load(ring + q * Q::STAGE_F2, input(q), Q::STAGE_BYTES, &bar[q]);
     }
   }
-  load_twiddles(s_tw, a.tw, N);
   float2 keep[C::RMAX];
 #pragma unroll 1
   for (int q = 0; q < NQ; ++q) {
@@ -594,6 +599,8 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_adj_source(ZA
     for (int st = 0; st < Q::STAGES; ++st) mbar_init(&bar[st], 1);
     mbar_init_fence();
   }
+  load_twiddles(s_tw, a.tw, N);
+  grid_sync_and_trigger();
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int q = 0; q < Q::STAGES; ++q) {
@@ -601,7 +608,6 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_adj_source(ZA
       bulk_load(ring + q * Q::STAGE_F2, a.in[field(q)] + zs + tile, Q::STAGE_BYTES, &bar[q]);
     }
   }
-  load_twiddles(s_tw, a.tw, N);
   // Stage q of the ring into v (z_assemble with the field's z-derivative order), then the
   // copy of stage q + STAGES; false if a wait ran out (the CTA has then drained its copies
   // and reported, and must return).
@@ -727,11 +733,14 @@ __global__ void __launch_bounds__(ZAdjFpCfg<N>::THREADS, 2) k_z_adj_source_fp(ZA
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
     mbar_init_fence();
-    issue(0);
-    issue(1);
   }
   const float* gsr = a.gs + zr + row * N;   // g_S of this row (read where used: registers are short)
   load_twiddles(s_tw, a.tw, N);
+  grid_sync_and_trigger();
+  if (threadIdx.x == 0) {
+    issue(0);
+    issue(1);
+  }
   __syncthreads();
   // pencil k of this warp's row into v (Hermitian extension of both fields with their z
   // derivative orders, Z = A + i B); false if a wait ran out (drained and reported)
@@ -815,6 +824,7 @@ __global__ void __launch_bounds__(YCfg<N, KIND, WY>::XT, YCfg<N, KIND, WY>::MINB
   extern __shared__ float2 smem[];
   float2* s_tw = smem;
   load_twiddles(s_tw, a.tw, N);
+  grid_sync_and_trigger();
   const int w = threadIdx.x % C::W, t = threadIdx.x / C::W;
   const SmemCol<C::W> sm{smem + N + w};
   const int kz = blockIdx.x * C::W + w;
@@ -1253,6 +1263,7 @@ __global__ void __launch_bounds__(PassCfg<N>::XT, x_minb<N>(MODE)) k_x(XArgs a) 
   extern __shared__ float2 smem[];
   float2* s_tw = smem;
   load_twiddles(s_tw, a.tw, N);
+  grid_sync_and_trigger();
   const int w = threadIdx.x % C::W, t = threadIdx.x / C::W;
   const SmemCol<C::W> sm{smem + N + w};
   double* s_acc = reinterpret_cast<double*>(smem + N + N * C::W);   // per-warp accumulators
@@ -1339,10 +1350,13 @@ __global__ void __launch_bounds__(PassCfg<N>::XT, x_minb<N>(MODE)) k_x_tma(const
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
     mbar_init_fence();
+  }
+  load_twiddles(s_tw, a.tw, N);
+  grid_sync_and_trigger();
+  if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i)
       if (blockIdx.x + i * gridDim.x < ntiles) issue(i, blockIdx.x + i * gridDim.x);
   }
-  load_twiddles(s_tw, a.tw, N);
   __syncthreads();
   for (int i = 0, tile = blockIdx.x; tile < ntiles; ++i, tile += gridDim.x) {
     const int st = i & 1;
@@ -1432,9 +1446,11 @@ __global__ void __launch_bounds__(PassCfg<N>::XT, x_minb<N>(MODE)) k_x_tma_adj(c
     s_fail = 0;
     for (int st = 0; st < 3; ++st) mbar_init(&bar[st], 1);
     mbar_init_fence();
-    while (issued < 3 && issued < nload) issue();
   }
   load_twiddles(s_tw, a.tw, N);
+  grid_sync_and_trigger();
+  if (threadIdx.x == 0)
+    while (issued < 3 && issued < nload) issue();
   __syncthreads();
   int c = 0;                           // next input to wait for
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
@@ -1505,8 +1521,7 @@ template <int N, int SRC> cudaError_t launch_z_r2c_m(const ZR2CArgs& a, cudaStre
   LPT2_CHECK_BATCH(a);
   constexpr int smem = zr2c_smem<N, SRC>();
   cudaFuncSetAttribute(k_z_r2c<N, SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  k_z_r2c<N, SRC><<<dim3(N * N / 2 / C::ZP, 1, a.g.batch), C::ZT, smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_overlapped(k_z_r2c<N, SRC>, dim3(N * N / 2 / C::ZP, 1, a.g.batch), C::ZT, smem, s, a);
 }
 template <int N> cudaError_t launch_z_r2c_t(const ZR2CArgs& a, cudaStream_t s) {
   switch (a.src) {
@@ -1520,16 +1535,14 @@ template <int N> cudaError_t launch_z_c2r_t(const ZC2RArgs& a, cudaStream_t s) {
   using C = PassCfg<N>;
   LPT2_CHECK_BATCH(a);
   cudaFuncSetAttribute(k_z_c2r<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::ZSMEM);
-  k_z_c2r<N><<<dim3(N * N / 2 / C::ZP, 1, a.g.batch), C::ZT, C::ZSMEM, s>>>(a);
-  return cudaGetLastError();
+  return launch_overlapped(k_z_c2r<N>, dim3(N * N / 2 / C::ZP, 1, a.g.batch), C::ZT, C::ZSMEM, s, a);
 }
 template <int N> cudaError_t launch_z_source_t(const ZSourceArgs& a, cudaStream_t s) {
   using C = PassCfg<N>;
   LPT2_CHECK_BATCH(a);
   using Q = ZSrcCfg<N>;
   cudaFuncSetAttribute(k_z_source<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, Q::SMEM);
-  k_z_source<N><<<dim3(N * N / Q::ROWS, 1, a.g.batch), C::ZT, Q::SMEM, s>>>(a);
-  return cudaGetLastError();
+  return launch_overlapped(k_z_source<N>, dim3(N * N / Q::ROWS, 1, a.g.batch), C::ZT, Q::SMEM, s, a);
 }
 template <int N> cudaError_t launch_z_final_t(const ZFinalArgs& a, cudaStream_t s) {
   using C = PassCfg<N>;
@@ -1537,8 +1550,7 @@ template <int N> cudaError_t launch_z_final_t(const ZFinalArgs& a, cudaStream_t 
   using Q = ZSrcCfg<N>;
   auto k = a.split ? k_z_final<N, true> : k_z_final<N, false>;
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Q::SMEM);
-  k<<<dim3(N * N / Q::ROWS, 1, a.g.batch), C::ZT, Q::SMEM, s>>>(a);
-  return cudaGetLastError();
+  return launch_overlapped(k, dim3(N * N / Q::ROWS, 1, a.g.batch), C::ZT, Q::SMEM, s, a);
 }
 template <int N> cudaError_t launch_z_adj_source_t(const ZAdjSourceArgs& a, cudaStream_t s) {
   using C = PassCfg<N>;
@@ -1547,20 +1559,17 @@ template <int N> cudaError_t launch_z_adj_source_t(const ZAdjSourceArgs& a, cuda
   if constexpr (zadj_field_pairs<N>()) {
     using F = ZAdjFpCfg<N>;
     cudaFuncSetAttribute(k_z_adj_source_fp<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, F::SMEM);
-    k_z_adj_source_fp<N><<<dim3(N * N / F::ROWS, 1, a.g.batch), F::THREADS, F::SMEM, s>>>(a);
-    return cudaGetLastError();
+    return launch_overlapped(k_z_adj_source_fp<N>, dim3(N * N / F::ROWS, 1, a.g.batch), F::THREADS, F::SMEM, s, a);
   }
   cudaFuncSetAttribute(k_z_adj_source<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, Q::SMEM);
-  k_z_adj_source<N><<<dim3(N * N / Q::ROWS, 1, a.g.batch), C::ZT, Q::SMEM, s>>>(a);
-  return cudaGetLastError();
+  return launch_overlapped(k_z_adj_source<N>, dim3(N * N / Q::ROWS, 1, a.g.batch), C::ZT, Q::SMEM, s, a);
 }
 template <int N, int KIND, int WYA> cudaError_t launch_y_k(const YArgs& a, cudaStream_t s) {
   constexpr int WY = WYA == YCfg<N, KIND>::W ? 0 : WYA;   // the default by its number: one instance
   using C = YCfg<N, KIND, WY>;
   LPT2_CHECK_BATCH(a);
   cudaFuncSetAttribute(k_y<N, KIND, WY>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::XSMEM);
-  k_y<N, KIND, WY><<<dim3(C::H / C::W, N, a.g.batch), C::XT, C::XSMEM, s>>>(a);
-  return cudaGetLastError();
+  return launch_overlapped(k_y<N, KIND, WY>, dim3(C::H / C::W, N, a.g.batch), C::XT, C::XSMEM, s, a);
 }
 template <int N, int WY> cudaError_t launch_y_w(const YArgs& a, cudaStream_t s) {
   if (a.job.sum) return launch_y_k<N, Y_SUM, WY>(a, s);
@@ -1594,8 +1603,7 @@ template <int N, int MODE, bool SC> cudaError_t launch_x_tma(const XArgs& a, int
     return e;
   const long long tiles = (long long)Q::KZB * N * a.g.batch;
   const int grid = (int)std::min<long long>(tiles, (long long)sms * std::max(per_sm, 1));
-  k_x_tma<N, MODE, SC><<<grid, C::XT, smem, s>>>(b);
-  return cudaGetLastError();
+  return launch_overlapped(k_x_tma<N, MODE, SC>, grid, C::XT, smem, s, b);
 }
 #ifndef LPT2_X_TMA_ADJ
 #define LPT2_X_TMA_ADJ 1
@@ -1618,8 +1626,7 @@ template <int N, int MODE> cudaError_t launch_x_tma_adj(const XArgs& a, int acc,
     return e;
   const long long tiles = (long long)Q::KZB * N * a.g.batch;
   const int grid = (int)std::min<long long>(tiles, (long long)sms * std::max(per_sm, 1));
-  k_x_tma_adj<N, MODE><<<grid, C::XT, smem, s>>>(b);
-  return cudaGetLastError();
+  return launch_overlapped(k_x_tma_adj<N, MODE>, grid, C::XT, smem, s, b);
 }
 template <int N, int MODE> cudaError_t launch_x_m(const XArgs& a, cudaStream_t s) {
   using C = PassCfg<N>;
@@ -1647,8 +1654,7 @@ template <int N, int MODE> cudaError_t launch_x_m(const XArgs& a, cudaStream_t s
   constexpr bool has_split = MODE == X_DELTA || MODE == X_SOURCE;
   auto k = has_split && a.split ? k_x<N, MODE, has_split> : k_x<N, MODE, false>;
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  k<<<dim3(C::H / C::W, N, a.g.batch), C::XT, smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_overlapped(k, dim3(C::H / C::W, N, a.g.batch), C::XT, smem, s, a);
 }
 template <int N> cudaError_t launch_x_t(const XArgs& a, cudaStream_t s) {
   switch (a.mode) {

@@ -9,6 +9,23 @@
 
 namespace lpt2 {
 
+// Launches a kernel that calls grid_sync_and_trigger(): it may start while the stream's
+// previous kernel drains, up to that call (programmatic dependent launch).
+template <class... P, class... A>
+cudaError_t launch_overlapped(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, P(args)...);
+}
+
 // Written by the cosmology set-up kernels (FP64 in, FP32 constants out).
 struct DevCosmo {
   double amp;        // P(k) amplitude A (sigma_8 normalisation), (Mpc/h)^(3+n_s)

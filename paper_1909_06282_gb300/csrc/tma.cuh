@@ -15,6 +15,17 @@ namespace lpt2 {
 #define LPT2_WAIT_CYCLES 2000000000LL   // ~1 s at 2 GHz
 #endif
 
+// Start of a kernel launched with launch_overlapped (passes.h): waits until the stream's earlier
+// kernels have completed and their writes are visible, then lets the next kernel's CTAs start
+// where this one's leave room.  Before it a kernel touches only shared memory and tables that
+// the plan wrote once (twiddles): whatever starts here has all but its direct predecessor
+// behind it, because that one has passed its own wait.  At 64^3 the launches of a step are
+// 1.5-2 us apart without it.
+__device__ __forceinline__ void grid_sync_and_trigger() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
 }
