@@ -15,6 +15,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "packed.cuh"
+
 namespace lpt2 {
 
 // ---------------------------------------------------------------- complex ops
@@ -23,31 +25,12 @@ __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
-// cadd and csub as one packed instruction (add / sub.rn.f32x2: the same roundings).  The packed
-// form has the arithmetic rate of two scalar adds but takes one issue slot instead of two
-// (measured: 0.53 against 1.04 instructions per cycle and scheduler), and the passes with
-// several transforms per field are bound by issue and shared-memory slots: z_source at 512^3
-// 1141 -> 1071 us, z_final 636 -> 617 us, x_pkadj 367 -> 341 us.  Products stay scalar: a packed
-// complex product needs swapped or doubled operands, whose moves cost what it saves.
-__device__ __forceinline__ float2 padd(float2 a, float2 b) {
-#ifdef __CUDA_ARCH__
-  return __fadd2_rn(a, b);
-#else
-  return cadd(a, b);
-#endif
-}
-__device__ __forceinline__ float2 psub(float2 a, float2 b) {
-#ifdef __CUDA_ARCH__
-  float2 o;
-  asm("{\n\t.reg .b64 p, q, r;\n\tmov.b64 p, {%2, %3};\n\tmov.b64 q, {%4, %5};\n\tsub.rn.f32x2 r, p, q;\n\t"
-      "mov.b64 {%0, %1}, r;\n\t}"
-      : "=f"(o.x), "=f"(o.y)
-      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-  return o;
-#else
-  return csub(a, b);
-#endif
-}
+// The radix butterflies add with padd / psub (packed.cuh).  A packed add has the arithmetic rate
+// of two scalar adds but takes one issue slot instead of two (measured: 0.53 against 1.04
+// instructions per cycle and scheduler), and the passes with several transforms per field are
+// bound by issue and shared-memory slots: z_source at 512^3 1141 -> 1071 us, z_final 636 -> 617
+// us, x_pkadj 367 -> 341 us.  Products stay scalar: a packed complex product needs swapped or
+// doubled operands, whose moves cost what it saves.
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
 __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
 __device__ __forceinline__ float2 mul_i(float2 a) { return make_float2(-a.y, a.x); }    // i a

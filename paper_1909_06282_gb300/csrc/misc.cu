@@ -441,15 +441,20 @@ cudaError_t launch_pk_finalize_p(const double* part, int n_blocks, int n_shells,
   return launch_overlapped(k_pk_finalize_p, batch, 256, 0, s, scratch, G, n_shells, ksum, count, pk, k_mean, n_modes);
 }
 
+// A thread draws the pairs of two consecutive cells along z: rows iy (even) and iy + 1.
 __global__ void k_noise(int n, uint32_t k0, uint32_t k1, const float4* __restrict__ g_bm, float* out) {
   __shared__ float4 bm[kBmTableLen];
   bm_load_table(bm, g_bm);
   __syncthreads();
-  const size_t n3 = (size_t)n * n * n;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n3; i += (size_t)gridDim.x * blockDim.x) {
-    const bool odd = ((i / n) % n) & 1;   // iy odd: sine output of the draw at iy - 1
-    const float2 g2 = philox_gauss2(odd ? i - n : i, k0, k1, bm);
-    out[i] = odd ? g2.y : g2.x;
+  const size_t quads = (size_t)n * n * n / 4;
+  const int nz = n / 2;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < quads; i += (size_t)gridDim.x * blockDim.x) {
+    const size_t cell = (i / nz) * 2 * n + 2 * (i % nz);   // (ix, iy, iz) with iy and iz even
+    const float4 g = philox_gauss2x2(cell, cell + 1, k0, k1, bm);
+    out[cell] = g.x;
+    out[cell + 1] = g.z;
+    out[cell + n] = g.y;
+    out[cell + n + 1] = g.w;
   }
 }
 
@@ -463,9 +468,13 @@ __global__ void k_box_muller(const uint2* __restrict__ w, int64_t count, const f
   __shared__ float4 bm[kBmTableLen];
   bm_load_table(bm, g_bm);
   __syncthreads();
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
-    const uint2 x = w[i];
-    out[i] = bm_pair(x.x, x.y, bm);
+  const int64_t pairs = (count + 1) / 2;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < pairs; i += (int64_t)gridDim.x * blockDim.x) {
+    const bool two = 2 * i + 1 < count;
+    const uint2 x = w[2 * i];
+    const float4 g = bm_pair2(x, two ? w[2 * i + 1] : x, bm);
+    out[2 * i] = make_float2(g.x, g.y);
+    if (two) out[2 * i + 1] = make_float2(g.z, g.w);
   }
 }
 

@@ -194,15 +194,19 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, SRC == Z_NOISE ? LPT2_ZNOISE_M
     a.seed_hi = (uint32_t)(sd >> 32);
   }
   float2 v[C::RMAX];
+  if (SRC == Z_NOISE) {   // rows (x, y) and (x, y+1), y even: one Box-Muller pair per z, two z at a time
 #pragma unroll
-  for (int r = 0; r < C::RMAX; ++r) {
-    const int n = elem<N>(t, r);
-    float fa, fb;
-    if (SRC == Z_NOISE) {   // rows (x, y) and (x, y+1), y even: one Box-Muller pair per z
-      const float2 g2 = philox_gauss2((uint64_t)rowa * N + n, a.seed_lo, a.seed_hi, s_bm);
-      fa = g2.x;
-      fb = g2.y;
-    } else {
+    for (int r = 0; r < C::RMAX; r += 2) {
+      const uint64_t row = (uint64_t)rowa * N;
+      const float4 g = philox_gauss2x2(row + elem<N>(t, r), row + elem<N>(t, r + 1), a.seed_lo, a.seed_hi, s_bm);
+      v[r] = make_float2(g.x, g.y);
+      v[r + 1] = make_float2(g.z, g.w);
+    }
+  } else {
+#pragma unroll
+    for (int r = 0; r < C::RMAX; ++r) {
+      const int n = elem<N>(t, r);
+      float fa, fb;
       fa = __ldg(a.in + (size_t)rowa * N + n);
       fb = __ldg(a.in + (size_t)rowb * N + n);
       if (SRC == Z_DENSITY) {
@@ -215,8 +219,8 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, SRC == Z_NOISE ? LPT2_ZNOISE_M
           a.contrast[(size_t)rowb * N + n] = fb;
         }
       }
+      v[r] = make_float2(fa, fb);
     }
-    v[r] = make_float2(fa, fb);
   }
   if (SRC == Z_NOISE) grid_sync_and_trigger();   // the draws need nothing of the earlier kernels
   __syncthreads();   // twiddles visible

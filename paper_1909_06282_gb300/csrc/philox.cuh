@@ -28,12 +28,14 @@ __host__ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, ui
   return c;
 }
 
-// (g_even, g_odd) = sqrt(-2 ln u0) (cos, sin)(2 pi u1), u = ((x >> 8) + 1) 2^-24, for the
-// pair drawn at `cell`, each the correctly rounded FP32 value (boxmuller.cuh).
-__device__ __forceinline__ float2 philox_gauss2(uint64_t cell, uint32_t k0, uint32_t k1,
-                                                const float4* bm) {
-  const uint4 x = philox4x32_10(make_uint4((uint32_t)cell, (uint32_t)(cell >> 32), 0u, 0u), k0, k1);
-  return bm_pair(x.x, x.y, bm);
+// (g_even, g_odd) = sqrt(-2 ln u0) (cos, sin)(2 pi u1), u = ((x >> 8) + 1) 2^-24, for the pairs
+// drawn at `cell0` (.x, .y) and `cell1` (.z, .w), each the correctly rounded FP32 value
+// (boxmuller.cuh).
+__device__ __forceinline__ float4 philox_gauss2x2(uint64_t cell0, uint64_t cell1, uint32_t k0, uint32_t k1,
+                                                  const float4* bm) {
+  const uint4 x = philox4x32_10(make_uint4((uint32_t)cell0, (uint32_t)(cell0 >> 32), 0u, 0u), k0, k1);
+  const uint4 y = philox4x32_10(make_uint4((uint32_t)cell1, (uint32_t)(cell1 >> 32), 0u, 0u), k0, k1);
+  return bm_pair2(make_uint2(x.x, x.y), make_uint2(y.x, y.y), bm);
 }
 
 }  // namespace lpt2
