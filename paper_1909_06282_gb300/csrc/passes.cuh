@@ -71,6 +71,24 @@ template <int N, int KIND, int WY = 0> struct YCfg {
   static_assert(H % W == 0, "a CTA's kz block must tile the half spectrum");
 };
 
+// x passes: the tile of a mode.  V = 1 as in the y passes (N = 512, modes that hold one array of
+// values): 16 kz and 32 values per thread, x_fwd 275 -> 185 us, x_inv 284 -> 182, x_pkadj 343 ->
+// 334.  Not the shell sums: they want the resident warps that 64 registers allow (250 us against
+// 275 with 32 values).
+template <int N, int MODE> struct XCfg {
+  static constexpr int V = N == 512 && (MODE == X_FWD || MODE == X_INV || MODE == X_PKADJ || MODE == X_MUL) ? 1 : 0;
+  static constexpr int RMAX = Cfg<N, V>::RMAX;
+  static constexpr int TPP = N / RMAX;
+  static constexpr int H = N / 2;
+  static constexpr int W = V ? 16 : PassCfg<N>::W;   // kz per CTA
+  static constexpr int XT = TPP * W;
+  static constexpr int XSMEM = (N + N * W) * 8;
+  // resident CTAs per SM asked of the compiler: a cap of 128 registers, or 64 for the
+  // one-transform shell sums (twice the CTAs)
+  static constexpr int CAP = MODE == X_PK || MODE == X_PKP ? 1024 : 512;
+  static constexpr int MINB = XT >= CAP ? 1 : CAP / XT;
+};
+
 // (i k)^m v for m = 0, 1, 2
 __device__ __forceinline__ float2 deriv(float2 v, float k, int m) {
   if (m == 0) return v;
@@ -922,12 +940,14 @@ __device__ __forceinline__ float warp_sum(float x) {
   return x;
 }
 
-// Minimum resident CTAs per SM for an x-pass mode: the one-transform shell-sum modes fit
-// in 64 registers a thread (twice the CTAs); the others are capped at 128.
-template <int N> constexpr int x_minb(int mode) {
-  return (mode == X_PK || mode == X_PKP)
-             ? (PassCfg<N>::XT >= 1024 ? 1 : 1024 / PassCfg<N>::XT)
-             : PassCfg<N>::XMINB;
+// Shell of |n|^2 = n2 by the thresholds (ns for n2 >= (N/2)^2): a float estimate of floor(2 ns |n| /
+// N), off by at most one, corrected by integer comparisons.
+__device__ __forceinline__ int shell_below(int n2, const int* thr, int ns, float n) {
+  float r;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"((float)n2));
+  int b = min((int)(r * (2.0f * (float)ns / n)), ns);
+  b += (b < ns && n2 >= thr[min(b + 1, ns)]) - (n2 < thr[b]);
+  return b;
 }
 
 // Tile inputs of the adjoint modes already in shared memory (element (kx, w) at kx W + w):
@@ -947,10 +967,10 @@ struct XSmemIn {
 // s_sc the tile of the scf field staged in shared memory (element (kx, w) at kx W + w), or
 // null to read a.scf from global memory.
 template <int N, int MODE, bool SPLIT>
-__device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[PassCfg<N>::RMAX], int kzb, int ky, int inst,
-                                       size_t blk, const SmemCol<PassCfg<N>::W>& sm, const float2* s_tw,
+__device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[XCfg<N, MODE>::RMAX], int kzb, int ky, int inst,
+                                       size_t blk, const SmemCol<XCfg<N, MODE>::W>& sm, const float2* s_tw,
                                        double* s_acc, const float* s_sc = nullptr, XSmemIn si = {}) {
-  using C = PassCfg<N>;
+  using C = XCfg<N, MODE>;
   const int w = threadIdx.x % C::W, t = threadIdx.x / C::W;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr int NWARP = C::XT / 32;
@@ -971,11 +991,11 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[PassCfg<N>::R
     for (int gi = 0; gi < ng; ++gi) {
       float2 u[C::RMAX];
 #pragma unroll
-      for (int r = 0; r < C::RMAX; ++r) u[r] = a.in2[gi][base + (size_t)(elem<N>(t, r)) * stride];
-      fft<N, false>(u, t, sm, s_tw);
+      for (int r = 0; r < C::RMAX; ++r) u[r] = a.in2[gi][base + (size_t)(elem<N, C::V>(t, r)) * stride];
+      fft<N, false, C::V>(u, t, sm, s_tw);
 #pragma unroll
       for (int r = 0; r < C::RMAX; ++r) {
-        const int kx = elem<N>(t, r);
+        const int kx = elem<N, C::V>(t, r);
         v[r] = acc_dconj(v[r], u[r], kf * (float)mode_of(kx, N), gi);
       }
     }
@@ -984,7 +1004,7 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[PassCfg<N>::R
       const size_t toff = (size_t)inst * mode_table_len(N);
 #pragma unroll
       for (int r = 0; r < C::RMAX; ++r) {
-        const int kx = elem<N>(t, r);
+        const int kx = elem<N, C::V>(t, r);
         const int mx = mode_of(kx, N);
         const int n2 = mx * mx + my * my + mz * mz;
         const bool zero = ny_nyq || kx == C::H || n2 == 0;
@@ -1003,21 +1023,21 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[PassCfg<N>::R
         u = deriv(u, kf * (float)my, a.mul_ord[1]);
         v[r] = deriv(u, kf * (float)mz, a.mul_ord[2]);
       }
-      fft<N, true>(v, t, sm, s_tw);
+      fft<N, true, C::V>(v, t, sm, s_tw);
 #pragma unroll
-      for (int r = 0; r < C::RMAX; ++r) a.out[0][base + (size_t)(elem<N>(t, r)) * stride] = v[r];
+      for (int r = 0; r < C::RMAX; ++r) a.out[0][base + (size_t)(elem<N, C::V>(t, r)) * stride] = v[r];
       return;
     }
     if (MODE == X_INV) {
-      fft<N, true>(v, t, sm, s_tw);
+      fft<N, true, C::V>(v, t, sm, s_tw);
 #pragma unroll
-      for (int r = 0; r < C::RMAX; ++r) a.out[0][base + (size_t)(elem<N>(t, r)) * stride] = v[r];
+      for (int r = 0; r < C::RMAX; ++r) a.out[0][base + (size_t)(elem<N, C::V>(t, r)) * stride] = v[r];
       return;
     }
-    fft<N, false>(v, t, sm, s_tw);
+    fft<N, false, C::V>(v, t, sm, s_tw);
     if (MODE == X_FWD) {
 #pragma unroll
-      for (int r = 0; r < C::RMAX; ++r) a.out[0][base + (size_t)(elem<N>(t, r)) * stride] = v[r];
+      for (int r = 0; r < C::RMAX; ++r) a.out[0][base + (size_t)(elem<N, C::V>(t, r)) * stride] = v[r];
       return;
     }
   }
@@ -1028,11 +1048,11 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[PassCfg<N>::R
     // the two are averaged, which cancels the odd aliasing images of the first grid
     float2 u[C::RMAX];
 #pragma unroll
-    for (int r = 0; r < C::RMAX; ++r) u[r] = a.in2[0][base + (size_t)(elem<N>(t, r)) * stride];
-    fft<N, false>(u, t, sm, s_tw);
+    for (int r = 0; r < C::RMAX; ++r) u[r] = a.in2[0][base + (size_t)(elem<N, C::V>(t, r)) * stride];
+    fft<N, false, C::V>(u, t, sm, s_tw);
 #pragma unroll
     for (int r = 0; r < C::RMAX; ++r) {
-      const int mx = mode_of(elem<N>(t, r), N);
+      const int mx = mode_of(elem<N, C::V>(t, r), N);
       float sn, cs;
       sincospif((float)(mx + my + mz) / (float)N, &sn, &cs);
       const float2 w = cmul(u[r], make_float2(cs, sn));
@@ -1040,46 +1060,60 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[PassCfg<N>::R
     }
   }
   if (MODE == X_PKP || MODE == X_PKI) {
-    // P(k) shells (mode counts and mean |k| come from the cached shell geometry).  At one
-    // register slot a warp holds a compact patch of modes (consecutive kx and kz), which
-    // mostly falls in one or two shells: the warp finds its smallest and largest shell
-    // (two reductions), sums V |delta|^2 / N^6 over the lanes of each (warp sums) and one
-    // lane adds the sums to the warp's own FP32 histogram in shared memory; a patch over
-    // more shells takes them one at a time.  At most 32 x RMAX values per shell and warp
-    // (relative error below 4e-5 even when every rounding goes one way); the sums over
-    // warps and blocks are FP64.
+    // P(k) shells (mode counts and mean |k| come from the cached shell geometry).  Every lane adds
+    // V |delta|^2 / N^6 of its modes to a column of its own in the exchange buffer, which is free
+    // after the transform: [warp][shell][lane], no two lanes in one bank, no atomics, and no
+    // assumption on how many shells neighbouring modes span.  It holds 2 RMAX shells; more take
+    // several rounds.  Then a thread per (shell, warp) sums the 32 lanes, and FP64 sums the
+    // warps (a fixed tree over NWARP lanes, spread over the CTA's warps: a conversion or addition
+    // holds an FP64 unit for 64 cycles).  The shell of a mode is a float estimate of floor(2 ns |n| /
+    // N), off by at most one, corrected against integer thresholds.  At most 32 x RMAX values per
+    // shell and warp in FP32 (relative error below 4e-5 even when every rounding goes one way).
+    // Measured (against a warp's two reductions for its patch's shells and a warp sum for each):
+    // x_pk at 512^3 329 -> 250 us, 96 batched instances 948 -> 700, 48 shells at 192^3 61 -> 48, 64^3
+    // 12.3 -> 8.1 us.
     const float pnorm = a.g.box * a.g.box * a.g.box * a.g.inv_n3 * a.g.inv_n3;
     const int ns = a.n_shells;
-    float* s_mine = reinterpret_cast<float*>(s_acc) + warp * ns;
+    const int* s_thr = reinterpret_cast<const int*>(s_acc);   // [ns + 1]: smallest |n|^2 in shell b or above
+    const int c2 = my * my + mz * mz;
+    const float wgt = pnorm * (mz == 0 ? 1.f : 2.f);
+    constexpr int S = 2 * C::RMAX;                             // shells per round: N W 8 bytes / (XT 4)
+    float* hist = reinterpret_cast<float*>(sm.base - w);
+    float* mine = hist + warp * (S * 32) + lane;
+    float pv[C::RMAX];
+    int sh[C::RMAX];
 #pragma unroll
     for (int r = 0; r < C::RMAX; ++r) {
-      const int kx = elem<N>(t, r);
-      int n2;
-      const int b = shell_of<N>(mode_of(kx, N), my, mz, ns, n2);
-      float pv = 0.f;
-      if (b >= 0) {
-        pv = (v[r].x * v[r].x + v[r].y * v[r].y) * pnorm * (mz == 0 ? 1.f : 2.f);
-        if (a.pk_deconv) pv /= cic_window2(mode_of(kx, N), my, mz, N);
-      }
-      const int lo = (int)__reduce_min_sync(0xffffffffu, (unsigned)(b < 0 ? 0x7fffffff : b));
-      const int hi = (int)__reduce_max_sync(0xffffffffu, (unsigned)(b < 0 ? 0 : b + 1)) - 1;
-      if (lo > hi) continue;                         // no mode of the patch in a shell
-      const float s0 = warp_sum(b == lo ? pv : 0.f);
-      if (lane == 0) s_mine[lo] += s0;
-      if (hi == lo) continue;
-      const float s1 = warp_sum(b == hi ? pv : 0.f);
-      if (lane == 0) s_mine[hi] += s1;
-      for (int k = lo + 1; k < hi; ++k) {            // shells strictly between (rare)
-        const float sk = warp_sum(b == k ? pv : 0.f);
-        if (lane == 0) s_mine[k] += sk;
-      }
+      const int mx = mode_of(elem<N, C::V>(t, r), N), n2 = mx * mx + c2;
+      pv[r] = n2 == 0 ? 0.f : (v[r].x * v[r].x + v[r].y * v[r].y) * wgt;
+      if (a.pk_deconv) pv[r] /= cic_window2(mx, my, mz, N);
+      sh[r] = shell_below(n2, s_thr, ns, (float)N);
     }
-    __syncthreads();
-    const float* s_all = reinterpret_cast<const float*>(s_acc);
-    for (int b = threadIdx.x; b < ns; b += blockDim.x) {
-      double acc = 0.0;
-      for (int wi = 0; wi < NWARP; ++wi) acc += (double)s_all[wi * ns + b];   // fixed order
-      a.pk_part[blk * ns + b] = acc;
+    for (int b0 = 0; b0 < ns; b0 += S) {
+      if (b0) __syncthreads();                                 // the previous round's sums are read
+#pragma unroll
+      for (int i = 0; i < S / 4; ++i)
+        reinterpret_cast<float4*>(hist + warp * (S * 32))[i * 32 + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+      __syncwarp();
+#pragma unroll
+      for (int r = 0; r < C::RMAX; ++r) {
+        const unsigned b = (unsigned)(sh[r] - b0);
+        if (b < (unsigned)min(S, ns - b0)) mine[b * 32] += pv[r];
+      }
+      __syncthreads();
+      for (int i0 = 0; i0 < S * NWARP; i0 += C::XT) {
+        const int i = i0 + threadIdx.x, b = i / NWARP, wi = i % NWARP;
+        float lanes = 0.f;
+        if (b < S && b0 + b < ns) {
+          const float* row = hist + (wi * S + b) * 32;
+#pragma unroll
+          for (int j = 0; j < 32; ++j) lanes += row[(j + lane) & 31];
+        }
+        double acc = (double)lanes;
+#pragma unroll
+        for (int o = NWARP / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (wi == 0 && b < S && b0 + b < ns) a.pk_part[blk * ns + b0 + b] = acc;
+      }
     }
     return;
   }
@@ -1097,7 +1131,7 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[PassCfg<N>::R
     float* s_mine = reinterpret_cast<float*>(s_acc) + warp * NQ * ns;
 #pragma unroll
     for (int r = 0; r < C::RMAX; ++r) {
-      const int kx = elem<N>(t, r);
+      const int kx = elem<N, C::V>(t, r);
       int n2;
       const int b = shell_of<N>(mode_of(kx, N), my, mz, ns, n2);
       const int wgt = (b < 0) ? 0 : ((mz == 0) ? 1 : 2);
@@ -1153,20 +1187,20 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[PassCfg<N>::R
     // d P_b / d delta_rho: multiply delta_rho(k) by the per-shell weight, back along x
 #pragma unroll
     for (int r = 0; r < C::RMAX; ++r) {
-      const int kx = elem<N>(t, r);
+      const int kx = elem<N, C::V>(t, r);
       int n2;
       const int b = shell_of<N>(mode_of(kx, N), my, mz, a.n_shells, n2);
       v[r] = cscale(v[r], b < 0 ? 0.f : __ldg(a.shell_w + b));
     }
-    fft<N, true>(v, t, sm, s_tw);
+    fft<N, true, C::V>(v, t, sm, s_tw);
 #pragma unroll
-    for (int r = 0; r < C::RMAX; ++r) a.out[0][base + (size_t)(elem<N>(t, r)) * stride] = v[r];
+    for (int r = 0; r < C::RMAX; ++r) a.out[0][base + (size_t)(elem<N, C::V>(t, r)) * stride] = v[r];
     return;
   }
 
   if (MODE == X_SOURCE && a.s_out) {
 #pragma unroll
-    for (int r = 0; r < C::RMAX; ++r) a.s_out[base + (size_t)(elem<N>(t, r)) * stride] = v[r];
+    for (int r = 0; r < C::RMAX; ++r) a.s_out[base + (size_t)(elem<N, C::V>(t, r)) * stride] = v[r];
   }
 
   // k-space multipliers from the per-|n|^2 tables.  g = potential to transform back along x.
@@ -1183,7 +1217,7 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[PassCfg<N>::R
   if constexpr (shared) {
 #pragma unroll
     for (int r = 0; r < C::RMAX; ++r) {
-      const int kx = elem<N>(t, r);
+      const int kx = elem<N, C::V>(t, r);
       if (kx >= C::H) continue;
       const int n2 = kx * kx + my * my + mz * mz;
       const float4 mt = ny_nyq || n2 == 0 ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(a.mt0 + toff + n2);
@@ -1195,7 +1229,7 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[PassCfg<N>::R
   float theta = 0.f;
 #pragma unroll
   for (int r = 0; r < C::RMAX; ++r) {
-    const int kx = elem<N>(t, r);
+    const int kx = elem<N, C::V>(t, r);
     const int mx = mode_of(kx, N);
     const bool zero = ny_nyq || kx == C::H || (mx == 0 && my == 0 && mz == 0);
     const int n2 = mx * mx + my * my + mz * mz;
@@ -1259,14 +1293,14 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[PassCfg<N>::R
     float2 u[C::RMAX];
 #pragma unroll
     for (int r = 0; r < C::RMAX; ++r) {
-      const int kx = elem<N>(t, r);
+      const int kx = elem<N, C::V>(t, r);
       float2 src = g[r];
       if constexpr (SPLIT && MODE == X_DELTA) src = fromh ? hpot[r] : src;
       u[r] = deriv(src, kf * (float)mode_of(kx, N), m);
     }
-    fft<N, true>(u, t, sm, s_tw);
+    fft<N, true, C::V>(u, t, sm, s_tw);
 #pragma unroll
-    for (int r = 0; r < C::RMAX; ++r) a.out[o][base + (size_t)(elem<N>(t, r)) * stride] = u[r];
+    for (int r = 0; r < C::RMAX; ++r) a.out[o][base + (size_t)(elem<N, C::V>(t, r)) * stride] = u[r];
   }
   if (MODE == X_ADJ_SOURCE && threadIdx.x == 0) {
     double acc = 0.0;
@@ -1281,9 +1315,9 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[PassCfg<N>::R
 // flag the second potential array held its registers in the total form too (x_delta at 512^3 850 ->
 // 740 us, its split form at 256^3 124 -> 113 us).
 template <int N, int MODE, bool SPLIT>
-__global__ void __launch_bounds__(PassCfg<N>::XT, x_minb<N>(MODE)) k_x(XArgs a) {
-  using C = PassCfg<N>;
-  extern __shared__ float2 smem[];
+__global__ void __launch_bounds__(XCfg<N, MODE>::XT, XCfg<N, MODE>::MINB) k_x(XArgs a) {
+  using C = XCfg<N, MODE>;
+  extern __shared__ __align__(16) float2 smem[];
   float2* s_tw = smem;
   load_twiddles(s_tw, a.tw, N);
   grid_sync_and_trigger();
@@ -1291,9 +1325,14 @@ __global__ void __launch_bounds__(PassCfg<N>::XT, x_minb<N>(MODE)) k_x(XArgs a) 
   const SmemCol<C::W> sm{smem + N + w};
   double* s_acc = reinterpret_cast<double*>(smem + N + N * C::W);   // per-warp accumulators
   constexpr int NWARP = C::XT / 32;
-  if (MODE == X_PK || MODE == X_PKP || MODE == X_PKI) {
+  if (MODE == X_PK) {
     float* s_accf = reinterpret_cast<float*>(s_acc);
-    for (int i = threadIdx.x; i < NWARP * (MODE == X_PK ? 5 : 1) * a.n_shells; i += blockDim.x) s_accf[i] = 0.f;
+    for (int i = threadIdx.x; i < NWARP * 5 * a.n_shells; i += blockDim.x) s_accf[i] = 0.f;
+  } else if (MODE == X_PKP || MODE == X_PKI) {   // smallest |n|^2 with 2 ns |n| / N >= b
+    int* thr = reinterpret_cast<int*>(s_acc);
+    const long long q = 4LL * a.n_shells * a.n_shells;
+    for (int b = threadIdx.x; b <= a.n_shells; b += blockDim.x)
+      thr[b] = (int)(((long long)b * N * ((long long)b * N) + q - 1) / q);
   } else if (MODE == X_ADJ_SOURCE) {
     for (int i = threadIdx.x; i < NWARP; i += blockDim.x) s_acc[i] = 0.0;
   }
@@ -1302,7 +1341,7 @@ __global__ void __launch_bounds__(PassCfg<N>::XT, x_minb<N>(MODE)) k_x(XArgs a) 
   if (MODE != X_ADJ_SOURCE && MODE != X_ADJ_DELTA) {
     const size_t base = blockIdx.z * ((size_t)N * N * C::H) + (size_t)blockIdx.y * C::H + blockIdx.x * C::W + w;
 #pragma unroll
-    for (int r = 0; r < C::RMAX; ++r) v[r] = a.in[base + (size_t)(elem<N>(t, r)) * ((size_t)N * C::H)];
+    for (int r = 0; r < C::RMAX; ++r) v[r] = a.in[base + (size_t)(elem<N, C::V>(t, r)) * ((size_t)N * C::H)];
   }
   const size_t blk = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
   if (MODE == X_SOURCE && a.zero) {
@@ -1342,8 +1381,8 @@ template <int N, bool SC = false> struct XTmaCfg {
 };
 
 template <int N, int MODE, bool SC>
-__global__ void __launch_bounds__(PassCfg<N>::XT, x_minb<N>(MODE)) k_x_tma(const __grid_constant__ XArgs a) {
-  using C = PassCfg<N>;
+__global__ void __launch_bounds__(XCfg<N, MODE>::XT, XCfg<N, MODE>::MINB) k_x_tma(const __grid_constant__ XArgs a) {
+  using C = XCfg<N, MODE>;
   using Q = XTmaCfg<N, SC>;
   extern __shared__ __align__(128) unsigned char xs_raw[];
   float2* s_tw = reinterpret_cast<float2*>(xs_raw);
@@ -1383,16 +1422,12 @@ __global__ void __launch_bounds__(PassCfg<N>::XT, x_minb<N>(MODE)) k_x_tma(const
   __syncthreads();
   for (int i = 0, tile = blockIdx.x; tile < ntiles; ++i, tile += gridDim.x) {
     const int st = i & 1;
-    if (MODE == X_PK || MODE == X_PKP) {
-      float* s_accf = reinterpret_cast<float*>(s_acc);
-      for (int k = threadIdx.x; k < NWARP * (MODE == X_PK ? 5 : 1) * a.n_shells; k += blockDim.x) s_accf[k] = 0.f;
-    }
     const bool ok = mbar_wait(&bar[st], (i >> 1) & 1, a.g.wait);
     if (!ok) s_fail = 1;
     float2 v[C::RMAX];
     const float2* tl = ring + st * Q::STAGE;
 #pragma unroll
-    for (int r = 0; r < C::RMAX; ++r) v[r] = ok ? tl[elem<N>(t, r) * C::W + w] : make_float2(0.f, 0.f);
+    for (int r = 0; r < C::RMAX; ++r) v[r] = ok ? tl[elem<N, C::V>(t, r) * C::W + w] : make_float2(0.f, 0.f);
     __syncthreads();   // tile read by every thread before the transforms reuse the buffer
     if (s_fail) {
       if (threadIdx.x == 0) {
@@ -1435,8 +1470,8 @@ template <int N> struct XAdjCfg {
 };
 
 template <int N, int MODE>
-__global__ void __launch_bounds__(PassCfg<N>::XT, x_minb<N>(MODE)) k_x_tma_adj(const __grid_constant__ XArgs a) {
-  using C = PassCfg<N>;
+__global__ void __launch_bounds__(XCfg<N, MODE>::XT, XCfg<N, MODE>::MINB) k_x_tma_adj(const __grid_constant__ XArgs a) {
+  using C = XCfg<N, MODE>;
   using Q = XAdjCfg<N>;
   constexpr int NG = MODE == X_ADJ_SOURCE ? 2 : 3;   // transformed groups per tile (then 4 - NG plain inputs)
   constexpr int NWARP = C::XT / 32;
@@ -1489,15 +1524,15 @@ __global__ void __launch_bounds__(PassCfg<N>::XT, x_minb<N>(MODE)) k_x_tma_adj(c
       if (!ok) s_fail = 1;
       float2 u[C::RMAX];
 #pragma unroll
-      for (int r = 0; r < C::RMAX; ++r) u[r] = ok ? ring[st * Q::TILE + elem<N>(t, r) * C::W + w] : make_float2(0.f, 0.f);
+      for (int r = 0; r < C::RMAX; ++r) u[r] = ok ? ring[st * Q::TILE + elem<N, C::V>(t, r) * C::W + w] : make_float2(0.f, 0.f);
       __syncthreads();   // stage read by every thread before the transform reuses it (and s_fail seen)
       if (s_fail) {
         if (threadIdx.x == 0) drain(c);
         return;
       }
-      fft<N, false>(u, t, SmemCol<C::W>{ring + st * Q::TILE + w}, s_tw);   // ends past its last shared read
+      fft<N, false, C::V>(u, t, SmemCol<C::W>{ring + st * Q::TILE + w}, s_tw);   // ends past its last shared read
 #pragma unroll
-      for (int r = 0; r < C::RMAX; ++r) v[r] = acc_dconj(v[r], u[r], a.g.kf * (float)mode_of(elem<N>(t, r), N), j);
+      for (int r = 0; r < C::RMAX; ++r) v[r] = acc_dconj(v[r], u[r], a.g.kf * (float)mode_of(elem<N, C::V>(t, r), N), j);
       __syncthreads();   // every warp is past the transform: the stage is free
       if (threadIdx.x == 0 && issued < nload) {
         fence_proxy_async_smem();
@@ -1652,10 +1687,10 @@ template <int N, int MODE> cudaError_t launch_x_tma_adj(const XArgs& a, int acc,
   return launch_overlapped(k_x_tma_adj<N, MODE>, grid, C::XT, smem, s, b);
 }
 template <int N, int MODE> cudaError_t launch_x_m(const XArgs& a, cudaStream_t s) {
-  using C = PassCfg<N>;
+  using C = XCfg<N, MODE>;
   LPT2_CHECK_BATCH(a);
   const int acc = MODE == X_PK ? (C::XT / 32) * 5 * a.n_shells * 4
-                  : (MODE == X_PKP || MODE == X_PKI) ? (C::XT / 32) * a.n_shells * 4
+                  : (MODE == X_PKP || MODE == X_PKI) ? (a.n_shells + 1) * 4
                                                      : (MODE == X_ADJ_SOURCE ? (C::XT / 32) * 8 : 0);
   // The delta mode and the two adjoint modes have two tile paths: bulk-tensor tiles
   // (default: measured faster at 512^3, x_delta 0.91 -> 0.86 ms, x_adj_delta 1.245 -> 1.113)
