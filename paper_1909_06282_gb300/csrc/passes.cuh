@@ -958,6 +958,10 @@ struct XSmemIn {
   const float2* hpsi = nullptr;
   const float2* delta = nullptr;
   const float2* s = nullptr;
+  float4* table = nullptr;   // X_ADJ_SOURCE: N W / 2 entries of scratch for the shared table gathers
+};
+struct XNothing {
+  __device__ __forceinline__ void operator()() const {}
 };
 
 // One x-pass tile: kz block kzb (W consecutive kz), fixed ky, instance inst, all kx.
@@ -966,10 +970,13 @@ struct XSmemIn {
 // s_acc the per-warp accumulators (zeroed by the caller), blk the tile's linear index,
 // s_sc the tile of the scf field staged in shared memory (element (kx, w) at kx W + w), or
 // null to read a.scf from global memory.
-template <int N, int MODE, bool SPLIT>
+// after_mult() runs between the multiplier and the inverse transforms, after a barrier (modes
+// that have one there): every thread has read its shared-memory inputs and the table.
+template <int N, int MODE, bool SPLIT, class F = XNothing>
 __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[XCfg<N, MODE>::RMAX], int kzb, int ky, int inst,
                                        size_t blk, const SmemCol<XCfg<N, MODE>::W>& sm, const float2* s_tw,
-                                       double* s_acc, const float* s_sc = nullptr, XSmemIn si = {}) {
+                                       double* s_acc, const float* s_sc = nullptr, XSmemIn si = {},
+                                       F after_mult = F()) {
   using C = XCfg<N, MODE>;
   const int w = threadIdx.x % C::W, t = threadIdx.x / C::W;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1209,21 +1216,29 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[XCfg<N, MODE>
   // staged with the tile) and the second is computed.
   const size_t toff = (size_t)inst * mode_table_len(N);
   constexpr bool field = (MODE == X_DELTA && !SPLIT) || MODE == X_ADJ_DELTA;
-  // X_SOURCE: kx and N - kx have the same |n|^2, so the thread that holds kx < N/2 gathers its
-  // entry and hands D1 / (k^2 N^3), D2 / (k^2 N^3) to the one that holds N - kx through the
-  // exchange buffer (free between the transforms): half the gathers, whose 32 scattered entries
-  // per warp take an L1 cycle each (512^3 777 -> 726 us, split form at 256^3 84 -> 70 us).
-  constexpr bool shared = MODE == X_SOURCE;
+  // Source modes: kx and N - kx have the same |n|^2, so the thread that holds kx < N/2 gathers its
+  // entries and hands the products D1, D2 (and the tangents) over k^2 N^3 to the one that
+  // holds N - kx, through the exchange buffer (free between the transforms) or the caller's
+  // scratch: half the gathers, whose 32 scattered entries per warp take an L1 cycle each (512^3:
+  // x_source 777 -> 726 us, its split form at 256^3 84 -> 70 us, x_adj_source 1319 -> 1029 us with the earlier refill of its ring).
+  constexpr bool shared = MODE == X_SOURCE || MODE == X_ADJ_SOURCE;
+  float4* table = MODE == X_ADJ_SOURCE ? (si.table ? si.table : reinterpret_cast<float4*>(sm.base - w)) + w : nullptr;
   if constexpr (shared) {
 #pragma unroll
     for (int r = 0; r < C::RMAX; ++r) {
       const int kx = elem<N, C::V>(t, r);
       if (kx >= C::H) continue;
       const int n2 = kx * kx + my * my + mz * mz;
-      const float4 mt = ny_nyq || n2 == 0 ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(a.mt0 + toff + n2);
-      sm.st(kx, make_float2(mt.z * mt.y, mt.w * mt.y));
+      const bool none = ny_nyq || n2 == 0;
+      const float4 mt = none ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(a.mt0 + toff + n2);
+      if (MODE == X_SOURCE) {
+        sm.st(kx, make_float2(mt.z * mt.y, mt.w * mt.y));
+      } else {
+        const float2 tt = none ? make_float2(0.f, 0.f) : __ldg(a.mt1 + toff + n2);
+        table[kx * C::W] = make_float4(mt.z * mt.y, mt.w * mt.y, tt.x * mt.y, tt.y * mt.y);
+      }
     }
-    sm.sync();
+    __syncthreads();
   }
   float2 g[C::RMAX], hpot[SPLIT && MODE == X_DELTA ? C::RMAX : 1];
   float theta = 0.f;
@@ -1261,15 +1276,15 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[XCfg<N, MODE>
       g[r] = u;
     } else if (MODE == X_ADJ_SOURCE) {                    // v = g_u(k)
       const float2 gu = zero ? make_float2(0.f, 0.f) : v[r];
-      a.hpsi_out[e] = cscale(gu, d1 * inv);                 // h_Psi = D1 g_u / (k^2 N^3)
-      g[r] = cscale(gu, -d2 * inv);                         // h_S = -D2 g_u / (k^2 N^3)
+      const float4 m = kx == C::H ? make_float4(0.f, 0.f, 0.f, 0.f) : table[(kx < C::H ? kx : N - kx) * C::W];
+      a.hpsi_out[e] = cscale(gu, m.x);                      // h_Psi = D1 g_u / (k^2 N^3)
+      g[r] = cscale(gu, -m.y);                              // h_S = -D2 g_u / (k^2 N^3)
       if (!zero) {                                          // dL/dln|fR0| contribution
-        const float2 tt = __ldg(a.mt1 + toff + n2);
         const float2 dl = si.delta ? si.delta[kx * C::W + w] : a.delta_in[e];
         const float2 sk = si.s ? si.s[kx * C::W + w] : a.s_in[e];
-        const float cx = __fmaf_rn(tt.x, dl.x, -__fmul_rn(tt.y, sk.x));
-        const float cy = __fmaf_rn(tt.x, dl.y, -__fmul_rn(tt.y, sk.y));
-        theta = __fmaf_rn(__fmul_rn(__fmaf_rn(cx, gu.x, __fmul_rn(cy, gu.y)), inv), mz == 0 ? 1.f : 2.f, theta);
+        const float cx = __fmaf_rn(m.z, dl.x, -__fmul_rn(m.w, sk.x));
+        const float cy = __fmaf_rn(m.z, dl.y, -__fmul_rn(m.w, sk.y));
+        theta = __fmaf_rn(__fmaf_rn(cx, gu.x, __fmul_rn(cy, gu.y)), mz == 0 ? 1.f : 2.f, theta);
       }
     } else {                                                // X_ADJ_DELTA: v = sum of h_phi groups
       const float2 hp = si.hpsi ? si.hpsi[kx * C::W + w] : a.hpsi_in[e];
@@ -1285,6 +1300,7 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[XCfg<N, MODE>
   // x-inverse transforms with x-derivative orders (the exchange buffer may hold the
   // shared-memory inputs read above: every thread has read its own first)
   if (si.summed || shared) __syncthreads();
+  after_mult();
   constexpr int nout = MODE == X_DELTA ? (SPLIT ? 5 : 3) : (MODE == X_SOURCE ? 2 : 1);
 #pragma unroll 1
   for (int o = 0; o < nout; ++o) {
@@ -1534,6 +1550,7 @@ __global__ void __launch_bounds__(XCfg<N, MODE>::XT, XCfg<N, MODE>::MINB) k_x_tm
 #pragma unroll
       for (int r = 0; r < C::RMAX; ++r) v[r] = acc_dconj(v[r], u[r], a.g.kf * (float)mode_of(elem<N, C::V>(t, r), N), j);
       __syncthreads();   // every warp is past the transform: the stage is free
+      if (MODE == X_ADJ_SOURCE && j == NG - 1) continue;   // (it holds the multiplier table first)
       if (threadIdx.x == 0 && issued < nload) {
         fence_proxy_async_smem();
         issue();
@@ -1557,13 +1574,22 @@ __global__ void __launch_bounds__(XCfg<N, MODE>::XT, XCfg<N, MODE>::MINB) k_x_tm
     } else {
       si.delta = ring + s0 * Q::TILE;
       si.s = ring + s1 * Q::TILE;
+      si.table = reinterpret_cast<float4*>(ring + ((c + 2) % 3) * Q::TILE);   // the last group's stage
       ex = ring + s1 * Q::TILE;
     }
-    x_tile<N, MODE, false>(a, v, kzb, ky, inst, (size_t)tile, SmemCol<C::W>{ex + w}, s_tw, s_acc, nullptr, si);
+    // X_ADJ_SOURCE: the table's and delta(k)'s stages take the next inputs while the inverse
+    // transform runs
+    auto refill = [&]() {
+      if (MODE == X_ADJ_SOURCE && threadIdx.x == 0) {
+        fence_proxy_async_smem();
+        for (int j = 0; j < 2 && issued < nload; ++j) issue();
+      }
+    };
+    x_tile<N, MODE, false>(a, v, kzb, ky, inst, (size_t)tile, SmemCol<C::W>{ex + w}, s_tw, s_acc, nullptr, si, refill);
     __syncthreads();   // stages and accumulators free
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && issued < nload) {
       fence_proxy_async_smem();
-      for (int j = 0; j < 4 - NG && issued < nload; ++j) issue();
+      issue();
     }
     c += 4 - NG;
   }
