@@ -186,6 +186,18 @@ template <bool WARP = false> struct SmemRowT {
 using SmemRow = SmemRowT<false>;
 // z-pass pencils of N points lie in one warp when N / RMAX <= 32 threads hold one
 template <int N> inline constexpr bool kRowWarp = (N / Cfg<N>::RMAX) <= 32;
+// The same row for a group of GT threads that runs on its own: a warp, or GT / 32 warps that meet
+// at the CTA's named barrier `bar`.
+template <int GT> struct SmemRowG {
+  float2* base;
+  int bar;
+  __device__ __forceinline__ void st(int n, float2 v) const { base[n + (n >> 4)] = v; }
+  __device__ __forceinline__ float2 ld(int n) const { return base[n + (n >> 4)]; }
+  __device__ __forceinline__ void sync() const {
+    if constexpr (GT == 32) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(GT) : "memory");
+  }
+};
 // Column layout: W pencils interleaved, element (n, w) at n * W + w (a pencil spans warps).
 template <int W> struct SmemCol {
   float2* base;   // already offset by w

@@ -277,15 +277,26 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_c2r(ZC2RArgs 
   }
 }
 
-// Six phi_ij -> S = sum_{i<j} (phi_ii phi_jj - phi_ij^2)  (Eq. second-ini) -> forward z.
+// z passes over several fields (z_source, z_final, z_adj_source).  The rows of one field are
+// contiguous in the half-spectrum layout, so a tile of rows is one bulk copy per field into a
+// ring of two shared-memory stages: the copy of field f + 2 is in flight while field f is
+// transformed.  Rows 2p and 2p + 1 of a field are packed as one complex pencil (Z = A + i B),
+// so its inverse transform gives the field on both rows.  Two forms:
 //
-// A CTA owns ROWS = 2 ZP consecutive real rows (x, y) of every field.  The rows of
-// one field are contiguous in the half-spectrum layout, so each field's tile is one
-// bulk copy into a ring of STAGES shared-memory buffers: the copy of field f +
-// STAGES is in flight while field f is transformed.  Rows 2p and 2p + 1 of a field
-// are packed as one complex pencil (Z = A + i B), so its inverse transform gives the
-// field on both rows; the source term accumulates per row in registers:
-//   S = phi_xx phi_yy + (phi_xx + phi_yy) phi_zz - phi_xy^2 - phi_xz^2 - phi_yz^2.
+// CTA form (ZSrcCfg): a CTA owns 2 ZP rows and a ring, and meets at a barrier per field.
+//
+// Group form (ZGrp): a group of threads (a warp; two warps at N = 1024, where a pencil has 64
+// threads) owns ROWS rows at a time and a ring of its own, is persistent (group g takes tiles
+// g, g + G, ...) and synchronises with nobody: while one group waits for a copy or an exchange
+// the others issue, and the next tile's first copies fly during this one's last transforms.
+//
+// Which: warps that run apart fetch different instructions, so the group form pays where its
+// code is short.  The total form of z_final (one transform body) at every N: 512^3 622 -> 516
+// us, 256^3 82 -> 72, 96 batched instances 1605 -> 1307.  The others (several bodies) up to N =
+// 192, where a pencil's transform is short: z_source 2859 -> 2435 us (the 96 instances), split
+// z_final at 128^3 31.1 -> 26.6, z_adj_source at 128^3 52 -> 47; from N = 256 on the CTA form:
+// z_source 123 against 141 us at 256^3 and 1096 against 1416 at 512^3 (where the loop state also
+// spills), split z_final 156 against 171 at 256^3, z_adj_source 261 against 272.
 #ifndef LPT2_ZS_STAGES
 #define LPT2_ZS_STAGES 2
 #endif
@@ -302,6 +313,91 @@ template <int N> struct ZSrcCfg {
   static_assert(STAGE_BYTES % 16 == 0 && (C::H * 8) % 16 == 0, "bulk copies need 16-byte multiples");
 };
 
+template <int N> constexpr bool zgroups() { return N <= 192; }   // group form for several bodies
+template <int N> struct ZGrp {
+  using C = PassCfg<N>;
+  static constexpr int GT = C::TPP > 32 ? C::TPP : 32;       // threads of a group
+  static constexpr int PP = GT / C::TPP;                     // pencils (row pairs) of a group
+  static constexpr int GROUPS = C::ZT / GT;
+  static constexpr int ROWS = 2 * PP;
+  static constexpr int STAGE_F2 = ROWS * C::H;               // one field's tile (float2)
+  static constexpr unsigned STAGE_BYTES = STAGE_F2 * 8u;
+  static constexpr int RING_OFF = N, ROW_OFF = RING_OFF + GROUPS * 2 * STAGE_F2;   // float2 offsets
+  static constexpr int BAR_OFF = (ROW_OFF + C::ZP * SmemRow::words(N)) * 8;        // bytes
+  static constexpr int SMEM = BAR_OFF + GROUPS * 16;
+  static constexpr int TILES = N * N / ROWS;                                       // per instance
+  static_assert(STAGE_BYTES % 16 == 0 && BAR_OFF % 8 == 0 && RING_OFF % 2 == 0, "bulk copies need 16-byte alignment");
+  static_assert(C::ZT % GT == 0 && GROUPS < 15 && (N * N) % ROWS == 0, "groups must tile the CTA and the rows");
+};
+
+// The copy ring of one group: NF copies per tile, in the order the kernel consumes them; src(f,
+// tile) gives the address of copy f of a tile (tiles run over the instances of the batch: their
+// rows are consecutive).  Two copies are in flight or in use; state is kept to two registers.
+template <int N, int NF, class Src> struct ZRing {
+  using Q = ZGrp<N>;
+  Src src;
+  float2* ring;   // the group's two stages
+  uint64_t* bar;
+  int tiles;      // of the batch
+  int tile = 0;   // the group's current tile
+  int used = 0;   // copies consumed so far
+  __device__ __forceinline__ bool lead() const { return threadIdx.x % Q::GT == 0; }
+  __device__ __forceinline__ int step() const { return gridDim.x * Q::GROUPS; }
+  // copy f (< 2 NF) counted from the current tile's first, into stage st
+  __device__ __forceinline__ bool exists(int f) const { return tile + (f >= NF ? step() : 0) < tiles; }
+  __device__ __forceinline__ void issue(int f, int st) const {
+    mbar_expect_tx(&bar[st], Q::STAGE_BYTES);
+    bulk_load(ring + st * Q::STAGE_F2, src(f >= NF ? f - NF : f, tile + (f >= NF ? step() : 0)), Q::STAGE_BYTES, &bar[st]);
+  }
+  __device__ __forceinline__ void start(int first) {
+    tile = first;
+    if (lead() && tile < tiles) {
+      issue(0, 0);
+      issue(1, 1);
+    }
+  }
+  // waits for copy f of the current tile; its stage, or null (after the group drained and reported)
+  template <class SM>
+  __device__ __forceinline__ const float2* next(int f, const SM& sm, int* s_fail, int* err, int code, long long wait) const {
+    const bool ok = mbar_wait(&bar[used & 1], (used >> 1) & 1, wait);
+    bool bad;
+    if constexpr (Q::GT == 32) {
+      bad = __any_sync(0xffffffffu, !ok);
+    } else {
+      if (!ok) *s_fail = 1;
+      sm.sync();
+      bad = *s_fail != 0;
+    }
+    if (bad) {
+      if (lead()) {
+        for (int i = 0; i < 2; ++i)
+          if (exists(f + i)) mbar_wait(&bar[(used + i) & 1], ((used + i) >> 1) & 1);
+        report_device_error(err, code);
+      }
+      return nullptr;
+    }
+    return ring + (used & 1) * Q::STAGE_F2;
+  }
+  // every thread of the group has read copy f: its stage takes copy f + 2
+  template <class SM> __device__ __forceinline__ void release(int f, const SM& sm) {
+    sm.sync();
+    if (lead() && exists(f + 2)) issue(f + 2, used & 1);
+    ++used;
+  }
+};
+template <int N, int NF, class Src>
+__device__ __forceinline__ ZRing<N, NF, Src> make_zring(Src src, unsigned char* raw, int group, int batch) {
+  using Q = ZGrp<N>;
+  ZRing<N, NF, Src> r{src, reinterpret_cast<float2*>(raw) + Q::RING_OFF + group * 2 * Q::STAGE_F2,
+                      reinterpret_cast<uint64_t*>(raw + Q::BAR_OFF) + 2 * group, Q::TILES * batch};
+  if (r.lead()) {
+    mbar_init(&r.bar[0], 1);
+    mbar_init(&r.bar[1], 1);
+    mbar_init_fence();
+  }
+  return r;
+}
+
 // Z value at element n of the Hermitian extension of half rows ra, rb (shared
 // memory), both multiplied by (i k_z)^m first: Z = A + i B.
 template <int N>
@@ -317,8 +413,77 @@ __device__ __forceinline__ float2 z_assemble_smem(const float2* ra, const float2
   return make_float2(A.x - B.y, A.y + B.x);
 }
 
+// Six phi_ij -> S = sum_{i<j} (phi_ii phi_jj - phi_ij^2)  (Eq. second-ini) -> forward z.  The
+// source term accumulates per row in registers:
+//   S = phi_xx phi_yy + (phi_xx + phi_yy) phi_zz - phi_xy^2 - phi_xz^2 - phi_yz^2.
 template <int N>
 __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_source(ZSourceArgs a) {
+  using C = PassCfg<N>;
+  using Q = ZGrp<N>;
+  extern __shared__ __align__(128) unsigned char zs_raw[];
+  float2* s_tw = reinterpret_cast<float2*>(zs_raw);
+  __shared__ int s_fail[Q::GROUPS];
+  const int group = threadIdx.x / Q::GT, p = threadIdx.x / C::TPP, pl = p % Q::PP, t = threadIdx.x % C::TPP;
+  const SmemRowG<Q::GT> sm{s_tw + Q::ROW_OFF + p * SmemRow::words(N), 1 + group};
+  auto src = [&](int f, int tile) { return a.in[f] + (size_t)tile * Q::STAGE_F2; };
+  auto ring = make_zring<N, 6>(src, zs_raw, group, a.g.batch);
+  if (threadIdx.x < Q::GROUPS) s_fail[threadIdx.x] = 0;
+  load_twiddles(s_tw, a.tw, N);
+  grid_sync_and_trigger();
+  __syncthreads();
+  ring.start(blockIdx.x * Q::GROUPS + group);
+  // the ring's next field into v; false if the wait ran out (the group must return)
+  auto fetch = [&](int f, float2 (&v)[C::RMAX]) -> bool {
+    const float2* st = ring.next(f, sm, &s_fail[group], a.g.err, LPT2_DEV_ETIMEOUT_ZSOURCE, a.g.wait);
+    if (!st) return false;
+    const float2* ra = st + 2 * pl * C::H;
+    const int m = a.ord[f];
+#pragma unroll
+    for (int r = 0; r < C::RMAX; ++r) v[r] = z_assemble_smem<N>(ra, ra + C::H, elem<N>(t, r), a.g.kf, m);
+    ring.release(f, sm);
+    return true;
+  };
+  for (; ring.tile < ring.tiles; ring.tile += ring.step()) {
+    float S0[C::RMAX], S1[C::RMAX], T0[C::RMAX], T1[C::RMAX];
+#pragma unroll
+    for (int r = 0; r < C::RMAX; ++r) S0[r] = S1[r] = T0[r] = T1[r] = 0.f;
+#pragma unroll 1
+    for (int f = 0; f < 3; ++f) {   // phi_xx, phi_yy, phi_zz: S += T phi, T += phi on rows 2p and 2p + 1
+      float2 v[C::RMAX];
+      if (!fetch(f, v)) return;
+      fft<N, true>(v, t, sm, s_tw);
+#pragma unroll
+      for (int r = 0; r < C::RMAX; ++r) {
+        S0[r] = fmaf(T0[r], v[r].x, S0[r]);
+        S1[r] = fmaf(T1[r], v[r].y, S1[r]);
+        T0[r] += v[r].x;
+        T1[r] += v[r].y;
+      }
+    }
+#pragma unroll 1
+    for (int f = 3; f < 6; ++f) {   // phi_xy, phi_xz, phi_yz
+      float2 v[C::RMAX];
+      if (!fetch(f, v)) return;
+      fft<N, true>(v, t, sm, s_tw);
+#pragma unroll
+      for (int r = 0; r < C::RMAX; ++r) {
+        S0[r] = fmaf(-v[r].x, v[r].x, S0[r]);
+        S1[r] = fmaf(-v[r].y, v[r].y, S1[r]);
+      }
+    }
+    float2 v[C::RMAX];
+#pragma unroll
+    for (int r = 0; r < C::RMAX; ++r) v[r] = make_float2(S0[r], S1[r]);
+    fft<N, false>(v, t, sm, s_tw);
+    float2* out = a.out + (size_t)ring.tile * Q::STAGE_F2 + 2 * pl * C::H;
+    z_store_pair<N>(v, t, sm, out, out + C::H);
+    sm.sync();   // the row's reads are done before the next tile's transforms reuse it
+  }
+}
+
+// The same in CTA form.
+template <int N>
+__global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_source_cta(ZSourceArgs a) {
   using C = PassCfg<N>;
   using Q = ZSrcCfg<N>;
   extern __shared__ __align__(128) unsigned char zs_raw[];
@@ -456,17 +621,90 @@ __device__ __forceinline__ float wrapN(float u) {
 }
 
 // Psi inputs (z order 1 -> Psi_z, 0 -> Psi_y, 0 -> Psi_x) -> particle positions
-// x = q + Psi (Eq. position), periodic.  The tile and copy ring are those of
-// k_z_source: a CTA owns ROWS consecutive rows of every input, one bulk copy per
-// input tile, rows 2p and 2p + 1 of a field packed as one complex pencil.  The
-// three components are independent, so nothing is carried from one input to the
-// next except, when SPLIT (separate Psi1 / Psi2 inputs), the Psi1 part of the
-// current component.
+// x = q + Psi (Eq. position), periodic.  The three components are independent, so nothing is
+// carried from one input to the next except, when SPLIT (separate Psi1 / Psi2 inputs), the
+// Psi1 part of the current component.
 template <int N, bool SPLIT>
 __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_final(ZFinalArgs a) {
   using C = PassCfg<N>;
-  using Q = ZSrcCfg<N>;
+  using Q = ZGrp<N>;
   constexpr int NQ = SPLIT ? 6 : 3;   // input tiles: (Psi1, Psi2) per component, or the totals
+  extern __shared__ __align__(128) unsigned char zs_raw[];
+  float2* s_tw = reinterpret_cast<float2*>(zs_raw);
+  __shared__ int s_fail[Q::GROUPS];
+  const int group = threadIdx.x / Q::GT, p = threadIdx.x / C::TPP, pl = p % Q::PP, t = threadIdx.x % C::TPP;
+  const SmemRowG<Q::GT> sm{s_tw + Q::ROW_OFF + p * SmemRow::words(N), 1 + group};
+  constexpr size_t n3 = (size_t)N * N * N;
+  auto src = [&](int q, int tile) {
+    return (SPLIT ? ((q & 1) ? a.b[q >> 1] : a.a[q >> 1]) : a.a[q]) + (size_t)tile * Q::STAGE_F2;
+  };
+  auto ring = make_zring<N, NQ>(src, zs_raw, group, a.g.batch);
+  if (threadIdx.x < Q::GROUPS) s_fail[threadIdx.x] = 0;
+  load_twiddles(s_tw, a.tw, N);
+  grid_sync_and_trigger();
+  __syncthreads();
+  ring.start(blockIdx.x * Q::GROUPS + group);
+  for (; ring.tile < ring.tiles; ring.tile += ring.step()) {
+    const size_t inst = (size_t)(ring.tile / Q::TILES);
+    const int row = (ring.tile % Q::TILES) * Q::ROWS + 2 * pl;       // rows `row`, `row` + 1
+    float2 keep[C::RMAX];
+#pragma unroll 1
+    for (int q = 0; q < NQ; ++q) {
+      const int c = SPLIT ? (q >> 1) : q;   // 0: Psi_z, 1: Psi_y, 2: Psi_x
+      const float2* st = ring.next(q, sm, &s_fail[group], a.g.err, LPT2_DEV_ETIMEOUT_ZFINAL, a.g.wait);
+      if (!st) return;
+      float2 v[C::RMAX];
+      const float2* ra = st + 2 * pl * C::H;
+#pragma unroll
+      for (int r = 0; r < C::RMAX; ++r)
+        v[r] = z_assemble_smem<N>(ra, ra + C::H, elem<N>(t, r), a.g.kf, c == 0 ? 1 : 0);
+      ring.release(q, sm);
+      fft<N, true>(v, t, sm, s_tw);
+      const int d = 2 - c;                  // output component: x 0, y 1, z 2
+      if (SPLIT) {
+        float* outp = (q & 1) ? a.psi2 : a.psi1;
+        if (outp) {
+          outp += 3 * inst * n3 + d * n3;
+#pragma unroll
+          for (int r = 0; r < C::RMAX; ++r) {
+            const int iz = elem<N>(t, r);
+            outp[(size_t)row * N + iz] = v[r].x;
+            outp[(size_t)(row + 1) * N + iz] = v[r].y;
+          }
+        }
+        if (!(q & 1)) {
+#pragma unroll
+          for (int r = 0; r < C::RMAX; ++r) keep[r] = v[r];
+          continue;
+        }
+#pragma unroll
+        for (int r = 0; r < C::RMAX; ++r) v[r] = cadd(v[r], keep[r]);
+      }
+      if (a.pos) {
+        float* pos = a.pos + 3 * inst * n3 + d * n3;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int R = row + h;
+          const float q0 = (d == 0) ? (float)(R / N) : (float)(R % N);   // Lagrangian x or y
+#pragma unroll
+          for (int r = 0; r < C::RMAX; ++r) {
+            const int iz = elem<N>(t, r);
+            const float psi = h ? v[r].y : v[r].x;
+            const float u = wrapN<N>((d == 2 ? (float)iz : q0) + psi * a.g.inv_cell);
+            pos[(size_t)R * N + iz] = u * a.g.cell;
+          }
+        }
+      }
+    }
+  }
+}
+
+// The split form with CTAs.
+template <int N>
+__global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_split_cta(ZFinalArgs a) {
+  using C = PassCfg<N>;
+  using Q = ZSrcCfg<N>;
+  constexpr int NQ = 6;   // input tiles: (Psi1, Psi2) per component
   extern __shared__ __align__(128) unsigned char zs_raw[];
   float2* ring = reinterpret_cast<float2*>(zs_raw);
   uint64_t* bar = reinterpret_cast<uint64_t*>(zs_raw + Q::BAR_OFF);
@@ -479,7 +717,7 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_final(ZFinalA
   const size_t tile = (size_t)blockIdx.x * Q::STAGE_F2;
   const int row = blockIdx.x * Q::ROWS + 2 * p;                    // rows `row`, `row` + 1
   auto input = [&](int q) -> const float2* {
-    return (SPLIT ? ((q & 1) ? a.b[q >> 1] : a.a[q >> 1]) : a.a[q]) + zs + tile;
+    return ((q & 1) ? a.b[q >> 1] : a.a[q >> 1]) + zs + tile;
   };
   if (threadIdx.x == 0) {
     s_fail = 0;
@@ -499,7 +737,7 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_final(ZFinalA
 #pragma unroll 1
   for (int q = 0; q < NQ; ++q) {
     const int st = q % Q::STAGES;
-    const int c = SPLIT ? (q >> 1) : q;   // 0: Psi_z, 1: Psi_y, 2: Psi_x
+    const int c = q >> 1;   // 0: Psi_z, 1: Psi_y, 2: Psi_x
     const bool ok = mbar_wait(&bar[st], (q / Q::STAGES) & 1, a.g.wait);
     if (!ok) s_fail = 1;
     float2 v[C::RMAX];
@@ -521,25 +759,23 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_final(ZFinalA
     }
     fft<N, true>(v, t, sm, s_tw);
     const int d = 2 - c;                  // output component: x 0, y 1, z 2
-    if (SPLIT) {
-      float* outp = (q & 1) ? a.psi2 : a.psi1;
-      if (outp) {
-        outp += 3 * zr + d * n3;
+    float* outp = (q & 1) ? a.psi2 : a.psi1;
+    if (outp) {
+      outp += 3 * zr + d * n3;
 #pragma unroll
-        for (int r = 0; r < C::RMAX; ++r) {
-          const int iz = elem<N>(t, r);
-          outp[(size_t)row * N + iz] = v[r].x;
-          outp[(size_t)(row + 1) * N + iz] = v[r].y;
-        }
+      for (int r = 0; r < C::RMAX; ++r) {
+        const int iz = elem<N>(t, r);
+        outp[(size_t)row * N + iz] = v[r].x;
+        outp[(size_t)(row + 1) * N + iz] = v[r].y;
       }
-      if (!(q & 1)) {
-#pragma unroll
-        for (int r = 0; r < C::RMAX; ++r) keep[r] = v[r];
-        continue;
-      }
-#pragma unroll
-      for (int r = 0; r < C::RMAX; ++r) v[r] = cadd(v[r], keep[r]);
     }
+    if (!(q & 1)) {
+#pragma unroll
+      for (int r = 0; r < C::RMAX; ++r) keep[r] = v[r];
+      continue;
+    }
+#pragma unroll
+    for (int r = 0; r < C::RMAX; ++r) v[r] = cadd(v[r], keep[r]);
     if (a.pos) {
       float* pos = a.pos + 3 * zr + d * n3;
 #pragma unroll
@@ -593,13 +829,81 @@ __device__ __forceinline__ void cic_gather_grad(const float* __restrict__ g, con
 }
 
 // Transpose of k_z_source.  g_S = dL/dS is given in real space (the inverse z of h_S,
-// one z_c2r pass); the six phi_ij are recomputed (inverse z) and
+// one z_c2r pass); the six phi_ij are transformed again (inverse z) and
 //   dL/dphi_ii = g_S (Tr - phi_ii),  Tr = phi_xx + phi_yy + phi_zz,   dL/dphi_ij = -2 g_S phi_ij,
-// each transformed forward with conj z-derivatives.  Tiles and copy ring as k_z_source
-// (rows 2p, 2p + 1 of one field per complex pencil); the diagonal fields are read twice,
+// each transformed forward with conj z-derivatives.  The diagonal fields are read twice,
 // first for Tr (kept in registers for both rows), then for their cotangents.
 template <int N>
 __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_adj_source(ZAdjSourceArgs a) {
+  using C = PassCfg<N>;
+  using Q = ZGrp<N>;
+  constexpr int NQ = 9;                         // xx, yy, zz (trace), then xx .. yz (cotangents)
+  extern __shared__ __align__(128) unsigned char zs_raw[];
+  float2* s_tw = reinterpret_cast<float2*>(zs_raw);
+  __shared__ int s_fail[Q::GROUPS];
+  const int group = threadIdx.x / Q::GT, p = threadIdx.x / C::TPP, pl = p % Q::PP, t = threadIdx.x % C::TPP;
+  const SmemRowG<Q::GT> sm{s_tw + Q::ROW_OFF + p * SmemRow::words(N), 1 + group};
+  const float kf = a.g.kf;
+  auto field = [](int q) { return q < 3 ? q : q - 3; };
+  auto src = [&](int q, int tile) { return a.in[field(q)] + (size_t)tile * Q::STAGE_F2; };
+  auto ring = make_zring<N, NQ>(src, zs_raw, group, a.g.batch);
+  if (threadIdx.x < Q::GROUPS) s_fail[threadIdx.x] = 0;
+  load_twiddles(s_tw, a.tw, N);
+  grid_sync_and_trigger();
+  __syncthreads();
+  ring.start(blockIdx.x * Q::GROUPS + group);
+  // the ring's next input into v (with the field's z-derivative order); false if the wait ran out
+  auto fetch = [&](int q, float2 (&v)[C::RMAX]) -> bool {
+    const float2* st = ring.next(q, sm, &s_fail[group], a.g.err, LPT2_DEV_ETIMEOUT_ZADJSOURCE, a.g.wait);
+    if (!st) return false;
+    const float2* ra = st + 2 * pl * C::H;
+    const int m = a.ord[field(q)];
+#pragma unroll
+    for (int r = 0; r < C::RMAX; ++r) v[r] = z_assemble_smem<N>(ra, ra + C::H, elem<N>(t, r), kf, m);
+    ring.release(q, sm);
+    return true;
+  };
+  for (; ring.tile < ring.tiles; ring.tile += ring.step()) {
+    // trace of the Hessian for both rows (fields xx, yy, zz)
+    float T0[C::RMAX], T1[C::RMAX];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      float2 v[C::RMAX];
+      if (!fetch(q, v)) return;
+      fft<N, true>(v, t, sm, s_tw);
+#pragma unroll
+      for (int r = 0; r < C::RMAX; ++r) {
+        T0[r] = q == 0 ? v[r].x : T0[r] + v[r].x;
+        T1[r] = q == 0 ? v[r].y : T1[r] + v[r].y;
+      }
+    }
+    // the six cotangents: one loop body (not unrolled: nine copies of the two transforms
+    // overflow the instruction cache)
+    const float* g0 = a.gs + 2 * ((size_t)ring.tile * Q::STAGE_F2 + 2 * pl * C::H);   // real row of the same tile
+#pragma unroll 1
+    for (int q = 3; q < NQ; ++q) {
+      float2 v[C::RMAX];
+      if (!fetch(q, v)) return;
+      const int f = q - 3;
+      fft<N, true>(v, t, sm, s_tw);
+#pragma unroll
+      for (int r = 0; r < C::RMAX; ++r) {
+        const int iz = elem<N>(t, r);
+        const float ga = __ldg(g0 + iz), gb = __ldg(g0 + N + iz);
+        v[r] = f < 3 ? make_float2(ga * (T0[r] - v[r].x), gb * (T1[r] - v[r].y))
+                     : make_float2(-2.f * ga * v[r].x, -2.f * gb * v[r].y);
+      }
+      fft<N, false>(v, t, sm, s_tw);
+      float2* out = a.out[f] + (size_t)ring.tile * Q::STAGE_F2 + 2 * pl * C::H;
+      z_store_pair_d<N>(v, t, sm, out, out + C::H, kf, a.ord[f], a.ord[f]);
+      sm.sync();   // the row's reads above are done before the next transform reuses it
+    }
+  }
+}
+
+// The same in CTA form.
+template <int N>
+__global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_adj_source_cta(ZAdjSourceArgs a) {
   using C = PassCfg<N>;
   using Q = ZSrcCfg<N>;
   constexpr int NQ = 9;                         // xx, yy, zz (trace), then xx .. yz (cotangents)
@@ -1621,32 +1925,51 @@ template <int N> cudaError_t launch_z_c2r_t(const ZC2RArgs& a, cudaStream_t s) {
   cudaFuncSetAttribute(k_z_c2r<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::ZSMEM);
   return launch_overlapped(k_z_c2r<N>, dim3(N * N / 2 / C::ZP, 1, a.g.batch), C::ZT, C::ZSMEM, s, a);
 }
-template <int N> cudaError_t launch_z_source_t(const ZSourceArgs& a, cudaStream_t s) {
-  using C = PassCfg<N>;
+// persistent grid: as many CTAs as fit on the GPU at once, or one per `per_cta` units of work
+template <class K>
+cudaError_t persistent_grid(K k, int threads, int smem, long long units, int per_cta, int* grid) {
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  int dev = 0, sms = 0, per_sm = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem)) != cudaSuccess) return e;
+  *grid = (int)std::min<long long>((units + per_cta - 1) / per_cta, (long long)sms * std::max(per_sm, 1));
+  return cudaSuccess;
+}
+template <int N, class K, class A> cudaError_t launch_zgrp(K k, const A& a, cudaStream_t s) {
+  using Q = ZGrp<N>;
   LPT2_CHECK_BATCH(a);
+  int grid = 0;
+  const cudaError_t e = persistent_grid(k, PassCfg<N>::ZT, Q::SMEM, Q::TILES * a.g.batch, Q::GROUPS, &grid);
+  return e != cudaSuccess ? e : launch_overlapped(k, grid, PassCfg<N>::ZT, Q::SMEM, s, a);
+}
+template <int N, class K, class A> cudaError_t launch_zcta(K k, const A& a, cudaStream_t s) {
   using Q = ZSrcCfg<N>;
-  cudaFuncSetAttribute(k_z_source<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, Q::SMEM);
-  return launch_overlapped(k_z_source<N>, dim3(N * N / Q::ROWS, 1, a.g.batch), C::ZT, Q::SMEM, s, a);
+  LPT2_CHECK_BATCH(a);
+  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Q::SMEM);
+  return launch_overlapped(k, dim3(N * N / Q::ROWS, 1, a.g.batch), PassCfg<N>::ZT, Q::SMEM, s, a);
+}
+template <int N> cudaError_t launch_z_source_t(const ZSourceArgs& a, cudaStream_t s) {
+  if constexpr (zgroups<N>()) return launch_zgrp<N>(k_z_source<N>, a, s);
+  else return launch_zcta<N>(k_z_source_cta<N>, a, s);
 }
 template <int N> cudaError_t launch_z_final_t(const ZFinalArgs& a, cudaStream_t s) {
-  using C = PassCfg<N>;
-  LPT2_CHECK_BATCH(a);
-  using Q = ZSrcCfg<N>;
-  auto k = a.split ? k_z_final<N, true> : k_z_final<N, false>;
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Q::SMEM);
-  return launch_overlapped(k, dim3(N * N / Q::ROWS, 1, a.g.batch), C::ZT, Q::SMEM, s, a);
+  if (!a.split) return launch_zgrp<N>(k_z_final<N, false>, a, s);
+  if constexpr (zgroups<N>()) return launch_zgrp<N>(k_z_final<N, true>, a, s);
+  else return launch_zcta<N>(k_z_split_cta<N>, a, s);
 }
 template <int N> cudaError_t launch_z_adj_source_t(const ZAdjSourceArgs& a, cudaStream_t s) {
-  using C = PassCfg<N>;
-  using Q = ZSrcCfg<N>;
-  LPT2_CHECK_BATCH(a);
   if constexpr (zadj_field_pairs<N>()) {
     using F = ZAdjFpCfg<N>;
+    LPT2_CHECK_BATCH(a);
     cudaFuncSetAttribute(k_z_adj_source_fp<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, F::SMEM);
     return launch_overlapped(k_z_adj_source_fp<N>, dim3(N * N / F::ROWS, 1, a.g.batch), F::THREADS, F::SMEM, s, a);
+  } else if constexpr (zgroups<N>()) {
+    return launch_zgrp<N>(k_z_adj_source<N>, a, s);
+  } else {
+    return launch_zcta<N>(k_z_adj_source_cta<N>, a, s);
   }
-  cudaFuncSetAttribute(k_z_adj_source<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, Q::SMEM);
-  return launch_overlapped(k_z_adj_source<N>, dim3(N * N / Q::ROWS, 1, a.g.batch), C::ZT, Q::SMEM, s, a);
 }
 template <int N, int KIND, int WYA> cudaError_t launch_y_k(const YArgs& a, cudaStream_t s) {
   constexpr int WY = WYA == YCfg<N, KIND>::W ? 0 : WYA;   // the default by its number: one instance
@@ -1678,15 +2001,9 @@ template <int N, int MODE, bool SC> cudaError_t launch_x_tma(const XArgs& a, int
   if (!encode_x_tile_map(&b.tmap, a.in, N, N, 2 * C::W, a.g.batch)) return cudaErrorInvalidValue;
   if (SC && !encode_x_tile_map(&b.tmap_sc, a.scf, N / 2, N, C::W, a.g.batch)) return cudaErrorInvalidValue;
   const int smem = Q::ACC_OFF + acc;
-  cudaError_t e = cudaFuncSetAttribute(k_x_tma<N, MODE, SC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  int grid = 0;
+  const cudaError_t e = persistent_grid(k_x_tma<N, MODE, SC>, C::XT, smem, (long long)Q::KZB * N * a.g.batch, 1, &grid);
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0, per_sm = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_x_tma<N, MODE, SC>, C::XT, smem)) != cudaSuccess)
-    return e;
-  const long long tiles = (long long)Q::KZB * N * a.g.batch;
-  const int grid = (int)std::min<long long>(tiles, (long long)sms * std::max(per_sm, 1));
   return launch_overlapped(k_x_tma<N, MODE, SC>, grid, C::XT, smem, s, b);
 }
 #ifndef LPT2_X_TMA_ADJ
@@ -1701,15 +2018,9 @@ template <int N, int MODE> cudaError_t launch_x_tma_adj(const XArgs& a, int acc,
   for (int j = 0; j < 4; ++j)
     if (!src[j] || !encode_x_tile_map(&b.tmap_l[j], src[j], N, N, 2 * C::W, a.g.batch)) return cudaErrorInvalidValue;
   const int smem = Q::ACC_OFF + acc;
-  cudaError_t e = cudaFuncSetAttribute(k_x_tma_adj<N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  int grid = 0;
+  const cudaError_t e = persistent_grid(k_x_tma_adj<N, MODE>, C::XT, smem, (long long)Q::KZB * N * a.g.batch, 1, &grid);
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0, per_sm = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_x_tma_adj<N, MODE>, C::XT, smem)) != cudaSuccess)
-    return e;
-  const long long tiles = (long long)Q::KZB * N * a.g.batch;
-  const int grid = (int)std::min<long long>(tiles, (long long)sms * std::max(per_sm, 1));
   return launch_overlapped(k_x_tma_adj<N, MODE>, grid, C::XT, smem, s, b);
 }
 template <int N, int MODE> cudaError_t launch_x_m(const XArgs& a, cudaStream_t s) {
