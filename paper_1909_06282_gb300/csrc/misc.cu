@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(CIC_THREADS, LPT2_CIC_MINB) k_cic(CicArgs a) {
   const int x0 = (b / (NT * NT)) * CIC_T, y0 = ((b / NT) % NT) * CIC_T, z0 = (b % NT) * CIC_T;
   const int ox = x0 - CIC_H, oy = y0 - CIC_H, oz = z0 - CIC_HZ;   // window origin (may be < 0)
   const bool wraps = ox < 0 || oy < 0 || oz < 0 || ox + CIC_E > N || oy + CIC_E > N || oz + CIC_EZ > N;
-  grid_sync_and_trigger();
+  grid_sync();
   // all position loads of this thread first: their latency overlaps the zeroing
   float u[CIC_PER][3];
 #pragma unroll
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(CIC_THREADS, LPT2_CIC_MINB) k_cic_grad(CicGrad
   const int x0 = (b / (NT * NT)) * CIC_T, y0 = ((b / NT) % NT) * CIC_T, z0 = (b % NT) * CIC_T;
   const int ox = x0 - CIC_H, oy = y0 - CIC_H, oz = z0 - CIC_HZ;
   const bool wraps = ox < 0 || oy < 0 || oz < 0 || ox + CIC_E > N || oy + CIC_E > N || oz + CIC_EZ > N;
-  grid_sync_and_trigger();
+  grid_sync();
   float u[CIC_PER][3];
 #pragma unroll
   for (int k = 0; k < CIC_PER; ++k) {
@@ -267,7 +267,7 @@ cudaError_t launch_cic(const CicArgs& a, cudaStream_t s) {
 }
 
 __global__ void k_fill0(float4* p, size_t n4) {
-  grid_sync_and_trigger();
+  grid_sync();
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x)
     p[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
@@ -388,7 +388,7 @@ cudaError_t launch_shell_geometry(int n, double box, int n_shells, double* ksum,
 // rows of scratch per shell (a warp per shell: strided lane sums, then a fixed shuffle
 // tree) and divides by the shell's mode count.
 __global__ void k_pk_rows(const double* __restrict__ part, int n_blocks, int ns, int rows, double* __restrict__ scratch) {
-  grid_sync_and_trigger();
+  grid_sync();
   const int g = blockIdx.x, inst = blockIdx.y;
   part += (size_t)inst * n_blocks * ns;
   const int L = blockDim.x / ns, lane = threadIdx.x / ns, b = threadIdx.x % ns;
@@ -410,7 +410,7 @@ __global__ void k_pk_rows(const double* __restrict__ part, int n_blocks, int ns,
 
 __global__ void k_pk_finalize_p(const double* __restrict__ scratch, int G, int ns, const double* ksum,
                                 const unsigned long long* count, double* pk, double* kmean, int64_t* nmodes) {
-  grid_sync_and_trigger();
+  grid_sync();
   const int inst = blockIdx.x, lane = threadIdx.x & 31;
   // a warp per shell: lane l sums rows l, l + 32, ... in order, then a fixed shuffle tree
   for (int b = threadIdx.x >> 5; b < ns; b += blockDim.x >> 5) {
@@ -573,7 +573,7 @@ cudaError_t launch_philox_words(uint32_t k0, uint32_t k1, uint64_t first, int64_
 // so the density cotangent gains IDFT[w_b delta(k)] with w_b = 2 V g_pk[b] / (N^6 c_b).
 __global__ void k_pk_adj_weights(const double* g_pk, const int64_t* n_modes, int ns, double v_over_n6,
                                  float* w) {
-  grid_sync_and_trigger();
+  grid_sync();
   for (int b = threadIdx.x; b < ns; b += blockDim.x) {
     const double c = (double)n_modes[b];
     w[b] = (c > 0 && g_pk) ? (float)(2.0 * v_over_n6 * g_pk[b] / c) : 0.f;
@@ -587,7 +587,7 @@ cudaError_t launch_pk_adj_weights(const double* g_pk, const int64_t* n_modes, in
 
 // Deterministic sum of n FP64 partials (fixed-order strided sums, then a tree).
 __global__ void k_sum_partials(const double* part, int n, double* out) {
-  grid_sync_and_trigger();
+  grid_sync();
   double acc = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) acc += part[i];
   __shared__ double s[256];

@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, SRC == Z_NOISE ? LPT2_ZNOISE_M
     bm_load_table(s_bm, a.bm);
     __syncthreads();
   }
-  if (SRC != Z_NOISE) grid_sync_and_trigger();
+  if (SRC != Z_NOISE) grid_sync();
   const int p = threadIdx.x / C::TPP, t = threadIdx.x % C::TPP;
   const SmemRowT<kRowWarp<N>> sm{smem + N + p * SmemRow::words(N)};
   const int pair = blockIdx.x * C::ZP + p;
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, SRC == Z_NOISE ? LPT2_ZNOISE_M
       v[r] = make_float2(fa, fb);
     }
   }
-  if (SRC == Z_NOISE) grid_sync_and_trigger();   // the draws need nothing of the earlier kernels
+  if (SRC == Z_NOISE) grid_sync();   // the draws need nothing of the earlier kernels
   __syncthreads();   // twiddles visible
   fft<N, false>(v, t, sm, s_tw);
   z_store_pair<N>(v, t, sm, a.out + (size_t)rowa * C::H, a.out + (size_t)rowb * C::H);
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_c2r(ZC2RArgs 
   extern __shared__ float2 smem[];
   float2* s_tw = smem;
   load_twiddles(s_tw, a.tw, N);
-  grid_sync_and_trigger();
+  grid_sync();
   const int p = threadIdx.x / C::TPP, t = threadIdx.x % C::TPP;
   const SmemRowT<kRowWarp<N>> sm{smem + N + p * SmemRow::words(N)};
   const int pair = blockIdx.x * C::ZP + p;
@@ -429,7 +429,7 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_source(ZSourc
   auto ring = make_zring<N, 6>(src, zs_raw, group, a.g.batch);
   if (threadIdx.x < Q::GROUPS) s_fail[threadIdx.x] = 0;
   load_twiddles(s_tw, a.tw, N);
-  grid_sync_and_trigger();
+  grid_sync();
   __syncthreads();
   ring.start(blockIdx.x * Q::GROUPS + group);
   // the ring's next field into v; false if the wait ran out (the group must return)
@@ -501,7 +501,7 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_source_cta(ZS
     mbar_init_fence();
   }
   load_twiddles(s_tw, a.tw, N);
-  grid_sync_and_trigger();
+  grid_sync();
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int f = 0; f < Q::STAGES; ++f) {
@@ -641,7 +641,7 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_final(ZFinalA
   auto ring = make_zring<N, NQ>(src, zs_raw, group, a.g.batch);
   if (threadIdx.x < Q::GROUPS) s_fail[threadIdx.x] = 0;
   load_twiddles(s_tw, a.tw, N);
-  grid_sync_and_trigger();
+  grid_sync();
   __syncthreads();
   ring.start(blockIdx.x * Q::GROUPS + group);
   for (; ring.tile < ring.tiles; ring.tile += ring.step()) {
@@ -725,7 +725,7 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_split_cta(ZFi
     mbar_init_fence();
   }
   load_twiddles(s_tw, a.tw, N);
-  grid_sync_and_trigger();
+  grid_sync();
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int q = 0; q < Q::STAGES && q < NQ; ++q) {
@@ -849,7 +849,7 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_adj_source(ZA
   auto ring = make_zring<N, NQ>(src, zs_raw, group, a.g.batch);
   if (threadIdx.x < Q::GROUPS) s_fail[threadIdx.x] = 0;
   load_twiddles(s_tw, a.tw, N);
-  grid_sync_and_trigger();
+  grid_sync();
   __syncthreads();
   ring.start(blockIdx.x * Q::GROUPS + group);
   // the ring's next input into v (with the field's z-derivative order); false if the wait ran out
@@ -926,7 +926,7 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_adj_source_ct
     mbar_init_fence();
   }
   load_twiddles(s_tw, a.tw, N);
-  grid_sync_and_trigger();
+  grid_sync();
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int q = 0; q < Q::STAGES; ++q) {
@@ -1062,7 +1062,7 @@ __global__ void __launch_bounds__(ZAdjFpCfg<N>::THREADS, 2) k_z_adj_source_fp(ZA
   }
   const float* gsr = a.gs + zr + row * N;   // g_S of this row (read where used: registers are short)
   load_twiddles(s_tw, a.tw, N);
-  grid_sync_and_trigger();
+  grid_sync();
   if (threadIdx.x == 0) {
     issue(0);
     issue(1);
@@ -1150,7 +1150,7 @@ __global__ void __launch_bounds__(YCfg<N, KIND, WY>::XT, YCfg<N, KIND, WY>::MINB
   extern __shared__ float2 smem[];
   float2* s_tw = smem;
   load_twiddles(s_tw, a.tw, N);
-  grid_sync_and_trigger();
+  grid_sync();
   const int w = threadIdx.x % C::W, t = threadIdx.x / C::W;
   const SmemCol<C::W> sm{smem + N + w};
   const int kz = blockIdx.x * C::W + w;
@@ -1640,7 +1640,7 @@ __global__ void __launch_bounds__(XCfg<N, MODE>::XT, XCfg<N, MODE>::MINB) k_x(XA
   extern __shared__ __align__(16) float2 smem[];
   float2* s_tw = smem;
   load_twiddles(s_tw, a.tw, N);
-  grid_sync_and_trigger();
+  grid_sync();
   const int w = threadIdx.x % C::W, t = threadIdx.x / C::W;
   const SmemCol<C::W> sm{smem + N + w};
   double* s_acc = reinterpret_cast<double*>(smem + N + N * C::W);   // per-warp accumulators
@@ -1734,7 +1734,7 @@ __global__ void __launch_bounds__(XCfg<N, MODE>::XT, XCfg<N, MODE>::MINB) k_x_tm
     mbar_init_fence();
   }
   load_twiddles(s_tw, a.tw, N);
-  grid_sync_and_trigger();
+  grid_sync();
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i)
       if (blockIdx.x + i * gridDim.x < ntiles) issue(i, blockIdx.x + i * gridDim.x);
@@ -1826,7 +1826,7 @@ __global__ void __launch_bounds__(XCfg<N, MODE>::XT, XCfg<N, MODE>::MINB) k_x_tm
     mbar_init_fence();
   }
   load_twiddles(s_tw, a.tw, N);
-  grid_sync_and_trigger();
+  grid_sync();
   if (threadIdx.x == 0)
     while (issued < 3 && issued < nload) issue();
   __syncthreads();

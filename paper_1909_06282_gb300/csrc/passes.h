@@ -9,8 +9,8 @@
 
 namespace lpt2 {
 
-// Launches a kernel that calls grid_sync_and_trigger(): it may start while the stream's
-// previous kernel drains, up to that call (programmatic dependent launch).
+// Launches a kernel that calls grid_sync(): its launch and the part before that call overlap the
+// end of the stream's previous kernel (programmatic dependent launch).
 template <class... P, class... A>
 cudaError_t launch_overlapped(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A&... args) {
   cudaLaunchConfig_t cfg = {};

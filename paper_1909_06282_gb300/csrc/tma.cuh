@@ -16,15 +16,14 @@ namespace lpt2 {
 #endif
 
 // Start of a kernel launched with launch_overlapped (passes.h): waits until the stream's earlier
-// kernels have completed and their writes are visible, then lets the next kernel's CTAs start
-// where this one's leave room.  Before it a kernel touches only shared memory and tables that
-// the plan wrote once (twiddles): whatever starts here has all but its direct predecessor
-// behind it, because that one has passed its own wait.  At 64^3 the launches of a step are
-// 1.5-2 us apart without it.
-__device__ __forceinline__ void grid_sync_and_trigger() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
+// kernels have completed and their writes are visible.  Before it a kernel touches only shared
+// memory and tables that the plan wrote once (twiddles, Box-Muller).  No kernel signals its
+// dependents early (griddepcontrol.launch_dependents): the next kernel's CTAs then start when the
+// last of this one's have exited, which hides the launch and the set-up (64^3 102 -> 78 us a
+// step).  Signalling at the start costs more than it hides: CTAs that start on an SM still
+// running the previous kernel keep its split of L1 and shared memory, and a pass that loads
+// through L1 then runs beside the 206 KB of a z pass (512^3 step 7.16 -> 8.43 ms).
+__device__ __forceinline__ void grid_sync() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
