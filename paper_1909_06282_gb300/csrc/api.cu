@@ -1820,38 +1820,29 @@ int lpt2_displace_vjp(lpt2_plan_t p, const float* noise, const float* g_pos, con
   // The forward map, keeping delta(k) (slot 1), S(k), positions and the CIC density, unless
   // the last lpt2_displace of a LPT2_KEEP_STATE plan left them for this noise; then the
   // delta_rho spectrum after the z and y passes, unless a later lpt2_cic_pk left it in slot A.
+  // With a cotangent of the positions alone (g_density and g_pk null) nothing flows back through
+  // the density: neither the forward's particles and deposit nor the passes that carry the
+  // density cotangent are run (at 512^3 0.73 + 0.46 + 0.52 + 1.03 ms of forward passes for one x
+  // pass of 0.19, and 3.7 ms of adjoint passes whose results were zeros added to g_pos).
+  const bool via_density = g_density || g_pk || !g_pos;
   const bool reuse = p->keep_state && p->kept_fwd && p->kept_noise == noise;
   const bool reuse_spec = reuse && p->kept_spec;
   drop_state(p);   // this call overwrites the kept slots
-  if (!reuse) {
+  if (!reuse && via_density) {
     rc = displace_impl(p, noise, nullptr, nullptr, nullptr, nullptr, S[S_SHAT], pos);
     if (rc) return rc;
-  }
-  if (!reuse_spec) {
-    rc = forward_zy(p, Z_DENSITY, rho, S[S_A]);
+  } else if (!reuse) {   // delta(k), the phi_ij and S(k)
+    const FwdSlots f = fwd_slots(p);
+    rc = displace_prefix(p, f, noise, false);
     if (rc) return rc;
+    XArgs xf{};
+    xf.g = g;
+    xf.tw = p->tw;
+    xf.mode = X_FWD;
+    xf.in = f.A;
+    xf.out[0] = S[S_SHAT];
+    LAUNCH(p, "x_fwd", 8.0 * V3(p), x_pass(n, xf, p->stream));
   }
-  // the P(k) transpose needs the mode count per shell (cached geometry), not P(k) itself
-  rc = ensure_geometry(p, 0, n_shells);
-  if (rc) return rc;
-  static_assert(sizeof(unsigned long long) == sizeof(int64_t), "mode counts are 64-bit");
-  const int64_t* nmodes = reinterpret_cast<const int64_t*>(p->groups[0].geo_n);
-  XArgs xp{};
-  xp.g = g;
-  xp.tw = p->tw;
-  xp.in = S[S_A];
-  xp.cosmo = p->cosmo_dev;
-  xp.pk_part = pk_part(p);
-  xp.n_shells = n_shells;
-
-  // 1. density cotangent: g_density + IDFT[w_b delta_rho(k)]
-  const double v_over_n6 = p->box * p->box * p->box / (V3d * V3d);
-  LAUNCH(p, "pk_adj_w", 0.0, launch_pk_adj_weights(g_pk, nmodes, n_shells, v_over_n6, shw, p->stream));
-  XArgs xa = xp;
-  xa.mode = X_PKADJ;
-  xa.shell_w = shw;
-  xa.out[0] = S[S_A];
-  LAUNCH(p, "x_pkadj", 8.0 * V3(p), x_pass(n, xa, p->stream));
   YArgs yi{};
   yi.g = g;
   yi.tw = p->tw;
@@ -1860,17 +1851,51 @@ int lpt2_displace_vjp(lpt2_plan_t p, const float* noise, const float* g_pos, con
   yi.job.n_out = 1;
   yi.job.in[0] = S[S_A];
   yi.job.out[0] = S[S_A];
-  LAUNCH(p, "y_inv", 8.0 * V3(p), y_pass(n, yi, p->stream));
-  float* grho = reinterpret_cast<float*>(S[2]);
-  ZC2RArgs zc{g, p->tw, S[S_A], grho, g_density};
-  LAUNCH(p, "z_c2r_grho", (g_density ? 12.0 : 8.0) * V3(p), z_c2r(n, zc, p->stream));
+  const float* gps[3];   // g_Psi: x, y, z
+  if (via_density) {
+    // 1. density cotangent: g_density + IDFT[w_b delta_rho(k)]; without g_pk it is g_density itself
+    // (the gather reads groups of four, so a pointer that is not 16-byte aligned takes the copy
+    // that the transform pass makes)
+    const float* grho = g_density;
+    if (g_pk || !g_density || !aligned(g_density, 16)) {
+      if (!reuse_spec) {
+        rc = forward_zy(p, Z_DENSITY, rho, S[S_A]);
+        if (rc) return rc;
+      }
+      // the P(k) transpose needs the mode count per shell (cached geometry), not P(k) itself
+      rc = ensure_geometry(p, 0, n_shells);
+      if (rc) return rc;
+      static_assert(sizeof(unsigned long long) == sizeof(int64_t), "mode counts are 64-bit");
+      const int64_t* nmodes = reinterpret_cast<const int64_t*>(p->groups[0].geo_n);
+      const double v_over_n6 = p->box * p->box * p->box / (V3d * V3d);
+      LAUNCH(p, "pk_adj_w", 0.0, launch_pk_adj_weights(g_pk, nmodes, n_shells, v_over_n6, shw, p->stream));
+      XArgs xa{};
+      xa.g = g;
+      xa.tw = p->tw;
+      xa.mode = X_PKADJ;
+      xa.in = S[S_A];
+      xa.out[0] = S[S_A];
+      xa.cosmo = p->cosmo_dev;
+      xa.n_shells = n_shells;
+      xa.shell_w = shw;
+      LAUNCH(p, "x_pkadj", 8.0 * V3(p), x_pass(n, xa, p->stream));
+      LAUNCH(p, "y_inv", 8.0 * V3(p), y_pass(n, yi, p->stream));
+      float* gr = reinterpret_cast<float*>(S[2]);
+      ZC2RArgs zc{g, p->tw, S[S_A], gr, g_density};
+      LAUNCH(p, "z_c2r_grho", (g_density ? 12.0 : 8.0) * V3(p), z_c2r(n, zc, p->stream));
+      grho = gr;
+    }
 
-  // 2-3. CIC transpose (tiled gather) into real g_Psi fields (slots 10-12), then their
-  // forward z transforms: slots 7 (z; its conj(i k_z) is applied in the y pass), 8 (y), 9 (x)
-  float* gps[3] = {reinterpret_cast<float*>(S[12]), reinterpret_cast<float*>(S[11]),
-                   reinterpret_cast<float*>(S[10])};   // x, y, z
-  CicGradArgs cg{g, grho, pos, g_pos, gps[0], gps[1], gps[2]};
-  LAUNCH(p, "cic_grad", (g_pos ? 40.0 : 28.0) * V3(p), launch_cic_grad(cg, p->stream));
+    // 2. CIC transpose (tiled gather) into real g_Psi fields (slots 10-12)
+    float* const gs3[3] = {reinterpret_cast<float*>(S[12]), reinterpret_cast<float*>(S[11]), reinterpret_cast<float*>(S[10])};
+    CicGradArgs cg{g, grho, pos, g_pos, gs3[0], gs3[1], gs3[2]};
+    LAUNCH(p, "cic_grad", (g_pos ? 40.0 : 28.0) * V3(p), launch_cic_grad(cg, p->stream));
+    for (int c = 0; c < 3; ++c) gps[c] = gs3[c];
+  } else {
+    for (int c = 0; c < 3; ++c) gps[c] = g_pos + c * (size_t)n * n * n;
+  }
+  // 3. forward z transforms of g_Psi: slots 7 (z; its conj(i k_z) is applied in the y pass), 8
+  // (y), 9 (x)
   ZR2CArgs zp{};
   zp.g = g;
   zp.tw = p->tw;
