@@ -380,13 +380,12 @@ cudaError_t launch_shell_geometry(int n, double box, int n_shells, double* ksum,
   return cudaGetLastError();
 }
 
-// Shell sums of the per-block P partials in two fixed-order stages (the result does not
-// depend on scheduling).  Stage 1: CTA (g, instance) takes rows [g R, g R + R) of the
-// partials; thread (lane, b) = (tid / ns, tid % ns) sums rows lane, lane + L, ... of shell b
-// (L = 256 / ns lanes; a warp reads consecutive shells of a row, i.e. contiguous doubles),
-// then the lanes are summed in order into scratch[instance][g][b].  Stage 2 sums the G
-// rows of scratch per shell (a warp per shell: strided lane sums, then a fixed shuffle
-// tree) and divides by the shell's mode count.
+// Shell sums of the per-block P partials in fixed order (the result does not depend on
+// scheduling).  An FP64 addition holds its unit for 64 cycles a warp, so many rows are first
+// summed by up to 128 CTAs: CTA (g, instance) takes rows [g R, g R + R) of the partials; thread
+// (lane, b) = (tid / ns, tid % ns) sums rows lane, lane + L, ... of shell b (L = 256 / ns lanes; a
+// warp reads consecutive shells of a row, i.e. contiguous doubles), then the lanes are summed in
+// order into scratch[instance][g][b].
 __global__ void k_pk_rows(const double* __restrict__ part, int n_blocks, int ns, int rows, double* __restrict__ scratch) {
   grid_sync();
   const int g = blockIdx.x, inst = blockIdx.y;
@@ -407,23 +406,33 @@ __global__ void k_pk_rows(const double* __restrict__ part, int n_blocks, int ns,
     scratch[((size_t)inst * gridDim.x + g) * ns + threadIdx.x] = sum;
   }
 }
-
-__global__ void k_pk_finalize_p(const double* __restrict__ scratch, int G, int ns, const double* ksum,
-                                const unsigned long long* count, double* pk, double* kmean, int64_t* nmodes) {
+// P(k) of an instance from n_rows rows of sums: as k_pk_rows over all rows, the lanes summed by a
+// fixed tree, divided by the shell's mode count.
+constexpr int kPkThreads = 1024;
+__global__ void __launch_bounds__(kPkThreads) k_pk_finalize_p(const double* __restrict__ sums, int n_rows, int ns,
+                                                              const double* ksum, const unsigned long long* count,
+                                                              double* pk, double* kmean, int64_t* nmodes) {
+  __shared__ double sh[kPkThreads];
   grid_sync();
-  const int inst = blockIdx.x, lane = threadIdx.x & 31;
-  // a warp per shell: lane l sums rows l, l + 32, ... in order, then a fixed shuffle tree
-  for (int b = threadIdx.x >> 5; b < ns; b += blockDim.x >> 5) {
-    double sp = 0.0;
-    for (int g = lane; g < G; g += 32) sp += scratch[((size_t)inst * G + g) * ns + b];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sp += __shfl_xor_sync(0xffffffffu, sp, o);
-    if (lane == 0) {
-      const double c = (double)count[b];
-      pk[(size_t)inst * ns + b] = c > 0 ? sp / c : 0.0;
-      if (kmean) kmean[(size_t)inst * ns + b] = c > 0 ? ksum[b] / c : 0.0;
-      if (nmodes) nmodes[(size_t)inst * ns + b] = (int64_t)count[b];
-    }
+  const int inst = blockIdx.x, L = kPkThreads / ns, lane = threadIdx.x / ns, b = threadIdx.x % ns;
+  sums += (size_t)inst * n_rows * ns;
+  double acc = 0.0;
+  if (lane < L) {
+#pragma unroll 4
+    for (int r = lane; r < n_rows; r += L) acc += sums[(size_t)r * ns + b];
+  }
+  sh[threadIdx.x] = acc;
+  for (int n = L; n > 1;) {
+    const int h = (n + 1) / 2;
+    __syncthreads();
+    if (lane + h < n) sh[threadIdx.x] += sh[threadIdx.x + h * ns];
+    n = h;
+  }
+  if (lane == 0) {
+    const double c = (double)count[b];
+    pk[(size_t)inst * ns + b] = c > 0 ? sh[b] / c : 0.0;
+    if (kmean) kmean[(size_t)inst * ns + b] = c > 0 ? ksum[b] / c : 0.0;
+    if (nmodes) nmodes[(size_t)inst * ns + b] = (int64_t)count[b];
   }
 }
 
@@ -431,14 +440,21 @@ cudaError_t launch_pk_finalize_p(const double* part, int n_blocks, int n_shells,
                                  const unsigned long long* count, double* pk, double* k_mean, int64_t* n_modes,
                                  cudaStream_t s, int batch) {
   if (n_shells < 1 || n_shells > 256 || n_blocks < 1 || batch < 1 || batch > 65535) return cudaErrorInvalidValue;
-  // the stage-1 sums follow the partials in their buffer (sized for three quantities per
-  // row and shell, of which P uses one): batch * G * n_shells <= batch * n_blocks * n_shells
-  const int G = n_blocks < 128 ? n_blocks : 128;
-  const int rows = (n_blocks + G - 1) / G;
-  double* scratch = const_cast<double*>(part) + (size_t)batch * n_blocks * n_shells;
-  const cudaError_t e = launch_overlapped(k_pk_rows, dim3(G, batch), 256, 0, s, part, n_blocks, n_shells, rows, scratch);
-  if (e != cudaSuccess) return e;
-  return launch_overlapped(k_pk_finalize_p, batch, 256, 0, s, scratch, G, n_shells, ksum, count, pk, k_mean, n_modes);
+  // One CTA adds 8192 partials in 2 us (4096 warp-lanes a microsecond), less than a second
+  // launch costs: five output times at 128^3 469 -> 454 us, the
+  // interlaced estimator at 192^3 278 -> 269, 64 batched 32^3 grids 113 -> 109.
+  if (pk_finalize_launches(n_blocks, n_shells) == 2) {
+    // the stage-1 sums follow the partials in their buffer (sized for three quantities per
+    // row and shell, of which P uses one): batch * G * n_shells <= batch * n_blocks * n_shells
+    const int G = n_blocks < 128 ? n_blocks : 128;
+    const int rows = (n_blocks + G - 1) / G;
+    double* scratch = const_cast<double*>(part) + (size_t)batch * n_blocks * n_shells;
+    const cudaError_t e = launch_overlapped(k_pk_rows, dim3(G, batch), 256, 0, s, part, n_blocks, n_shells, rows, scratch);
+    if (e != cudaSuccess) return e;
+    part = scratch;
+    n_blocks = G;
+  }
+  return launch_overlapped(k_pk_finalize_p, batch, kPkThreads, 0, s, part, n_blocks, n_shells, ksum, count, pk, k_mean, n_modes);
 }
 
 // A thread draws the pairs of two consecutive cells along z: rows iy (even) and iy + 1.

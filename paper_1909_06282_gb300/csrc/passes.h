@@ -295,6 +295,7 @@ cudaError_t launch_src_t1(int n_bins, const double* ksum, const unsigned long lo
 cudaError_t launch_pk_finalize_p(const double* part, int n_blocks, int n_shells, const double* ksum,
                                  const unsigned long long* count, double* pk, double* k_mean, int64_t* n_modes,
                                  cudaStream_t s, int batch);
+inline int pk_finalize_launches(int n_blocks, int n_shells) { return (long long)n_blocks * n_shells > 8192 ? 2 : 1; }
 cudaError_t launch_noise(const Geo& g, uint32_t seed_lo, uint32_t seed_hi, const float4* bm, float* out,
                          cudaStream_t);
 // Box-Muller transform of given word pairs (x0, x1) [count][2] -> floats [count][2].
