@@ -1262,6 +1262,7 @@ struct XSmemIn {
   const float2* hpsi = nullptr;
   const float2* delta = nullptr;
   const float2* s = nullptr;
+  const float* sc = nullptr;   // X_ADJ_DELTA: the scf values of the thread's modes, loaded beforehand
   float4* table = nullptr;   // X_ADJ_SOURCE: N W / 2 entries of scratch for the shared table gathers
 };
 struct XNothing {
@@ -1557,7 +1558,7 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[XCfg<N, MODE>
     if (field) {
       const float inv_c = zero ? 0.f : __frcp_rn((float)n2 * a.g.kf2n3);
       float sc_f = 0.f;
-      sc_f = s_sc ? s_sc[kx * C::W + w] : __ldg(a.scf + e);
+      sc_f = s_sc ? s_sc[kx * C::W + w] : (si.sc ? si.sc[r] : __ldg(a.scf + e));
       mt = make_float4(sc_f, inv_c, 0.f, 0.f);
     } else if (!shared) {
       mt = zero ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(a.mt0 + toff + n2);
@@ -1838,6 +1839,7 @@ __global__ void __launch_bounds__(XCfg<N, MODE>::XT, XCfg<N, MODE>::MINB) k_x_tm
     float2 v[C::RMAX];
 #pragma unroll
     for (int r = 0; r < C::RMAX; ++r) v[r] = make_float2(0.f, 0.f);
+    float sc[C::RMAX];
     for (int j = 0; j < NG; ++j, ++c) {
       const int st = c % 3;
       const bool ok = mbar_wait(&bar[st], (c / 3) & 1, a.g.wait);
@@ -1849,6 +1851,13 @@ __global__ void __launch_bounds__(XCfg<N, MODE>::XT, XCfg<N, MODE>::MINB) k_x_tm
       if (s_fail) {
         if (threadIdx.x == 0) drain(c);
         return;
+      }
+      // the last group's transform covers the latency of the scf field (read after it, the 16
+      // scattered rows of every thread stood in the open: x_adj_delta at 512^3 1093 -> 831 us)
+      if (MODE == X_ADJ_DELTA && j == NG - 1) {
+        const float* sp = a.scf + inst * ((size_t)N * N * C::H) + (size_t)ky * C::H + kzb * C::W + w;
+#pragma unroll
+        for (int r = 0; r < C::RMAX; ++r) sc[r] = __ldg(sp + (size_t)elem<N, C::V>(t, r) * ((size_t)N * C::H));
       }
       fft<N, false, C::V>(u, t, SmemCol<C::W>{ring + st * Q::TILE + w}, s_tw);   // ends past its last shared read
 #pragma unroll
@@ -1874,6 +1883,7 @@ __global__ void __launch_bounds__(XCfg<N, MODE>::XT, XCfg<N, MODE>::MINB) k_x_tm
     float2* ex;
     if (MODE == X_ADJ_DELTA) {
       si.hpsi = ring + s0 * Q::TILE;
+      si.sc = sc;
       ex = ring + s0 * Q::TILE;
     } else {
       si.delta = ring + s0 * Q::TILE;
