@@ -80,7 +80,7 @@ struct Group {
   float2* tw;      // twiddles, in the stages' order (twiddle_exponent)
   size_t off;      // floats before the group's first instance in per-instance real fields
   float4* mt0;     // per-|n|^2 multiplier tables [count][mode_table_len(n)]
-  float2* mt1;
+  float4* mt1;
   double* geo_k;             // P(k) shell geometry for geo_ns shells: sum of |k| per shell
   unsigned long long* geo_n; // and mode count per shell [kMaxShells]
   int geo_ns;                // 0: not computed yet
@@ -113,7 +113,7 @@ struct lpt2_plan_s {
   double box;
   float2* tw;
   const float4* mt0;
-  const float2* mt1;
+  const float4* mt1;
   int cur_batch, cur_inst0;
   int cur_ytile = 0, cur_xtile = 0;   // tile schedule of the current group
   size_t cur_slot_off = 0;    // bytes into every workspace slot of the current instances (a chunk of a group)
@@ -271,6 +271,7 @@ WsLayout ws_layout(size_t slot_sz, size_t total_cells, int xb_max, int n_inst, i
   w.out_tab = 0;
   w.out_tabf = up256((size_t)4 * nk * sizeof(double));
   w.out_mt0 = up256(w.out_tabf + (size_t)4 * nk * sizeof(float));
+  // (the adjoint reads no tables of an output time; the room of a second one stays in the layout)
   w.out_mt1 = up256(w.out_mt0 + len * sizeof(float4));
   w.out_each = up256(w.out_mt1 + len * sizeof(float2));
   w.total = w.outs + (size_t)max_out * w.out_each;
@@ -594,10 +595,6 @@ float4* out_mt0(lpt2_plan_t p, int j) {
   const WsLayout w = ws_layout(p);
   return reinterpret_cast<float4*>(p->ws + w.outs + j * w.out_each + w.out_mt0);
 }
-float2* out_mt1(lpt2_plan_t p, int j) {
-  const WsLayout w = ws_layout(p);
-  return reinterpret_cast<float2*>(p->ws + w.outs + j * w.out_each + w.out_mt1);
-}
 
 // Growth and multiplier tables of every output scale factor (single-instance plan).
 int run_output_growth(lpt2_plan_t p) {
@@ -607,7 +604,7 @@ int run_output_growth(lpt2_plan_t p) {
     LAUNCH(p, "growth", 0.0, launch_growth(gp, out_tab(p, j), out_tabf(p, j), p->stream));
     LAUNCH(p, "mode_tables", 0.0,
            launch_mode_tables(gp, p->cosmo_dev, out_tab(p, j), 0, 1, p->groups[0].n, p->groups[0].box,
-                              out_mt0(p, j), out_mt1(p, j), p->stream));
+                              out_mt0(p, j), nullptr, p->stream));
   }
   return LPT2_OK;
 }
@@ -782,7 +779,7 @@ int lpt2_plan(lpt2_plan_t* out, const lpt2_instance* inst, int n_inst, int n_k, 
   for (Group& g : p->groups) {
     if (e == cudaSuccess) e = plan_malloc((void**)&g.tw, g.n * sizeof(float2));
     if (e == cudaSuccess) e = plan_malloc((void**)&g.mt0, (size_t)g.count * mode_table_len(g.n) * sizeof(float4));
-    if (e == cudaSuccess) e = plan_malloc((void**)&g.mt1, (size_t)g.count * mode_table_len(g.n) * sizeof(float2));
+    if (e == cudaSuccess) e = plan_malloc((void**)&g.mt1, (size_t)g.count * mode_table_len(g.n) * sizeof(float4));
     if (e == cudaSuccess) e = plan_malloc((void**)&g.geo_k, kMaxShells * sizeof(double));
     if (e == cudaSuccess) e = plan_malloc((void**)&g.geo_n, kMaxShells * sizeof(unsigned long long));
     g.geo_ns = 0;
@@ -1084,10 +1081,10 @@ int displace_prefix(lpt2_plan_t p, const FwdSlots& f, const float* noise, bool s
 }
 
 // Steps of one output scale factor, whose D1(k, a), D2(k, a) enter through the
-// multiplier tables mt0 / mt1 and the growth tables tabf: S(k) -> phi2 (+ phi1 D1),
+// multiplier tables mt0 and the growth tables tabf: S(k) -> phi2 (+ phi1 D1),
 // Psi, positions, CIC density (slots A and D are read, not written).
 int displace_suffix(lpt2_plan_t p, const FwdSlots& f, bool split, float* psi1, float* psi2, float* pos,
-                    float2* s_keep, const float4* mt0, const float2* mt1, const float* tabf,
+                    float2* s_keep, const float4* mt0, const float* tabf,
                     float* pos_scratch = nullptr) {
   const int n = p->n;
   const Geo g = make_geo(p);
@@ -1108,7 +1105,6 @@ int displace_suffix(lpt2_plan_t p, const FwdSlots& f, bool split, float* psi1, f
   xs.out[1] = f.X[1];
   xs.cosmo = p->cosmo_dev;
   xs.mt0 = mt0;
-  xs.mt1 = mt1;
   xs.d1f = tabf;
   xs.d2f = tabf + p->nk;
   xs.t1f = tabf + 2 * p->nk;
@@ -1161,7 +1157,7 @@ int displace_impl(lpt2_plan_t p, const float* noise, float* psi1, float* psi2, f
   const FwdSlots f = fwd_slots(p);
   int rc = displace_prefix(p, f, noise, split);
   if (rc) return rc;
-  rc = displace_suffix(p, f, split, psi1, psi2, pos, s_keep, p->mt0, p->mt1, p->tabf, pos_scratch);
+  rc = displace_suffix(p, f, split, psi1, psi2, pos, s_keep, p->mt0, p->tabf, pos_scratch);
   if (rc) return rc;
   if (dk) {
     const size_t cells = (size_t)p->n * p->n * p->n * p->cur_batch;
@@ -1344,7 +1340,7 @@ int lpt2_displace_outputs(lpt2_plan_t p, const float* noise, float* pos, double*
   const size_t n3 = (size_t)p->n * p->n * p->n;
   for (int j = 0; j < p->n_out_a; ++j) {
     rc = displace_suffix(p, f, false, nullptr, nullptr, pos ? pos + j * 3 * n3 : nullptr, nullptr,
-                         out_mt0(p, j), out_mt1(p, j), out_tabf(p, j));
+                         out_mt0(p, j), out_tabf(p, j));
     if (rc) return rc;
     // the density spectrum goes to a slot the suffix does not use (A and D stay intact)
     rc = cic_pk_group(p, 0, nullptr, nullptr, pk + (size_t)j * n_shells, j == 0 ? k_mean : nullptr,

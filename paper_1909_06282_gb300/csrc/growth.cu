@@ -452,8 +452,9 @@ cudaError_t launch_growth(const GrowthParams& p, double* tab, float* tabf, cudaS
 // For every integer |n|^2 of an n^3 grid: k = (2 pi / L) sqrt(|n|^2),
 //   x = sqrt(P_lin(k) N^3 / V)  (EH no-wiggle, sigma_8 amplitude),
 //   y = 1 / (k^2 N^3),
-//   z, w = D1(k), D2(k) and (mt1) dD1, dD2 / dln|fR0|, linear in ln k between the
-// growth-table nodes and clamped at the ends - all in FP64, rounded once.
+//   z, w = D1(k), D2(k), linear in ln k between the growth-table nodes and clamped at the
+// ends - all in FP64, rounded once; and mt1 (where given) the FP32 products of D1, D2 and their
+// derivatives by ln|fR0| with y, the four values the adjoint source pass multiplies by.
 __device__ double interp_lnk64(const double* t, int nk, double lnkmin, double dlnk, double lnk) {
   double x = (lnk - lnkmin) / dlnk;
   if (x <= 0.0) return t[0];
@@ -465,17 +466,16 @@ __device__ double interp_lnk64(const double* t, int nk, double lnkmin, double dl
 }
 
 __global__ void k_mode_tables(GrowthParams p, const DevCosmo* cosmo, const double* tab, int inst0, int n, double box,
-                              float4* mt0, float2* mt1) {
+                              float4* mt0, float4* mt1) {
   const int len = mode_table_len(n);
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= len) return;
   const int inst = inst0 + blockIdx.y;
   const double* tb = tab + (size_t)inst * 4 * p.nk;
   float4* o0 = mt0 + (size_t)blockIdx.y * len;
-  float2* o1 = mt1 + (size_t)blockIdx.y * len;
   if (idx == 0) {
     o0[0] = make_float4(0.f, 0.f, 0.f, 0.f);
-    o1[0] = make_float2(0.f, 0.f);
+    if (mt1) mt1[(size_t)blockIdx.y * len] = make_float4(0.f, 0.f, 0.f, 0.f);
     return;
   }
   const double nd = n, kf = 2.0 * M_PI / box;
@@ -490,11 +490,13 @@ __global__ void k_mode_tables(GrowthParams p, const DevCosmo* cosmo, const doubl
   const double t1 = interp_lnk64(tb + 2 * p.nk, p.nk, lnkmin, dlnk, lk);
   const double t2 = interp_lnk64(tb + 3 * p.nk, p.nk, lnkmin, dlnk, lk);
   o0[idx] = make_float4((float)sp, (float)inv, (float)d1, (float)d2);
-  o1[idx] = make_float2((float)t1, (float)t2);
+  if (!mt1) return;
+  const float iv = (float)inv;
+  mt1[(size_t)blockIdx.y * len + idx] = make_float4((float)d1 * iv, (float)d2 * iv, (float)t1 * iv, (float)t2 * iv);
 }
 
 cudaError_t launch_mode_tables(const GrowthParams& p, const DevCosmo* cosmo, const double* tab, int inst0, int count,
-                               int n, double box, float4* mt0, float2* mt1, cudaStream_t s) {
+                               int n, double box, float4* mt0, float4* mt1, cudaStream_t s) {
   const int len = mode_table_len(n);
   k_mode_tables<<<dim3((len + 127) / 128, count), 128, 0, s>>>(p, cosmo, tab, inst0, n, box, mt0, mt1);
   return cudaGetLastError();

@@ -1262,6 +1262,7 @@ struct XSmemIn {
   const float2* hpsi = nullptr;
   const float2* delta = nullptr;
   const float2* s = nullptr;
+  const float4* mt = nullptr;   // X_ADJ_SOURCE: the thread's table entries (kx < N/2), loaded beforehand
   const float* sc = nullptr;   // X_ADJ_DELTA: the scf values of the thread's modes, loaded beforehand
   float4* table = nullptr;   // X_ADJ_SOURCE: N W / 2 entries of scratch for the shared table gathers
 };
@@ -1525,7 +1526,8 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[XCfg<N, MODE>
   // entries and hands the products D1, D2 (and the tangents) over k^2 N^3 to the one that
   // holds N - kx, through the exchange buffer (free between the transforms) or the caller's
   // scratch: half the gathers, whose 32 scattered entries per warp take an L1 cycle each (512^3:
-  // x_source 777 -> 726 us, its split form at 256^3 84 -> 70 us, x_adj_source 1319 -> 1029 us with the earlier refill of its ring).
+  // x_source 777 -> 726 us, its split form at 256^3 84 -> 70 us, x_adj_source 1319 -> 1029 us with the earlier
+  // refill of its ring).
   constexpr bool shared = MODE == X_SOURCE || MODE == X_ADJ_SOURCE;
   float4* table = MODE == X_ADJ_SOURCE ? (si.table ? si.table : reinterpret_cast<float4*>(sm.base - w)) + w : nullptr;
   if constexpr (shared) {
@@ -1535,12 +1537,11 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[XCfg<N, MODE>
       if (kx >= C::H) continue;
       const int n2 = kx * kx + my * my + mz * mz;
       const bool none = ny_nyq || n2 == 0;
-      const float4 mt = none ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(a.mt0 + toff + n2);
       if (MODE == X_SOURCE) {
+        const float4 mt = none ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(a.mt0 + toff + n2);
         sm.st(kx, make_float2(mt.z * mt.y, mt.w * mt.y));
       } else {
-        const float2 tt = none ? make_float2(0.f, 0.f) : __ldg(a.mt1 + toff + n2);
-        table[kx * C::W] = make_float4(mt.z * mt.y, mt.w * mt.y, tt.x * mt.y, tt.y * mt.y);
+        table[kx * C::W] = si.mt ? si.mt[r] : none ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(a.mt1 + toff + n2);
       }
     }
     __syncthreads();
@@ -1840,6 +1841,7 @@ __global__ void __launch_bounds__(XCfg<N, MODE>::XT, XCfg<N, MODE>::MINB) k_x_tm
 #pragma unroll
     for (int r = 0; r < C::RMAX; ++r) v[r] = make_float2(0.f, 0.f);
     float sc[C::RMAX];
+    float4 mt[C::RMAX];
     for (int j = 0; j < NG; ++j, ++c) {
       const int st = c % 3;
       const bool ok = mbar_wait(&bar[st], (c / 3) & 1, a.g.wait);
@@ -1854,6 +1856,19 @@ __global__ void __launch_bounds__(XCfg<N, MODE>::XT, XCfg<N, MODE>::MINB) k_x_tm
       }
       // the last group's transform covers the latency of the scf field (read after it, the 16
       // scattered rows of every thread stood in the open: x_adj_delta at 512^3 1093 -> 831 us)
+      // the same for the table entries (x_adj_source at 512^3 1022 -> 880 us with the entry one float4
+      // instead of a gather from each of two tables, which alone gave 913)
+      if (MODE == X_ADJ_SOURCE && j == NG - 1) {
+        const float4* mp = a.mt1 + (size_t)inst * mode_table_len(N);
+        const int kz = kzb * C::W + w, my = mode_of(ky, N);
+#pragma unroll
+        for (int r = 0; r < C::RMAX; ++r) {
+          const int kx = elem<N, C::V>(t, r);
+          if (kx >= C::H) continue;
+          const int n2 = kx * kx + my * my + kz * kz;
+          mt[r] = ky == C::H || n2 == 0 ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(mp + n2);
+        }
+      }
       if (MODE == X_ADJ_DELTA && j == NG - 1) {
         const float* sp = a.scf + inst * ((size_t)N * N * C::H) + (size_t)ky * C::H + kzb * C::W + w;
 #pragma unroll
@@ -1887,6 +1902,7 @@ __global__ void __launch_bounds__(XCfg<N, MODE>::XT, XCfg<N, MODE>::MINB) k_x_tm
       ex = ring + s0 * Q::TILE;
     } else {
       si.delta = ring + s0 * Q::TILE;
+      si.mt = mt;
       si.s = ring + s1 * Q::TILE;
       si.table = reinterpret_cast<float4*>(ring + ((c + 2) % 3) * Q::TILE);   // the last group's stage
       ex = ring + s1 * Q::TILE;

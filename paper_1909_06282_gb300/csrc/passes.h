@@ -187,9 +187,10 @@ struct XArgs {
   int n_shells;
   const float* shell_w;   // X_PKADJ: weight per shell
   // per-|n|^2 multiplier tables of the group (index = global instance - inst0 of the
-  // group, then |n|^2): {sqrt(P N^3/V), 1/(k^2 N^3), D1, D2} and {dD1, dD2}/dln|fR0|
+  // group, then |n|^2): {sqrt(P N^3/V), 1/(k^2 N^3), D1, D2} and {D1, D2, dD1/dln|fR0|,
+  // dD2/dln|fR0|} / (k^2 N^3) (X_ADJ_SOURCE)
   const float4* mt0;
-  const float2* mt1;
+  const float4* mt1;
   // X_DELTA (without the split) and X_ADJ_DELTA: sqrt(P N^3/V) of every mode of the group's
   // half spectra, float[batch][N][N][N/2] in the fields' layout (zero on the modes the
   // passes zero), or null for the mode table; with it, 1/(k^2 N^3) is computed
@@ -323,7 +324,7 @@ cudaError_t launch_growth(const GrowthParams&, double* tab /*[4][nk]*/, float* t
 // |n|^2 = 0 .. 3 (n/2)^2 per instance (FP64 evaluation, rounded once).
 __host__ __device__ inline int mode_table_len(int n) { return 3 * (n / 2) * (n / 2) + 1; }
 cudaError_t launch_mode_tables(const GrowthParams&, const DevCosmo* cosmo, const double* tab, int inst0, int count,
-                               int n, double box, float4* mt0, float2* mt1, cudaStream_t);
+                               int n, double box, float4* mt0, float4* mt1, cudaStream_t);
 cudaError_t launch_pk_adj_weights(const double* g_pk, const int64_t* n_modes, int n_shells, double v_over_n6,
                                   float* w, cudaStream_t);
 cudaError_t launch_sum_partials(const double* part, int n, double* out, cudaStream_t);
