@@ -1014,7 +1014,10 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_adj_source_ct
 // Per row: three inverse and three forward transforms, each phi_ij and g_S read once (the
 // paired-row form transforms 7.5 pencils per row and reads the diagonal fields twice).
 // Tiles as in the field-pair layout: a ring stage holds the two fields of a pencil for the
-// CTA's eight rows, each row in its warp's padded region, used in place as the exchange row.
+// CTA's eight rows, each row in its warp's padded region, used in place as the exchange row.  The
+// rows of g_S come with them: read from global memory where they are used, behind a
+// transform, they cost 250 us (512^3: 2005 -> 1754).  One tile per CTA: a persistent walk needs
+// registers that spill (2654 us).
 #ifndef LPT2_ZADJ_FIELD_PAIRS
 #define LPT2_ZADJ_FIELD_PAIRS 1
 #endif
@@ -1025,10 +1028,12 @@ template <int N> struct ZAdjFpCfg {
   static constexpr int ROWW = SmemRow::words(N);               // float2 per warp region
   static constexpr int STAGE_F2 = ROWS * ROWW;
   static constexpr unsigned STAGE_BYTES = ROWS * 2 * H * 8u;   // bytes landing per stage
-  static constexpr int BAR_OFF = (N + 2 * STAGE_F2) * 8;       // twiddles, two stages, barriers
+  static constexpr int GS_OFF = (N + 2 * STAGE_F2) * 8;        // twiddles, two stages, g_S rows, barriers
+  static constexpr unsigned GS_BYTES = ROWS * N * 4u;
+  static constexpr int BAR_OFF = GS_OFF + (int)GS_BYTES;
   static constexpr int SMEM = BAR_OFF + 64;
   static constexpr bool OK = TPP == 32;
-  static_assert(!OK || ((ROWW * 8) % 16 == 0 && (H * 8) % 16 == 0), "bulk copies need 16-byte alignment");
+  static_assert(!OK || ((ROWW * 8) % 16 == 0 && (H * 8) % 16 == 0 && GS_OFF % 16 == 0), "bulk copies need 16-byte alignment");
 };
 template <int N> constexpr bool zadj_field_pairs() { return LPT2_ZADJ_FIELD_PAIRS && ZAdjFpCfg<N>::OK; }
 
@@ -1058,25 +1063,30 @@ __global__ void __launch_bounds__(ZAdjFpCfg<N>::THREADS, 2) k_z_adj_source_fp(ZA
     s_fail = 0;
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
+    mbar_init(&bar[2], 1);
     mbar_init_fence();
   }
-  const float* gsr = a.gs + zr + row * N;   // g_S of this row (read where used: registers are short)
+  float* s_gs = reinterpret_cast<float*>(za_raw + Q::GS_OFF);   // g_S of the CTA's rows
+  const float* gsr = s_gs + warp * N;
   load_twiddles(s_tw, a.tw, N);
   grid_sync();
   if (threadIdx.x == 0) {
     issue(0);
     issue(1);
+    mbar_expect_tx(&bar[2], Q::GS_BYTES);
+    bulk_load(s_gs, a.gs + zr + row0 * N, Q::GS_BYTES, &bar[2]);
   }
   __syncthreads();
   // pencil k of this warp's row into v (Hermitian extension of both fields with their z
   // derivative orders, Z = A + i B); false if a wait ran out (drained and reported)
   auto fetch = [&](int k, float2 (&v)[RMAX]) -> bool {
-    const bool ok = mbar_wait(&bar[k & 1], (k >> 1) & 1, a.g.wait);
+    const bool ok = mbar_wait(&bar[k & 1], (k >> 1) & 1, a.g.wait) && (k != 1 || mbar_wait(&bar[2], 0, a.g.wait));
     if (!ok) s_fail = 1;
     __syncthreads();
     if (s_fail) {
       if (threadIdx.x == 0) {
         for (int g = k; g < (k == 0 ? 2 : 3); ++g) mbar_wait(&bar[g & 1], (g >> 1) & 1);
+        mbar_wait(&bar[2], 0);
         report_device_error(a.g.err, LPT2_DEV_ETIMEOUT_ZADJSOURCE);
       }
       return false;
@@ -1116,7 +1126,7 @@ __global__ void __launch_bounds__(ZAdjFpCfg<N>::THREADS, 2) k_z_adj_source_fp(ZA
   fft<N, true>(v, t, sm1, s_tw);
 #pragma unroll
   for (int r = 0; r < RMAX; ++r) {
-    const float A = ab[r].x, B = ab[r].y, Cz = v[r].x, D = v[r].y, g = __ldg(gsr + elem<N>(t, r));
+    const float A = ab[r].x, B = ab[r].y, Cz = v[r].x, D = v[r].y, g = gsr[elem<N>(t, r)];
     q[r] = make_float2(g * (A + B), -2.f * g * D);    // g_zz + i g_xy
     v[r] = make_float2(g * (B + Cz), g * (A + Cz));   // g_xx + i g_yy
   }
@@ -1130,7 +1140,7 @@ __global__ void __launch_bounds__(ZAdjFpCfg<N>::THREADS, 2) k_z_adj_source_fp(ZA
   fft<N, true>(v, t, sm0, s_tw);
 #pragma unroll
   for (int r = 0; r < RMAX; ++r) {
-    const float g = -2.f * __ldg(gsr + elem<N>(t, r));
+    const float g = -2.f * gsr[elem<N>(t, r)];
     v[r] = make_float2(g * v[r].x, g * v[r].y);
   }
   fft<N, false>(v, t, sm0, s_tw);
