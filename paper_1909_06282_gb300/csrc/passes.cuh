@@ -1306,6 +1306,8 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[XCfg<N, MODE>
   (void)warp;
   (void)lane;
   const bool adjoint = (MODE == X_ADJ_SOURCE || MODE == X_ADJ_DELTA);
+  float2* mult = sm.base + N * C::W;   // X_SOURCE: the multipliers, behind the exchange buffer (sm.base includes w)
+  float2 dl[MODE == X_SOURCE && !SPLIT ? C::RMAX : 1];
   if (adjoint && !si.summed) {
     // forward x transform of each x-order group, summed with conj((i kx)^m)
     const int ng = (MODE == X_ADJ_SOURCE) ? 2 : 3;
@@ -1356,6 +1358,25 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[XCfg<N, MODE>
 #pragma unroll
       for (int r = 0; r < C::RMAX; ++r) a.out[0][base + (size_t)(elem<N, C::V>(t, r)) * stride] = v[r];
       return;
+    }
+    // X_SOURCE: the multipliers to shared memory and delta(k) to registers before the transform, whose
+    // latency they would otherwise add to (x_source at 512^3 727 -> 698 us, 96 batched instances
+    // 1497 -> 1417, its split form at 256^3 69.6 -> 67.0; the multipliers alone 1550 for the batch)
+    if constexpr (MODE == X_SOURCE) {
+      const size_t toff = (size_t)inst * mode_table_len(N);
+#pragma unroll
+      for (int r = 0; r < C::RMAX; ++r) {
+        const int kx = elem<N, C::V>(t, r);
+        if (kx >= C::H) continue;
+        const int n2 = kx * kx + my * my + mz * mz;
+        const bool none = ny_nyq || n2 == 0;
+        const float4 mt = none ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(a.mt0 + toff + n2);
+        mult[kx * C::W] = make_float2(mt.z * mt.y, mt.w * mt.y);
+      }
+      if constexpr (!SPLIT) {
+#pragma unroll
+        for (int r = 0; r < C::RMAX; ++r) dl[r] = a.delta_in[base + (size_t)(elem<N, C::V>(t, r)) * stride];
+      }
     }
     fft<N, false, C::V>(v, t, sm, s_tw);
     if (MODE == X_FWD) {
@@ -1533,12 +1554,11 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[XCfg<N, MODE>
   const size_t toff = (size_t)inst * mode_table_len(N);
   constexpr bool field = (MODE == X_DELTA && !SPLIT) || MODE == X_ADJ_DELTA;
   // Source modes: kx and N - kx have the same |n|^2, so the thread that holds kx < N/2 gathers its
-  // entries and hands the products D1, D2 (and the tangents) over k^2 N^3 to the one that
-  // holds N - kx, through the exchange buffer (free between the transforms) or the caller's
-  // scratch: half the gathers, whose 32 scattered entries per warp take an L1 cycle each (512^3:
-  // x_source 777 -> 726 us, its split form at 256^3 84 -> 70 us, x_adj_source 1319 -> 1029 us with the earlier
-  // refill of its ring).
-  constexpr bool shared = MODE == X_SOURCE || MODE == X_ADJ_SOURCE;
+  // entry and hands the products D1, D2 (and the tangents) over k^2 N^3 to the one that holds N -
+  // kx through shared memory (`mult`, `table`): half the gathers, whose 32 scattered entries per
+  // warp take an L1 cycle each (x_source at 512^3 777 -> 726 us, its split form at 256^3 84 -> 70,
+  // x_adj_source at 512^3 1319 -> 1029 with the earlier refill of its ring).
+  constexpr bool shared = MODE == X_ADJ_SOURCE;
   float4* table = MODE == X_ADJ_SOURCE ? (si.table ? si.table : reinterpret_cast<float4*>(sm.base - w)) + w : nullptr;
   if constexpr (shared) {
 #pragma unroll
@@ -1546,13 +1566,9 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[XCfg<N, MODE>
       const int kx = elem<N, C::V>(t, r);
       if (kx >= C::H) continue;
       const int n2 = kx * kx + my * my + mz * mz;
-      const bool none = ny_nyq || n2 == 0;
-      if (MODE == X_SOURCE) {
-        const float4 mt = none ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(a.mt0 + toff + n2);
-        sm.st(kx, make_float2(mt.z * mt.y, mt.w * mt.y));
-      } else {
-        table[kx * C::W] = si.mt ? si.mt[r] : none ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(a.mt1 + toff + n2);
-      }
+      table[kx * C::W] =
+          si.mt ? si.mt[r]
+                : ny_nyq || n2 == 0 ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(a.mt1 + toff + n2);
     }
     __syncthreads();
   }
@@ -1571,7 +1587,7 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[XCfg<N, MODE>
       float sc_f = 0.f;
       sc_f = s_sc ? s_sc[kx * C::W + w] : (si.sc ? si.sc[r] : __ldg(a.scf + e));
       mt = make_float4(sc_f, inv_c, 0.f, 0.f);
-    } else if (!shared) {
+    } else if (!shared && MODE != X_SOURCE) {
       mt = zero ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(a.mt0 + toff + n2);
     } else {
       mt = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1583,11 +1599,10 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[XCfg<N, MODE>
       g[r] = cscale(d, inv);                                // phi1 = delta / k^2 (1/N^3 folded)
       if constexpr (SPLIT) hpot[r] = cscale(g[r], d1);
     } else if (MODE == X_SOURCE) {                        // v = S(k)
-      const float2 m = kx == C::H ? make_float2(0.f, 0.f) : sm.ld(kx < C::H ? kx : N - kx);
+      const float2 m = kx == C::H ? make_float2(0.f, 0.f) : mult[(kx < C::H ? kx : N - kx) * C::W];
       float2 u = cscale(v[r], -m.y);                        // phi2 = -S D2 / k^2
       if constexpr (!SPLIT) {
-        const float2 dl = a.delta_in[e];
-        u = cadd(u, cscale(dl, m.x));                       // + phi1 D1 (total potential)
+        u = cadd(u, cscale(dl[r], m.x));                       // + phi1 D1 (total potential)
       }
       g[r] = u;
     } else if (MODE == X_ADJ_SOURCE) {                    // v = g_u(k)
@@ -2081,7 +2096,7 @@ template <int N, int MODE> cudaError_t launch_x_m(const XArgs& a, cudaStream_t s
       return a.split ? launch_x_tma<N, MODE, false>(a, acc, s) : launch_x_tma<N, MODE, true>(a, acc, s);
     }
   }
-  const int smem = C::XSMEM + acc;
+  const int smem = C::XSMEM + acc + (MODE == X_SOURCE ? N * C::W * 4 : 0);
   constexpr bool has_split = MODE == X_DELTA || MODE == X_SOURCE;
   auto k = has_split && a.split ? k_x<N, MODE, has_split> : k_x<N, MODE, false>;
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
