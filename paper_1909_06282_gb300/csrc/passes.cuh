@@ -1592,7 +1592,7 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[XCfg<N, MODE>
     } else {
       mt = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    const float sc = mt.x, inv = mt.y, d1 = mt.z, d2 = mt.w;   // sqrt(P N^3/V), 1/(k^2 N^3), D1, D2
+    const float sc = mt.x, inv = mt.y, d1 = mt.z;   // sqrt(P N^3/V), 1/(k^2 N^3), D1
     if (MODE == X_DELTA) {
       const float2 d = cscale(v[r], sc);
       if (a.delta_out) a.delta_out[e] = d;
