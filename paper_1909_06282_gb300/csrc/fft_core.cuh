@@ -60,6 +60,7 @@ template <> struct Cfg<256>  { static constexpr int NS = 2, RMAX = 16; static __
 template <> struct Cfg<512>  { static constexpr int NS = 3, RMAX = LPT2_R512;
   static __host__ __device__ constexpr int rad(int s) { return LPT2_R512 == 8 ? 8 : (s == 1 ? 2 : 16); } };
 template <> struct Cfg<1024> { static constexpr int NS = 3, RMAX = 16; static __host__ __device__ constexpr int rad(int s) { return s == 1 ? 4 : 16; } };
+template <> struct Cfg<32, 1>  { static constexpr int NS = 2, RMAX = 8;  static __host__ __device__ constexpr int rad(int s) { return s == 0 ? 8 : 4; } };
 template <> struct Cfg<512, 1> { static constexpr int NS = 2, RMAX = 32; static __host__ __device__ constexpr int rad(int s) { return s == 0 ? 32 : 16; } };
 
 // element index held in register slot j by lane t (first-stage input, and output of fft())

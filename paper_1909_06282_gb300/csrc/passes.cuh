@@ -56,17 +56,18 @@ template <int N> struct PassCfg {
 // segments, so 16 kz per CTA; with 16 values per thread that CTA has 512 threads that
 // wait for one another (y_phi 1399 us), with 32 values 256 threads and one exchange instead
 // of two: y_phi 1067 -> 930 us, y_psi 537 -> 463, y_fwd 215 -> 184 against 8 kz and 16
-// values.  Two CTAs per SM: a third fits in registers (80), but its tile takes the L1 the loads in
+// values.  N = 32 (8-4 instead of 4-2-4): 64 batched grids y_phi 19.1 -> 16.4 us, x_pk 13.1 -> 10.5, the
+// call 108.5 -> 104.7.  Two CTAs per SM at 512: a third fits in registers (80), but its tile takes the L1 the loads in
 // flight need (y_phi 1098 us).  Y_SUM keeps an accumulator beside the values: 8 kz, 16 values.
 enum YKind { Y_MULTI = 0, Y_SUM = 1, Y_ONE = 2 };
 template <int N, int KIND, int WY = 0> struct YCfg {
   static constexpr int H = N / 2;
   static constexpr int W = WY ? WY : (N == 512 ? (KIND == Y_SUM ? 8 : 16) : PassCfg<N>::W);
-  static constexpr int V = N == 512 && W == 16 && KIND != Y_SUM ? 1 : 0;
+  static constexpr int V = ((N == 512 && W == 16) || N == 32) && KIND != Y_SUM ? 1 : 0;
   static constexpr int RMAX = Cfg<N, V>::RMAX;
   static constexpr int TPP = N / RMAX;
   static constexpr int XT = TPP * W;
-  static constexpr int MINB = V ? 2 : 0;   // resident CTAs asked of the compiler (0: none)
+  static constexpr int MINB = N == 512 && V ? 2 : 0;   // resident CTAs asked of the compiler (0: none)
   static constexpr int XSMEM = (N + N * W) * 8;
   static_assert(H % W == 0, "a CTA's kz block must tile the half spectrum");
 };
@@ -76,11 +77,12 @@ template <int N, int KIND, int WY = 0> struct YCfg {
 // 334.  Not the shell sums: they want the resident warps that 64 registers allow (250 us against
 // 275 with 32 values).
 template <int N, int MODE> struct XCfg {
-  static constexpr int V = N == 512 && (MODE == X_FWD || MODE == X_INV || MODE == X_PKADJ || MODE == X_MUL) ? 1 : 0;
+  static constexpr int V = (N == 512 && (MODE == X_FWD || MODE == X_INV || MODE == X_PKADJ || MODE == X_MUL)) ||
+                                   (N == 32 && (MODE == X_PKP || MODE == X_PKI)) ? 1 : 0;
   static constexpr int RMAX = Cfg<N, V>::RMAX;
   static constexpr int TPP = N / RMAX;
   static constexpr int H = N / 2;
-  static constexpr int W = V ? 16 : PassCfg<N>::W;   // kz per CTA
+  static constexpr int W = N == 512 && V ? 16 : PassCfg<N>::W;   // kz per CTA
   static constexpr int XT = TPP * W;
   static constexpr int XSMEM = (N + N * W) * 8;
   // resident CTAs per SM asked of the compiler: a cap of 128 registers, or 64 for the
