@@ -173,6 +173,18 @@ template <int R, bool INV> struct Dft {   // even R: split into even and odd hal
   }
 };
 
+// Three-stage sequences R0-2-R0 with R0 values per thread: the inputs e, e + R0 TPP / 2 of a radix-2
+// butterfly are the same register of threads t and t + TPP / 2.  Where those are lanes of one warp
+// (partner(): the lane mask, 0 where they are not), the middle stage can run on shuffles: one exchange
+// through shared memory per transform instead of two, which is what bounds the z passes (70 % of
+// their cycles) and whose CTA barriers the x passes wait at.  512^3: z_source 1099 -> 1043 us,
+// z_adj_source 1766 -> 1672, x_adj_delta 833 -> 769, x_adj_source 874 -> 857, x_pk 251 -> 240, z_c2r 208 ->
+// 198; 64 batched 32^3 grids: z_source 27.8 -> 22.7, z_final 20.4 -> 17.8.  Not where the 32 values in
+// flight spill (x_delta 740 -> 863, x_source 702 -> 723, the y passes that sum 1065 -> 1141), nor in
+// z_final at 512, whose independent warps miss the instruction cache (499 -> 512).
+template <int N, int V> inline constexpr bool kPaired =
+    Cfg<N, V>::NS == 3 && Cfg<N, V>::rad(1) == 2 && Cfg<N, V>::RMAX == Cfg<N, V>::rad(0);
+
 // --------------------------------------------------------- shared accessors
 // Z layout: one pencil per row of N + N/16 complex (one pad slot per 16).  The row is
 // private to its pencil; when the pencil's threads lie in one warp (WARP), the exchange
@@ -186,13 +198,17 @@ template <bool WARP = false> struct SmemRowT {
     else __syncthreads();
   }
   static __host__ __device__ constexpr int words(int n) { return n + n / 16; }
+  template <int N, int V> static constexpr int partner() { return WARP && kPaired<N, V> ? N / Cfg<N, V>::RMAX / 2 : 0; }
+  // where element n lies between the paired stages: stores from and loads into all lanes at once
+  // fall in different banks
+  template <int N> static __device__ __forceinline__ int paired_slot(int n) { return n + (n >> (N == 512 ? 5 : 4)); }
 };
 using SmemRow = SmemRowT<false>;
 // z-pass pencils of N points lie in one warp when N / RMAX <= 32 threads hold one
 template <int N> inline constexpr bool kRowWarp = (N / Cfg<N>::RMAX) <= 32;
 // The same row for a group of GT threads that runs on its own: a warp, or GT / 32 warps that meet
 // at the CTA's named barrier `bar`.
-template <int GT> struct SmemRowG {
+template <int GT, bool PAIR = true> struct SmemRowG {
   float2* base;
   int bar;
   __device__ __forceinline__ void st(int n, float2 v) const { base[n + (n >> 4)] = v; }
@@ -201,14 +217,29 @@ template <int GT> struct SmemRowG {
     if constexpr (GT == 32) __syncwarp();
     else asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(GT) : "memory");
   }
+  template <int N, int V> static constexpr int partner() {
+    return PAIR && GT == 32 && kPaired<N, V> ? N / Cfg<N, V>::RMAX / 2 : 0;
+  }
+  template <int N> static __device__ __forceinline__ int paired_slot(int n) { return n + (n >> (N == 512 ? 5 : 4)); }
 };
 // Column layout: W pencils interleaved, element (n, w) at n * W + w (a pencil spans warps).
-template <int W> struct SmemCol {
+template <int W, bool PAIR = false> struct SmemCol {
   float2* base;   // already offset by w
   __device__ __forceinline__ void st(int n, float2 v) const { base[n * W] = v; }
   __device__ __forceinline__ float2 ld(int n) const { return base[n * W]; }
   __device__ __forceinline__ void sync() const { __syncthreads(); }
+  // N = 512, W = 8: pencil_thread() puts t + 16 sixteen lanes from t
+  template <int N, int V> static constexpr int partner() { return PAIR && N == 512 && W == 8 && kPaired<N, V> ? 16 : 0; }
+  template <int N> static __device__ __forceinline__ int paired_slot(int n) { return (n ^ ((n >> 5) & 1)) * W; }
 };
+// Pencil position t of this thread in a CTA of W interleaved pencils (w = threadIdx.x % W).
+template <int N, int V, int W, bool PAIR> __device__ __forceinline__ int pencil_thread() {
+  if constexpr (SmemCol<W, PAIR>::template partner<N, V>() != 0) {   // lanes 0-15: t, t + 1; 16-31: t + 16, t + 17
+    return (int)((threadIdx.x >> 5) << 1) + (int)((threadIdx.x >> 3) & 1) + (int)(threadIdx.x & 16);
+  } else {
+    return threadIdx.x / W;
+  }
+}
 
 // ------------------------------------------------------------ stage engine
 // Runs all stages on v (in: x[t + r TPP], out: X[t + r TPP]).  Every thread of
@@ -237,7 +268,29 @@ __device__ __forceinline__ void fft_stages(float2 (&v)[Cfg<N, V>::RMAX], int t, 
     }
     Dft<R, INV>::run(&v[q * R]);
   }
-  if constexpr (S + 1 < C::NS) {
+  if constexpr (S == 0 && SM::template partner<N, V>() != 0) {
+    // radix 2 with the partner lane (its twiddles are constants of the register), then one exchange
+    constexpr int M = SM::template partner<N, V>();
+    const bool up = (t & (TPP / 2)) != 0;
+    if (up) {
+#pragma unroll
+      for (int r = 1; r < R; ++r) v[r] = cmul(v[r], root96(r * (96 / (2 * R)), INV));
+    }
+    const float2 sg = pair(up ? -1.f : 1.f);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const float2 o = make_float2(__shfl_xor_sync(0xffffffffu, v[r].x, M), __shfl_xor_sync(0xffffffffu, v[r].y, M));
+      v[r] = pfma(v[r], sg, o);
+    }
+    const int d = (t & (TPP / 2 - 1)) * (2 * R) + (up ? R : 0);
+#pragma unroll
+    for (int r = 0; r < R; ++r) sm.base[SM::template paired_slot<N>(d + r)] = v[r];
+    sm.sync();
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = sm.base[SM::template paired_slot<N>(t + r * TPP)];
+    sm.sync();
+    fft_stages<N, INV, S + 2, V, SM>(v, t, sm, tw);
+  } else if constexpr (S + 1 < C::NS) {
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
       const int b = t + q * TPP;

@@ -67,6 +67,7 @@ template <int N, int KIND, int WY = 0> struct YCfg {
   static constexpr int RMAX = Cfg<N, V>::RMAX;
   static constexpr int TPP = N / RMAX;
   static constexpr int XT = TPP * W;
+  static constexpr bool PAIR = false;
   static constexpr int MINB = N == 512 && V ? 2 : 0;   // resident CTAs asked of the compiler (0: none)
   static constexpr int XSMEM = (N + N * W) * 8;
   static_assert(H % W == 0, "a CTA's kz block must tile the half spectrum");
@@ -84,6 +85,9 @@ template <int N, int MODE> struct XCfg {
   static constexpr int H = N / 2;
   static constexpr int W = N == 512 && V ? 16 : PassCfg<N>::W;   // kz per CTA
   static constexpr int XT = TPP * W;
+  // middle radix by shuffles (N = 512; see kPaired)
+  static constexpr bool PAIR =
+      MODE == X_PKP || MODE == X_PKI || MODE == X_ADJ_SOURCE || MODE == X_ADJ_DELTA;
   static constexpr int XSMEM = (N + N * W) * 8;
   // resident CTAs per SM asked of the compiler: a cap of 128 registers, or 64 for the
   // one-transform shell sums (twice the CTAs)
@@ -635,7 +639,7 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_final(ZFinalA
   float2* s_tw = reinterpret_cast<float2*>(zs_raw);
   __shared__ int s_fail[Q::GROUPS];
   const int group = threadIdx.x / Q::GT, p = threadIdx.x / C::TPP, pl = p % Q::PP, t = threadIdx.x % C::TPP;
-  const SmemRowG<Q::GT> sm{s_tw + Q::ROW_OFF + p * SmemRow::words(N), 1 + group};
+  const SmemRowG<Q::GT, N != 512> sm{s_tw + Q::ROW_OFF + p * SmemRow::words(N), 1 + group};
   constexpr size_t n3 = (size_t)N * N * N;
   auto src = [&](int q, int tile) {
     return (SPLIT ? ((q & 1) ? a.b[q >> 1] : a.a[q >> 1]) : a.a[q]) + (size_t)tile * Q::STAGE_F2;
@@ -1150,7 +1154,7 @@ __global__ void __launch_bounds__(ZAdjFpCfg<N>::THREADS, 2) k_z_adj_source_fp(ZA
 }
 
 // ===================================================================== y pass
-// CTA = (kz block of W, fixed x). Thread tid = t * W + w.
+// CTA = (kz block of W, fixed x). Thread (t, w) = (pencil_thread(), tid % W).
 // KIND: Y_MULTI  each output = transform of (i k_y)^ord times its input; the input
 //                tile is re-read (an L2 hit after the first) for every output so no
 //                input copy stays in registers;
@@ -1163,8 +1167,8 @@ __global__ void __launch_bounds__(YCfg<N, KIND, WY>::XT, YCfg<N, KIND, WY>::MINB
   float2* s_tw = smem;
   load_twiddles(s_tw, a.tw, N);
   grid_sync();
-  const int w = threadIdx.x % C::W, t = threadIdx.x / C::W;
-  const SmemCol<C::W> sm{smem + N + w};
+  const int w = threadIdx.x % C::W, t = pencil_thread<N, C::V, C::W, C::PAIR>();
+  const SmemCol<C::W, C::PAIR> sm{smem + N + w};
   const int kz = blockIdx.x * C::W + w;
   const int x = blockIdx.y;
   const size_t base = blockIdx.z * ((size_t)N * N * C::H) + (size_t)x * N * C::H + kz;   // + y * H
@@ -1283,7 +1287,7 @@ struct XNothing {
 };
 
 // One x-pass tile: kz block kzb (W consecutive kz), fixed ky, instance inst, all kx.
-// Thread tid = t * W + w; kx = elem(t, r).  v holds the tile's input (non-adjoint modes;
+// Thread (t, w) = (pencil_thread(), tid % W); kx = elem(t, r).  v holds the tile's input (non-adjoint modes;
 // the adjoint modes load their x-order groups here), sm is the tile's exchange buffer,
 // s_acc the per-warp accumulators (zeroed by the caller), blk the tile's linear index,
 // s_sc the tile of the scf field staged in shared memory (element (kx, w) at kx W + w), or
@@ -1292,11 +1296,11 @@ struct XNothing {
 // that have one there): every thread has read its shared-memory inputs and the table.
 template <int N, int MODE, bool SPLIT, class F = XNothing>
 __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[XCfg<N, MODE>::RMAX], int kzb, int ky, int inst,
-                                       size_t blk, const SmemCol<XCfg<N, MODE>::W>& sm, const float2* s_tw,
+                                       size_t blk, const SmemCol<XCfg<N, MODE>::W, XCfg<N, MODE>::PAIR>& sm, const float2* s_tw,
                                        double* s_acc, const float* s_sc = nullptr, XSmemIn si = {},
                                        F after_mult = F()) {
   using C = XCfg<N, MODE>;
-  const int w = threadIdx.x % C::W, t = threadIdx.x / C::W;
+  const int w = threadIdx.x % C::W, t = pencil_thread<N, C::V, C::W, C::PAIR>();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr int NWARP = C::XT / 32;
   const int kz = kzb * C::W + w;
@@ -1670,8 +1674,8 @@ __global__ void __launch_bounds__(XCfg<N, MODE>::XT, XCfg<N, MODE>::MINB) k_x(XA
   float2* s_tw = smem;
   load_twiddles(s_tw, a.tw, N);
   grid_sync();
-  const int w = threadIdx.x % C::W, t = threadIdx.x / C::W;
-  const SmemCol<C::W> sm{smem + N + w};
+  const int w = threadIdx.x % C::W, t = pencil_thread<N, C::V, C::W, C::PAIR>();
+  const SmemCol<C::W, C::PAIR> sm{smem + N + w};
   double* s_acc = reinterpret_cast<double*>(smem + N + N * C::W);   // per-warp accumulators
   constexpr int NWARP = C::XT / 32;
   if (MODE == X_PK) {
@@ -1740,7 +1744,7 @@ __global__ void __launch_bounds__(XCfg<N, MODE>::XT, XCfg<N, MODE>::MINB) k_x_tm
   double* s_acc = reinterpret_cast<double*>(xs_raw + Q::ACC_OFF);
   __shared__ int s_fail;
   constexpr int NWARP = C::XT / 32;
-  const int w = threadIdx.x % C::W, t = threadIdx.x / C::W;
+  const int w = threadIdx.x % C::W, t = pencil_thread<N, C::V, C::W, C::PAIR>();
   const int ntiles = Q::KZB * N * a.g.batch;
   auto issue = [&](int st, int tile) {   // one thread
     const int kzb = tile % Q::KZB, ky = (tile / Q::KZB) % N, inst = tile / (Q::KZB * N);
@@ -1787,7 +1791,7 @@ __global__ void __launch_bounds__(XCfg<N, MODE>::XT, XCfg<N, MODE>::MINB) k_x_tm
       return;
     }
     const int kzb = tile % Q::KZB, ky = (tile / Q::KZB) % N, inst = tile / (Q::KZB * N);
-    const SmemCol<C::W> sm{ring + st * Q::STAGE + w};
+    const SmemCol<C::W, C::PAIR> sm{ring + st * Q::STAGE + w};
     const float* s_sc = SC ? reinterpret_cast<const float*>(ring + st * Q::STAGE + Q::TILE) : nullptr;
     x_tile<N, MODE, !SC>(a, v, kzb, ky, inst, (size_t)tile, sm, s_tw, s_acc, s_sc);
     __syncthreads();   // ring stage and accumulators free
@@ -1830,7 +1834,7 @@ __global__ void __launch_bounds__(XCfg<N, MODE>::XT, XCfg<N, MODE>::MINB) k_x_tm
   uint64_t* bar = reinterpret_cast<uint64_t*>(xa_raw + Q::BAR_OFF);
   double* s_acc = reinterpret_cast<double*>(xa_raw + Q::ACC_OFF);
   __shared__ int s_fail;
-  const int w = threadIdx.x % C::W, t = threadIdx.x / C::W;
+  const int w = threadIdx.x % C::W, t = pencil_thread<N, C::V, C::W, C::PAIR>();
   const int ntiles = Q::KZB * N * a.g.batch;
   const int mine = blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
   const int nload = 4 * mine;
@@ -1901,7 +1905,7 @@ __global__ void __launch_bounds__(XCfg<N, MODE>::XT, XCfg<N, MODE>::MINB) k_x_tm
 #pragma unroll
         for (int r = 0; r < C::RMAX; ++r) sc[r] = __ldg(sp + (size_t)elem<N, C::V>(t, r) * ((size_t)N * C::H));
       }
-      fft<N, false, C::V>(u, t, SmemCol<C::W>{ring + st * Q::TILE + w}, s_tw);   // ends past its last shared read
+      fft<N, false, C::V>(u, t, SmemCol<C::W, C::PAIR>{ring + st * Q::TILE + w}, s_tw);   // ends past its last shared read
 #pragma unroll
       for (int r = 0; r < C::RMAX; ++r) v[r] = acc_dconj(v[r], u[r], a.g.kf * (float)mode_of(elem<N, C::V>(t, r), N), j);
       __syncthreads();   // every warp is past the transform: the stage is free
@@ -1942,7 +1946,7 @@ __global__ void __launch_bounds__(XCfg<N, MODE>::XT, XCfg<N, MODE>::MINB) k_x_tm
         for (int j = 0; j < 2 && issued < nload; ++j) issue();
       }
     };
-    x_tile<N, MODE, false>(a, v, kzb, ky, inst, (size_t)tile, SmemCol<C::W>{ex + w}, s_tw, s_acc, nullptr, si, refill);
+    x_tile<N, MODE, false>(a, v, kzb, ky, inst, (size_t)tile, SmemCol<C::W, C::PAIR>{ex + w}, s_tw, s_acc, nullptr, si, refill);
     __syncthreads();   // stages and accumulators free
     if (threadIdx.x == 0 && issued < nload) {
       fence_proxy_async_smem();
