@@ -37,22 +37,22 @@ __device__ __forceinline__ float2 mul_i(float2 a) { return make_float2(-a.y, a.x
 __device__ __forceinline__ float2 mul_mi(float2 a) { return make_float2(a.y, -a.x); }   // -i a
 
 // ------------------------------------------------------------ radix schedules
-// V = 0: mostly radix sequences with the same radix first and last (so that stage-0 input and
-// last-stage output share one element pattern); every radix divides RMAX.  N = 128 takes two stages
-// (16 values per thread): against 8-2-8 with 8 values, five output times x_source 80 -> 74 us and
-// x_pk 63 -> 53, the batch of 96 mixed grids 16.06 -> 15.82 ms.  N = 32 as 8-4 gains in the y passes and
-// shell sums and loses in the z passes.
+// V = 0: radix sequences with the same radix first and last (so that stage-0 input and
+// last-stage output share one element pattern); every radix divides RMAX.
 // V = 1 (where it exists): twice the values per thread and two stages, so one shared-memory
 // exchange per transform instead of two, half the twiddle loads and half the threads per
 // pencil: for passes that hold one array of values (registers).  fft() brings the outputs
-// back into the input's pattern (a renaming of registers).
+// back into the input's pattern (a renaming of registers).  N = 128 in all passes instead of 8-2-8 was
+// slower where passes follow one another without a pause: the batch of 96 mixed grids 16.69 ms, against
+// 15.50 with 8-2-8 and 15.40 with 16-8 in the y passes, the plain x passes, the source and the shell sums
+// only (five output times 445, 421 and 409 us).
 template <int N, int V = 0> struct Cfg;
 template <> struct Cfg<96>   { static constexpr int NS = 3, RMAX = 12; static __host__ __device__ constexpr int rad(int s) { return s == 1 ? 6 : 4; } };
 template <> struct Cfg<192>  { static constexpr int NS = 3, RMAX = 12; static __host__ __device__ constexpr int rad(int s) { return s == 1 ? 12 : 4; } };
 template <> struct Cfg<16>   { static constexpr int NS = 2, RMAX = 4;  static __host__ __device__ constexpr int rad(int s) { return 4; } };
 template <> struct Cfg<32>   { static constexpr int NS = 3, RMAX = 4;  static __host__ __device__ constexpr int rad(int s) { return s == 1 ? 2 : 4; } };
 template <> struct Cfg<64>   { static constexpr int NS = 2, RMAX = 8;  static __host__ __device__ constexpr int rad(int s) { return 8; } };
-template <> struct Cfg<128>  { static constexpr int NS = 2, RMAX = 16; static __host__ __device__ constexpr int rad(int s) { return s == 0 ? 16 : 8; } };
+template <> struct Cfg<128>  { static constexpr int NS = 3, RMAX = 8;  static __host__ __device__ constexpr int rad(int s) { return s == 1 ? 2 : 8; } };
 template <> struct Cfg<256>  { static constexpr int NS = 2, RMAX = 16; static __host__ __device__ constexpr int rad(int s) { return 16; } };
 #ifndef LPT2_R512
 #define LPT2_R512 16   // N = 512: radix 16-2-16 (16 values per thread) or 8-8-8 (8 values)
@@ -60,6 +60,7 @@ template <> struct Cfg<256>  { static constexpr int NS = 2, RMAX = 16; static __
 template <> struct Cfg<512>  { static constexpr int NS = 3, RMAX = LPT2_R512;
   static __host__ __device__ constexpr int rad(int s) { return LPT2_R512 == 8 ? 8 : (s == 1 ? 2 : 16); } };
 template <> struct Cfg<1024> { static constexpr int NS = 3, RMAX = 16; static __host__ __device__ constexpr int rad(int s) { return s == 1 ? 4 : 16; } };
+template <> struct Cfg<128, 1> { static constexpr int NS = 2, RMAX = 16; static __host__ __device__ constexpr int rad(int s) { return s == 0 ? 16 : 8; } };
 template <> struct Cfg<32, 1>  { static constexpr int NS = 2, RMAX = 8;  static __host__ __device__ constexpr int rad(int s) { return s == 0 ? 8 : 4; } };
 template <> struct Cfg<512, 1> { static constexpr int NS = 2, RMAX = 32; static __host__ __device__ constexpr int rad(int s) { return s == 0 ? 32 : 16; } };
 

@@ -57,13 +57,13 @@ template <int N> struct PassCfg {
 // wait for one another (y_phi 1399 us), with 32 values 256 threads and one exchange instead
 // of two: y_phi 1067 -> 930 us, y_psi 537 -> 463, y_fwd 215 -> 184 against 8 kz and 16
 // values.  N = 32 (8-4 instead of 4-2-4): 64 batched grids y_phi 19.1 -> 16.4 us, x_pk 13.1 -> 10.5, the
-// call 108.5 -> 104.7.  Two CTAs per SM at 512: a third fits in registers (80), but its tile takes the L1 the loads in
+// call 108.5 -> 104.7.  N = 128 (16-8): five output times 414 -> 409 us a call.  Two CTAs per SM at 512: a third fits in registers (80), but its tile takes the L1 the loads in
 // flight need (y_phi 1098 us).  Y_SUM keeps an accumulator beside the values: 8 kz, 16 values.
 enum YKind { Y_MULTI = 0, Y_SUM = 1, Y_ONE = 2 };
 template <int N, int KIND, int WY = 0> struct YCfg {
   static constexpr int H = N / 2;
   static constexpr int W = WY ? WY : (N == 512 ? (KIND == Y_SUM ? 8 : 16) : PassCfg<N>::W);
-  static constexpr int V = ((N == 512 && W == 16) || N == 32) && KIND != Y_SUM ? 1 : 0;
+  static constexpr int V = ((N == 512 && W == 16) || N == 128 || N == 32) && KIND != Y_SUM ? 1 : 0;
   static constexpr int RMAX = Cfg<N, V>::RMAX;
   static constexpr int TPP = N / RMAX;
   static constexpr int XT = TPP * W;
@@ -75,11 +75,13 @@ template <int N, int KIND, int WY = 0> struct YCfg {
 
 // x passes: the tile of a mode.  V = 1 as in the y passes (N = 512, modes that hold one array of
 // values): 16 kz and 32 values per thread, x_fwd 275 -> 185 us, x_inv 284 -> 182, x_pkadj 343 ->
-// 334.  Not the shell sums: they want the resident warps that 64 registers allow (250 us against
-// 275 with 32 values).
+// 334.  Not the shell sums there: they want the resident warps that 64 registers allow (250 us against
+// 275 with 32 values).  N = 128 (16 values): x_pk of five output times 63 -> 53 us, x_source 80 -> 74.
 template <int N, int MODE> struct XCfg {
-  static constexpr int V = (N == 512 && (MODE == X_FWD || MODE == X_INV || MODE == X_PKADJ || MODE == X_MUL)) ||
-                                   (N == 32 && (MODE == X_PKP || MODE == X_PKI)) ? 1 : 0;
+  static constexpr bool PLAIN = MODE == X_FWD || MODE == X_INV || MODE == X_PKADJ || MODE == X_MUL;
+  static constexpr bool SHELLS = MODE == X_PKP || MODE == X_PKI;
+  static constexpr int V = (N == 512 && PLAIN) || (N == 128 && (PLAIN || SHELLS || MODE == X_SOURCE)) ||
+                                   (N == 32 && SHELLS) ? 1 : 0;
   static constexpr int RMAX = Cfg<N, V>::RMAX;
   static constexpr int TPP = N / RMAX;
   static constexpr int H = N / 2;
