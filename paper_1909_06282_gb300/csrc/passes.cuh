@@ -1024,7 +1024,7 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_adj_source_ct
 // Tiles as in the field-pair layout: a ring stage holds the two fields of a pencil for the
 // CTA's eight rows, each row in its warp's padded region, used in place as the exchange row.  The
 // rows of g_S come with them: read from global memory where they are used, behind a
-// transform, they cost 250 us (512^3: 2005 -> 1754).  One tile per CTA: a persistent walk needs
+// transform, they cost 250 us (512^3: 2005 -> 1754; 1672 with the middle radix on shuffles).  One tile per CTA: a persistent walk needs
 // registers that spill (2654 us).
 #ifndef LPT2_ZADJ_FIELD_PAIRS
 #define LPT2_ZADJ_FIELD_PAIRS 1
@@ -1422,7 +1422,7 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[XCfg<N, MODE>
     // N), off by at most one, corrected against integer thresholds.  At most 32 x RMAX values per
     // shell and warp in FP32 (relative error below 4e-5 even when every rounding goes one way).
     // Measured (against a warp's two reductions for its patch's shells and a warp sum for each):
-    // x_pk at 512^3 329 -> 250 us, 96 batched instances 948 -> 700, 48 shells at 192^3 61 -> 48, 64^3
+    // x_pk at 512^3 329 -> 250 us (240 with the middle radix on shuffles), 96 batched instances 948 -> 700, 48 shells at 192^3 61 -> 48, 64^3
     // 12.3 -> 8.1 us.
     const float pnorm = a.g.box * a.g.box * a.g.box * a.g.inv_n3 * a.g.inv_n3;
     const int ns = a.n_shells;

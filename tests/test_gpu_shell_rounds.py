@@ -1,5 +1,5 @@
-"""Shell sums at the edges of the kernel's rounds: it holds 2 RMAX shells at a time (8 at 16 and
-32 cubed, 16 at 64 and 128 cubed, 24 at 96 cubed, 32 at 256 cubed), so counts of one round, one
+"""Shell sums at the edges of the kernel's rounds: it holds two shells per value of a thread (8 at
+16 cubed, 16 at 32 and 64 cubed, 24 at 96 cubed, 32 at 128 and 256 cubed), so counts of one round, one
 more, several, one shell, and the most, with shells wider and narrower than a mode.
 
 P(k) of seeded particles is compared with the shell means of |FFT|^2 in float64 of the density
@@ -13,8 +13,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("n, n_shells", [
-    (16, 1), (16, 8), (16, 9), (16, 256), (32, 7), (32, 8), (32, 17), (64, 16), (64, 33), (96, 24), (96, 25),
-    (96, 121), (128, 16), (128, 65), (192, 23), (256, 32), (256, 33), (256, 256),
+    (16, 1), (16, 8), (16, 9), (16, 256), (32, 7), (32, 8), (32, 16), (32, 17), (64, 16), (64, 33), (96, 24), (96, 25),
+    (96, 121), (128, 16), (128, 32), (128, 33), (128, 65), (192, 23), (256, 32), (256, 33), (256, 256),
 ])
 def test_shell_sums_at_round_edges(n, n_shells):
     import torch
