@@ -330,8 +330,11 @@ int lpt2_set_fr0(lpt2_plan_t plan, double fr0_abs);
  * a call that overwrites the kept state (lpt2_displace, lpt2_cic_pk with positions,
  * lpt2_displace_vjp itself, lpt2_set_fr0, lpt2_set_workspace, ...) makes the next adjoint
  * recompute the forward map.  Cotangents that are NULL cost nothing: without g_pk the P(k)
- * transpose is not run, and with g_pos alone neither are the forward's particles and deposit
- * (the density that lpt2_cic_pk(plan, NULL, ...) reads stays that of the last lpt2_displace).
+ * transpose is not run.  A recomputed forward map also deposits its density, which a following
+ * lpt2_cic_pk(plan, NULL, ...) then reads, with one exception: with g_pos alone, while the
+ * workspace holds the density of the last lpt2_displace (no other call has deposited one since,
+ * and the stream is not being captured), that density stays and the forward's particles and
+ * deposit are not run.
  *   noise      float[N^3] white noise, or NULL for the plan's Philox noise
  *   g_pos      float[3][N^3] dL/d(positions), or NULL (zero)
  *   g_density  float[N^3] dL/d(density contrast), or NULL (zero)

@@ -136,6 +136,9 @@ struct lpt2_plan_s {
   // positions and CIC density of lpt2_displace with noise `kept_noise`; spec = also the
   // density spectrum after the z and y passes (a later lpt2_cic_pk of that density)
   bool kept_fwd = false, kept_spec = false;
+  // the density in the workspace is that of an lpt2_displace that has been issued (not only
+  // captured) and that no later call has replaced
+  bool displaced_rho = false;
   const float* kept_noise = nullptr;
   int max_out;                // LPT2_MAX_OUTPUTS(n): room for n output times' tables in the workspace
   bool use_graph;
@@ -443,6 +446,17 @@ int displace_impl(lpt2_plan_t p, const float* noise, float* psi1, float* psi2, f
 void drop_state(lpt2_plan_t p) {
   p->kept_fwd = false;
   p->kept_spec = false;
+}
+
+// Whether the plan's stream is being captured: what the captured kernels will find in the
+// workspace when they run is then not known to the host.
+bool capturing(lpt2_plan_t p) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(p->stream, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return st != cudaStreamCaptureStatusNone;
 }
 
 // Forgets the output times (their tables live in the workspace).
@@ -890,6 +904,7 @@ int lpt2_set_workspace(lpt2_plan_t p, void* dev_ptr, size_t bytes) {
   if (!p || !dev_ptr) return fail(LPT2_EINVAL, "null argument");
   if (!aligned(dev_ptr, 256)) return fail(LPT2_EINVAL, "workspace must be 256-byte aligned");
   if (bytes < ws_need(p)) return fail(LPT2_ENOWORKSPACE, "workspace too small: %zu < %zu", bytes, ws_need(p));
+  p->displaced_rho = false;
   p->ws = (char*)dev_ptr;
   p->ws_bytes = bytes;
   // the sqrt(P N^3/V) field of every group (P(k) only: no later call changes it)
@@ -951,6 +966,7 @@ int lpt2_displace(lpt2_plan_t p, const float* noise, float* psi1, float* psi2, f
   if (rc) return rc;
   if (dk && !aligned(dk, 16)) return fail(LPT2_EINVAL, "dk must be 16-byte aligned");
   drop_state(p);
+  p->displaced_rho = false;
   // with LPT2_KEEP_STATE a forward to the CIC density only (no Psi, no positions out) also
   // keeps S(k) and the positions in the slots the adjoint reads them from
   const bool keep = p->keep_state && !psi1 && !psi2 && !pos;
@@ -974,6 +990,7 @@ int lpt2_displace(lpt2_plan_t p, const float* noise, float* psi1, float* psi2, f
   };
   const void* key[8] = {noise, psi1, psi2, pos, dk, p->ws, nullptr, nullptr};
   const int r = p->use_graph ? run_graph(p, 0, key, body) : body();
+  if (!r) p->displaced_rho = !capturing(p);
   if (!r && keep) {
     p->kept_fwd = true;
     p->kept_noise = noise;
@@ -1199,7 +1216,10 @@ int lpt2_cic_pk(lpt2_plan_t p, const float* pos, float* density, double* pk, dou
     rc = ensure_geometry(p, gi, n_shells);
     if (rc) return rc;
   }
-  if (pos) drop_state(p);   // a new deposit replaces the kept density
+  if (pos) {   // a new deposit replaces the kept density
+    drop_state(p);
+    p->displaced_rho = false;
+  }
   const void* key[8] = {pos, density, pk, k_mean, n_modes, p->ws, (const void*)(intptr_t)n_shells, nullptr};
   const int r = p->use_graph ? run_graph(p, 1, key, body) : body();
   if (!r && !pos && p->kept_fwd) p->kept_spec = true;   // slot A now holds the density spectrum
@@ -1225,6 +1245,7 @@ int lpt2_displace_host(lpt2_plan_t p, int n_real, const float* noise_h, int64_t 
   if (!p->host_io || !p->hio)
     return fail(LPT2_EINVAL, "lpt2_displace_host needs a plan made with the LPT2_HOST_IO flag (the workspace "
                              "then holds its two device buffer sets)");
+  p->displaced_rho = false;
   host_io_buffers(p);
   rc = ensure_geometry(p, 0, n_shells);
   if (rc) return rc;
@@ -1332,6 +1353,7 @@ int lpt2_displace_outputs(lpt2_plan_t p, const float* noise, float* pos, double*
   if (!pk) return fail(LPT2_EINVAL, "pk must not be null");
   if (n_shells < 1 || n_shells > kMaxShells) return fail(LPT2_EINVAL, "n_shells must be in [1, 256]");
   set_group(p, 0);
+  p->displaced_rho = false;
   rc = ensure_geometry(p, 0, n_shells);
   if (rc) return rc;
   const FwdSlots f = fwd_slots(p);
@@ -1435,6 +1457,7 @@ int lpt2_autotune(lpt2_plan_t p, int n_shells, int reps) {
     cleanup();
     return fail(LPT2_ECUDA, "autotune events: %s", cudaGetErrorString(e));
   }
+  p->displaced_rho = false;
   for (int gi = 0; gi < (int)p->groups.size() && !rc; ++gi) rc = ensure_geometry(p, gi, n_shells);
   drop_graphs(p);
   for (int gi = 0; gi < (int)p->groups.size() && !rc; ++gi) {
@@ -1509,6 +1532,7 @@ int lpt2_cic_pk_est(lpt2_plan_t p, const float* pos, float* density, double* pk,
   if (flags & ~(unsigned)(LPT2_PK_DECONVOLVE | LPT2_PK_INTERLACE)) return fail(LPT2_EINVAL, "unknown flags");
   const bool inter = flags & LPT2_PK_INTERLACE;
   if (inter && !pos) return fail(LPT2_EINVAL, "interlacing needs the positions (pos must not be null)");
+  if (pos) p->displaced_rho = false;
   for (int gi = 0; gi < (int)p->groups.size(); ++gi) {
     rc = ensure_geometry(p, gi, n_shells);
     if (rc) return rc;
@@ -1817,14 +1841,18 @@ int lpt2_displace_vjp(lpt2_plan_t p, const float* noise, const float* g_pos, con
   // the last lpt2_displace of a LPT2_KEEP_STATE plan left them for this noise; then the
   // delta_rho spectrum after the z and y passes, unless a later lpt2_cic_pk left it in slot A.
   // With a cotangent of the positions alone (g_density and g_pk null) nothing flows back through
-  // the density: neither the forward's particles and deposit nor the passes that carry the
-  // density cotangent are run (at 512^3 0.73 + 0.46 + 0.52 + 1.03 ms of forward passes for one x
-  // pass of 0.19, and 3.7 ms of adjoint passes whose results were zeros added to g_pos).
+  // the density, so the passes that carry its cotangent are not run (at 512^3 3.7 ms of passes
+  // whose results were zeros added to g_pos).  The forward's particles and deposit are then only
+  // for the density that a following lpt2_cic_pk(plan, NULL, ...) reads: where the workspace holds
+  // that of an lpt2_displace, which is the one that call is to read, one x pass of 0.19 ms takes
+  // the place of 0.73 + 0.46 + 0.52 + 1.03 ms.
   const bool via_density = g_density || g_pk || !g_pos;
   const bool reuse = p->keep_state && p->kept_fwd && p->kept_noise == noise;
   const bool reuse_spec = reuse && p->kept_spec;
+  const bool deposit = via_density || !p->displaced_rho || capturing(p);
   drop_state(p);   // this call overwrites the kept slots
-  if (!reuse && via_density) {
+  if (!reuse && deposit) {
+    p->displaced_rho = false;
     rc = displace_impl(p, noise, nullptr, nullptr, nullptr, nullptr, S[S_SHAT], pos);
     if (rc) return rc;
   } else if (!reuse) {   // delta(k), the phi_ij and S(k)
