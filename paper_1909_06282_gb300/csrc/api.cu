@@ -1867,6 +1867,9 @@ int lpt2_displace_vjp(lpt2_plan_t p, const float* noise, const float* g_pos, con
     xf.out[0] = S[S_SHAT];
     LAUNCH(p, "x_fwd", 8.0 * V3(p), x_pass(n, xf, p->stream));
   }
+  // made whatever the cotangents: a caller that captures later calls with these shells finds it
+  rc = ensure_geometry(p, 0, n_shells);
+  if (rc) return rc;
   YArgs yi{};
   yi.g = g;
   yi.tw = p->tw;
@@ -1887,8 +1890,6 @@ int lpt2_displace_vjp(lpt2_plan_t p, const float* noise, const float* g_pos, con
         if (rc) return rc;
       }
       // the P(k) transpose needs the mode count per shell (cached geometry), not P(k) itself
-      rc = ensure_geometry(p, 0, n_shells);
-      if (rc) return rc;
       static_assert(sizeof(unsigned long long) == sizeof(int64_t), "mode counts are 64-bit");
       const int64_t* nmodes = reinterpret_cast<const int64_t*>(p->groups[0].geo_n);
       const double v_over_n6 = p->box * p->box * p->box / (V3d * V3d);

@@ -101,3 +101,16 @@ def test_captured_adjoint_deposits():
         graph.replay()
         _same(_density(L, plan), _of(L, plan, noise[1]))
         s.synchronize()
+
+
+@pytest.mark.parametrize("cotangent", ["g_pos", "g_density"])
+def test_every_adjoint_makes_the_shell_geometry(cotangent):
+    """So that a P(k) call captured after it holds the estimator's kernels only."""
+    L, plan, noise, g_pos, _ = _case()
+    g = g_pos if cotangent == "g_pos" else g_pos[0].contiguous()
+    L.lpt2_displace_vjp(plan, noise=noise[0], n_shells=NS, **{cotangent: g})
+    count = [L.lpt2_launch_count(plan)]
+    for _ in range(2):
+        _density(L, plan)
+        count.append(L.lpt2_launch_count(plan))
+    assert count[1] - count[0] == count[2] - count[1]
