@@ -87,13 +87,30 @@ template <int N, int V = 0> __host__ __device__ constexpr int ns_before(int s) {
 // stages' ranges tile [ns_before(1), N).  A table in the order of the exponent puts the lanes
 // r entries apart, up to 16 to a bank (512^3: z_source 1257 -> 1141 us, z_adj_source 2223 ->
 // 1907 us, x_pkadj 438 -> 367 us by this order).  Returns the exponent m of exp(-2 pi i m / N).
-// (V = 1 of N = 512 starts its one twiddled stage at the same 32 points as V = 0's last.)
 template <int N> __host__ __device__ constexpr int twiddle_exponent(int i) {
   for (int s = 1; s < Cfg<N>::NS; ++s) {
     const int ns = ns_before<N>(s), R = Cfg<N>::rad(s);
     if (i >= ns && i < ns * R) return (i / ns) * (i % ns) * (N / (ns * R));
   }
   return 0;
+}
+
+// Whether schedule V reads its twiddles from that table, which is laid out for V = 0: each of its
+// twiddled stages starts after the same number of points, with the same radix, as one of V = 0's
+// (32-16 as 16-2-16, 16-8 as 8-2-8, 8-4 as 4-2-4; 32-16 not as 8-8-8).
+template <int N, int V> __host__ __device__ constexpr bool shares_twiddles() {
+  for (int s = 1; s < Cfg<N, V>::NS; ++s) {
+    bool found = false;
+    for (int u = 1; u < Cfg<N>::NS; ++u)
+      found = found || (ns_before<N>(u) == ns_before<N, V>(s) && Cfg<N>::rad(u) == Cfg<N, V>::rad(s));
+    if (!found) return false;
+  }
+  return true;
+}
+// Whether N has a two-stage schedule V = 1 that a pass may take.
+template <int N> __host__ __device__ constexpr bool two_stage() {
+  if constexpr (N == 32 || N == 128 || N == 512) return shares_twiddles<N, 1>();
+  else return false;
 }
 
 // ------------------------------------------------------- in-register DFTs
@@ -250,6 +267,7 @@ template <int N, bool INV, int S, int V, class SM>
 __device__ __forceinline__ void fft_stages(float2 (&v)[Cfg<N, V>::RMAX], int t, const SM& sm,
                                            const float2* __restrict__ tw) {
   using C = Cfg<N, V>;
+  static_assert(shares_twiddles<N, V>(), "the twiddle table has no entries in this schedule's order");
   constexpr int RMAX = C::RMAX;
   constexpr int TPP = N / RMAX;
   constexpr int R = C::rad(S);

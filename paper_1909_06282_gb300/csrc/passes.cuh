@@ -62,8 +62,9 @@ template <int N> struct PassCfg {
 enum YKind { Y_MULTI = 0, Y_SUM = 1, Y_ONE = 2 };
 template <int N, int KIND, int WY = 0> struct YCfg {
   static constexpr int H = N / 2;
-  static constexpr int W = WY ? WY : (N == 512 ? (KIND == Y_SUM ? 8 : 16) : PassCfg<N>::W);
-  static constexpr int V = ((N == 512 && W == 16) || N == 128 || N == 32) && KIND != Y_SUM ? 1 : 0;
+  static constexpr bool TWO = two_stage<N>() && KIND != Y_SUM;
+  static constexpr int W = WY ? WY : (N == 512 && TWO ? 16 : PassCfg<N>::W);
+  static constexpr int V = TWO && (N != 512 || W == 16) ? 1 : 0;
   static constexpr int RMAX = Cfg<N, V>::RMAX;
   static constexpr int TPP = N / RMAX;
   static constexpr int XT = TPP * W;
@@ -80,8 +81,8 @@ template <int N, int KIND, int WY = 0> struct YCfg {
 template <int N, int MODE> struct XCfg {
   static constexpr bool PLAIN = MODE == X_FWD || MODE == X_INV || MODE == X_PKADJ || MODE == X_MUL;
   static constexpr bool SHELLS = MODE == X_PKP || MODE == X_PKI;
-  static constexpr int V = (N == 512 && PLAIN) || (N == 128 && (PLAIN || SHELLS || MODE == X_SOURCE)) ||
-                                   (N == 32 && SHELLS) ? 1 : 0;
+  static constexpr int V = two_stage<N>() && ((N == 512 && PLAIN) || (N == 32 && SHELLS) ||
+                                              (N == 128 && (PLAIN || SHELLS || MODE == X_SOURCE))) ? 1 : 0;
   static constexpr int RMAX = Cfg<N, V>::RMAX;
   static constexpr int TPP = N / RMAX;
   static constexpr int H = N / 2;
