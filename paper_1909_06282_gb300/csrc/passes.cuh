@@ -336,7 +336,8 @@ template <int N> struct ZGrp {
   static constexpr int SMEM = BAR_OFF + GROUPS * 16;
   static constexpr int TILES = N * N / ROWS;                                       // per instance
   static_assert(STAGE_BYTES % 16 == 0 && BAR_OFF % 8 == 0 && RING_OFF % 2 == 0, "bulk copies need 16-byte alignment");
-  static_assert(C::ZT % GT == 0 && GROUPS < 15 && (N * N) % ROWS == 0, "groups must tile the CTA and the rows");
+  static_assert(C::ZT % GT == 0 && (N * N) % ROWS == 0, "groups must tile the CTA and the rows");
+  static_assert(GT == 32 || GROUPS <= 15, "a group of several warps has a named barrier of its own");
 };
 
 // The copy ring of one group: NF copies per tile, in the order the kernel consumes them; src(f,

@@ -31,7 +31,14 @@ template <int N, int KIND> void y() {
   twiddles<N, YCfg<N, KIND, 8>::V>("y twiddles");
   if constexpr (N >= 32) twiddles<N, YCfg<N, KIND, 16>::V>("y twiddles");
 }
+// the z passes' groups exist and fit on an SM (227 KB); named barriers are 0 .. 15
+template <int N> void z() {
+  using Q = ZGrp<N>;
+  if (Q::SMEM > 232448) fail("z group memory", N, Q::SMEM, 0);
+  if (Q::GT > 32 && Q::GROUPS > 15) fail("z group barriers", N, Q::GT, Q::GROUPS);
+}
 template <int N> void all() {
+  z<N>();
   twiddles<N, 0>("z twiddles");
   y<N, Y_MULTI>(); y<N, Y_SUM>(); y<N, Y_ONE>();
   x<N, X_FWD>(); x<N, X_INV>(); x<N, X_MUL>(); x<N, X_DELTA>(); x<N, X_SOURCE>(); x<N, X_PK>(); x<N, X_PKP>();
@@ -44,7 +51,7 @@ int main() {
 """
 
 
-@pytest.mark.parametrize("setting", ["", "-DLPT2_R512=8", "-DLPT2_W512=16"])
+@pytest.mark.parametrize("setting", ["", "-DLPT2_R512=8", "-DLPT2_W512=16", "-DLPT2_ZTHREADS=128", "-DLPT2_ZTHREADS=512"])
 def test_pass_configurations(setting, tmp_path):
     from paper_1909_06282_gb300 import build as B
 
