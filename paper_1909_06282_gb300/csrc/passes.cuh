@@ -78,10 +78,11 @@ template <int N, int KIND, int WY = 0> struct YCfg {
 // values): 16 kz and 32 values per thread, x_fwd 275 -> 185 us, x_inv 284 -> 182, x_pkadj 343 ->
 // 334.  Not the shell sums there: they want the resident warps that 64 registers allow (250 us against
 // 275 with 32 values).  N = 128 (16 values): x_pk of five output times 63 -> 53 us, x_source 80 -> 74.
+// N = 32 (4 threads a pencil): where 8 pencils or more make whole warps.
 template <int N, int MODE> struct XCfg {
   static constexpr bool PLAIN = MODE == X_FWD || MODE == X_INV || MODE == X_PKADJ || MODE == X_MUL;
   static constexpr bool SHELLS = MODE == X_PKP || MODE == X_PKI;
-  static constexpr int V = two_stage<N>() && ((N == 512 && PLAIN) || (N == 32 && SHELLS) ||
+  static constexpr int V = two_stage<N>() && ((N == 512 && PLAIN) || (N == 32 && SHELLS && PassCfg<N>::W >= 8) ||
                                               (N == 128 && (PLAIN || SHELLS || MODE == X_SOURCE))) ? 1 : 0;
   static constexpr int RMAX = Cfg<N, V>::RMAX;
   static constexpr int TPP = N / RMAX;

@@ -25,7 +25,16 @@ template <int N, int V> void twiddles(const char* pass) {
         if (twiddle_exponent<N>(r * ns + j) != r * j * (N / (ns * R))) return fail(pass, N, s, r * ns + j);
   }
 }
-template <int N, int MODE> void x() { twiddles<N, XCfg<N, MODE>::V>("x twiddles"); }
+template <int N, int MODE> void x() {
+  using C = XCfg<N, MODE>;
+  twiddles<N, C::V>("x twiddles");
+  // the sums over modes go by whole warps, a power of two of them in the shell sums
+  const bool shells = MODE == X_PKP || MODE == X_PKI;
+  if (shells || MODE == X_PK || MODE == X_ADJ_SOURCE) {
+    const int nwarp = C::XT / 32;
+    if (C::XT % 32 || nwarp < 1 || (shells && (nwarp & (nwarp - 1)))) fail("x warps", N, MODE, C::XT);
+  }
+}
 template <int N, int KIND> void y() {
   twiddles<N, YCfg<N, KIND>::V>("y twiddles");
   twiddles<N, YCfg<N, KIND, 8>::V>("y twiddles");
@@ -51,7 +60,8 @@ int main() {
 """
 
 
-@pytest.mark.parametrize("setting", ["", "-DLPT2_R512=8", "-DLPT2_W512=16", "-DLPT2_ZTHREADS=128", "-DLPT2_ZTHREADS=512"])
+@pytest.mark.parametrize("setting", ["", "-DLPT2_R512=8", "-DLPT2_W512=16", "-DLPT2_WSMALL=4", "-DLPT2_WSMALL=8",
+                                     "-DLPT2_ZTHREADS=128", "-DLPT2_ZTHREADS=512"])
 def test_pass_configurations(setting, tmp_path):
     from paper_1909_06282_gb300 import build as B
 
