@@ -8,9 +8,9 @@ namespace lpt2 {
 
 // Periodic cloud-in-cell deposit of unit-mass particles (Sec. 4 density),
 // Lagrangian-tile form.  A CTA takes the CIC_T^3 particles of one block of
-// Lagrangian cells.  Their positions mostly stay within H cells of the block,
+// Lagrangian cells.  Their positions mostly stay within CIC_H cells of the block,
 // so the CTA sums the eight weights of each such particle in a shared-memory window
-// (the block grown by H cells on every side, by a 4-aligned CIC_HZ below in z)
+// (the block grown by CIC_H cells on every side, by a 4-aligned CIC_HZ below in z)
 // and then adds the window to the density with one 16-byte vector reduction per
 // non-zero group of four cells: about one L2 reduction per particle instead of the
 // five of a direct deposit, whose rate the L2 request throughput limits.  Window
@@ -22,23 +22,16 @@ namespace lpt2 {
 #define LPT2_CIC_MINB 2   // resident CIC CTAs per SM: register cap (3 fit in shared memory but spill)
 #endif
 namespace {
-constexpr int CIC_T = 16, CIC_HZ = 4;
-// window of a block with a halo of H cells.  The deposit takes 5: a particle outside the window
-// costs up to eight scattered L2 reductions, a cell of window a clear and a sum (512^3 at 2 Mpc/h
-// cells: H = 4 1030 us, 5 991, 6 1014; 96 batched instances at 4 Mpc/h 2091 -> 2057; a third CTA per
-// SM does not fit either way).  The gather, whose window loads cost more than a stray particle, 4
-// (1594 us against 1613).
-template <int HALO> struct CicWindow {
-  static constexpr int H = HALO;
-  static constexpr int E = CIC_T + 2 * H + 1;                        // window cells along x and y
-  static constexpr int EZ = (CIC_T + CIC_HZ + H + 1 + 3) / 4 * 4;    // along z, whole groups of 4
-  static constexpr int QZ = EZ / 4;
-  static constexpr int SMEM = E * E * EZ * 4;
-};
-using CicDeposit = CicWindow<5>;
-using CicGather = CicWindow<4>;
+// Four cells of halo: five make the deposit 4 % faster (512^3: 1030 -> 991 us) but round the FP32
+// weights of the particles between the two to the window's 2^-19 (interlaced P(k) at 192^3 2.80e-6
+// -> 2.83e-6 from float64); the gather is slower with five (1594 -> 1613).
+constexpr int CIC_T = 16, CIC_H = 4, CIC_HZ = 4;
+constexpr int CIC_E = CIC_T + 2 * CIC_H + 1;                        // window cells along x and y
+constexpr int CIC_EZ = (CIC_T + CIC_HZ + CIC_H + 1 + 3) / 4 * 4;    // along z, whole groups of 4
+constexpr int CIC_QZ = CIC_EZ / 4;
 constexpr int CIC_THREADS = 512;
 constexpr int CIC_PER = CIC_T * CIC_T * CIC_T / CIC_THREADS;         // particles per thread
+constexpr int CIC_SMEM = CIC_E * CIC_E * CIC_EZ * 4;
 constexpr float CIC_SCALE = 524288.0f;                              // 2^19
 static_assert(CIC_HZ % 4 == 0 && CIC_T % 4 == 0, "window groups of four must align with the grid's");
 static_assert(CIC_T * CIC_T * CIC_T < (1 << 13), "window sums must stay below 2^32 / 2^19");
@@ -51,17 +44,16 @@ __device__ __forceinline__ int wrap_cell(int i) {   // i in (-N, 2N) -> [0, N)
 
 template <int N>
 __global__ void __launch_bounds__(CIC_THREADS, LPT2_CIC_MINB) k_cic(CicArgs a) {
-  using W = CicDeposit;
   static_assert(N % CIC_T == 0 && N % 4 == 0, "grid side must be a multiple of the tile");
-  extern __shared__ __align__(16) unsigned int win[];   // [W::E][W::E][W::EZ]
+  extern __shared__ __align__(16) unsigned int win[];   // [CIC_E][CIC_E][CIC_EZ]
   const size_t n3 = (size_t)N * N * N;
   a.pos += (size_t)blockIdx.y * 3 * n3;   // instance blockIdx.y
   a.rho += (size_t)blockIdx.y * n3;
   constexpr int NT = N / CIC_T;
   const int b = blockIdx.x;
   const int x0 = (b / (NT * NT)) * CIC_T, y0 = ((b / NT) % NT) * CIC_T, z0 = (b % NT) * CIC_T;
-  const int ox = x0 - W::H, oy = y0 - W::H, oz = z0 - CIC_HZ;   // window origin (may be < 0)
-  const bool wraps = ox < 0 || oy < 0 || oz < 0 || ox + W::E > N || oy + W::E > N || oz + W::EZ > N;
+  const int ox = x0 - CIC_H, oy = y0 - CIC_H, oz = z0 - CIC_HZ;   // window origin (may be < 0)
+  const bool wraps = ox < 0 || oy < 0 || oz < 0 || ox + CIC_E > N || oy + CIC_E > N || oz + CIC_EZ > N;
   grid_sync();
   // all position loads of this thread first: their latency overlaps the zeroing
   float u[CIC_PER][3];
@@ -73,7 +65,7 @@ __global__ void __launch_bounds__(CIC_THREADS, LPT2_CIC_MINB) k_cic(CicArgs a) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) u[k][c] = __ldg(a.pos + c * n3 + e);
   }
-  for (int i = threadIdx.x; i < W::E * W::E * W::QZ; i += blockDim.x)
+  for (int i = threadIdx.x; i < CIC_E * CIC_E * CIC_QZ; i += blockDim.x)
     reinterpret_cast<uint4*>(win)[i] = make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();
 #pragma unroll
@@ -90,41 +82,41 @@ __global__ void __launch_bounds__(CIC_THREADS, LPT2_CIC_MINB) k_cic(CicArgs a) {
       ry = wrap_cell<N>(ry);
       rz = wrap_cell<N>(rz);
     }
-    if ((unsigned)rx < W::E - 1 && (unsigned)ry < W::E - 1 && (unsigned)rz < W::EZ - 1) {
+    if ((unsigned)rx < CIC_E - 1 && (unsigned)ry < CIC_E - 1 && (unsigned)rz < CIC_EZ - 1) {
       const float dx = ux - fx, dy = uy - fy, dz = uz - fz;   // exact
       const float wx0 = 1.f - dx, wy0 = 1.f - dy, wz0 = 1.f - dz;
-      unsigned int* c = win + (rx * W::E + ry) * W::EZ + rz;
+      unsigned int* c = win + (rx * CIC_E + ry) * CIC_EZ + rz;
       float w = wx0 * wy0;
       atomicAdd(c, __float2uint_rn(w * wz0 * CIC_SCALE));
       atomicAdd(c + 1, __float2uint_rn(w * dz * CIC_SCALE));
       w = wx0 * dy;
-      atomicAdd(c + W::EZ, __float2uint_rn(w * wz0 * CIC_SCALE));
-      atomicAdd(c + W::EZ + 1, __float2uint_rn(w * dz * CIC_SCALE));
+      atomicAdd(c + CIC_EZ, __float2uint_rn(w * wz0 * CIC_SCALE));
+      atomicAdd(c + CIC_EZ + 1, __float2uint_rn(w * dz * CIC_SCALE));
       w = dx * wy0;
-      atomicAdd(c + W::E * W::EZ, __float2uint_rn(w * wz0 * CIC_SCALE));
-      atomicAdd(c + W::E * W::EZ + 1, __float2uint_rn(w * dz * CIC_SCALE));
+      atomicAdd(c + CIC_E * CIC_EZ, __float2uint_rn(w * wz0 * CIC_SCALE));
+      atomicAdd(c + CIC_E * CIC_EZ + 1, __float2uint_rn(w * dz * CIC_SCALE));
       w = dx * dy;
-      atomicAdd(c + W::E * W::EZ + W::EZ, __float2uint_rn(w * wz0 * CIC_SCALE));
-      atomicAdd(c + W::E * W::EZ + W::EZ + 1, __float2uint_rn(w * dz * CIC_SCALE));
+      atomicAdd(c + CIC_E * CIC_EZ + CIC_EZ, __float2uint_rn(w * wz0 * CIC_SCALE));
+      atomicAdd(c + CIC_E * CIC_EZ + CIC_EZ + 1, __float2uint_rn(w * dz * CIC_SCALE));
     } else {
       cic_deposit_vec<N>(a.rho, ux, uy, uz);
     }
   }
   __syncthreads();
   const float inv_scale = 1.0f / CIC_SCALE;
-  // group q = (wx * W::E + wy) * W::QZ + qz, advanced by the CTA size without divisions
-  static_assert(CIC_THREADS / W::QZ / W::E < W::E, "flush stride must advance wx by less than a window");
-  constexpr int SQZ = CIC_THREADS % W::QZ, SR = CIC_THREADS / W::QZ;   // stride in (qz, row)
-  constexpr int SWY = SR % W::E, SWX = SR / W::E;                      // row stride in (wy, wx)
-  int qz = threadIdx.x % W::QZ, wy = (threadIdx.x / W::QZ) % W::E, wx = threadIdx.x / W::QZ / W::E;
-  for (int q = threadIdx.x; q < W::E * W::E * W::QZ; q += blockDim.x) {
+  // group q = (wx * CIC_E + wy) * CIC_QZ + qz, advanced by the CTA size without divisions
+  static_assert(CIC_THREADS / CIC_QZ / CIC_E < CIC_E, "flush stride must advance wx by less than a window");
+  constexpr int SQZ = CIC_THREADS % CIC_QZ, SR = CIC_THREADS / CIC_QZ;   // stride in (qz, row)
+  constexpr int SWY = SR % CIC_E, SWX = SR / CIC_E;                      // row stride in (wy, wx)
+  int qz = threadIdx.x % CIC_QZ, wy = (threadIdx.x / CIC_QZ) % CIC_E, wx = threadIdx.x / CIC_QZ / CIC_E;
+  for (int q = threadIdx.x; q < CIC_E * CIC_E * CIC_QZ; q += blockDim.x) {
     const uint4 iv = reinterpret_cast<const uint4*>(win)[q];
     const int cz = qz, cy = wy, cx = wx;
     qz += SQZ;
     wy += SWY;
     wx += SWX;
-    if (qz >= W::QZ) { qz -= W::QZ; ++wy; }
-    if (wy >= W::E) { wy -= W::E; ++wx; }
+    if (qz >= CIC_QZ) { qz -= CIC_QZ; ++wy; }
+    if (wy >= CIC_E) { wy -= CIC_E; ++wx; }
     if ((iv.x | iv.y | iv.z | iv.w) == 0u) continue;
     int gx = ox + cx, gy = oy + cy, gz = oz + 4 * cz;   // gz a multiple of 4: the group never straddles the wrap
     if (wraps) {
@@ -146,15 +138,14 @@ __global__ void __launch_bounds__(CIC_THREADS, LPT2_CIC_MINB) k_cic(CicArgs a) {
 // three components go to real fields at the particle's Lagrangian cell.
 template <int N>
 __global__ void __launch_bounds__(CIC_THREADS, LPT2_CIC_MINB) k_cic_grad(CicGradArgs a) {
-  using W = CicGather;
   static_assert(N % CIC_T == 0 && N % 4 == 0, "grid side must be a multiple of the tile");
-  extern __shared__ __align__(16) float gw[];   // [W::E][W::E][W::EZ]
+  extern __shared__ __align__(16) float gw[];   // [CIC_E][CIC_E][CIC_EZ]
   const size_t n3 = (size_t)N * N * N;
   constexpr int NT = N / CIC_T;
   const int b = blockIdx.x;
   const int x0 = (b / (NT * NT)) * CIC_T, y0 = ((b / NT) % NT) * CIC_T, z0 = (b % NT) * CIC_T;
-  const int ox = x0 - W::H, oy = y0 - W::H, oz = z0 - CIC_HZ;
-  const bool wraps = ox < 0 || oy < 0 || oz < 0 || ox + W::E > N || oy + W::E > N || oz + W::EZ > N;
+  const int ox = x0 - CIC_H, oy = y0 - CIC_H, oz = z0 - CIC_HZ;
+  const bool wraps = ox < 0 || oy < 0 || oz < 0 || ox + CIC_E > N || oy + CIC_E > N || oz + CIC_EZ > N;
   grid_sync();
   float u[CIC_PER][3];
 #pragma unroll
@@ -165,17 +156,17 @@ __global__ void __launch_bounds__(CIC_THREADS, LPT2_CIC_MINB) k_cic_grad(CicGrad
 #pragma unroll
     for (int c = 0; c < 3; ++c) u[k][c] = __ldg(a.pos + c * n3 + e);
   }
-  // group q = (wx * W::E + wy) * W::QZ + qz, advanced by the CTA size without divisions
-  constexpr int SQZ = CIC_THREADS % W::QZ, SR = CIC_THREADS / W::QZ;
-  constexpr int SWY = SR % W::E, SWX = SR / W::E;
-  int qz = threadIdx.x % W::QZ, wy = (threadIdx.x / W::QZ) % W::E, wx = threadIdx.x / W::QZ / W::E;
-  for (int q = threadIdx.x; q < W::E * W::E * W::QZ; q += blockDim.x) {
+  // group q = (wx * CIC_E + wy) * CIC_QZ + qz, advanced by the CTA size without divisions
+  constexpr int SQZ = CIC_THREADS % CIC_QZ, SR = CIC_THREADS / CIC_QZ;
+  constexpr int SWY = SR % CIC_E, SWX = SR / CIC_E;
+  int qz = threadIdx.x % CIC_QZ, wy = (threadIdx.x / CIC_QZ) % CIC_E, wx = threadIdx.x / CIC_QZ / CIC_E;
+  for (int q = threadIdx.x; q < CIC_E * CIC_E * CIC_QZ; q += blockDim.x) {
     int gx = ox + wx, gy = oy + wy, gz = oz + 4 * qz;   // gz a multiple of 4
     qz += SQZ;
     wy += SWY;
     wx += SWX;
-    if (qz >= W::QZ) { qz -= W::QZ; ++wy; }
-    if (wy >= W::E) { wy -= W::E; ++wx; }
+    if (qz >= CIC_QZ) { qz -= CIC_QZ; ++wy; }
+    if (wy >= CIC_E) { wy -= CIC_E; ++wx; }
     if (wraps) {
       gx = wrap_cell<N>(gx);
       gy = wrap_cell<N>(gy);
@@ -199,10 +190,10 @@ __global__ void __launch_bounds__(CIC_THREADS, LPT2_CIC_MINB) k_cic_grad(CicGrad
       rz = wrap_cell<N>(rz);
     }
     float gxv, gyv, gzv;
-    if ((unsigned)rx < W::E - 1 && (unsigned)ry < W::E - 1 && (unsigned)rz < W::EZ - 1) {
+    if ((unsigned)rx < CIC_E - 1 && (unsigned)ry < CIC_E - 1 && (unsigned)rz < CIC_EZ - 1) {
       const float dx = ux - fx, dy = uy - fy, dz = uz - fz;
       const float wx[2] = {1.f - dx, dx}, wy[2] = {1.f - dy, dy}, wz[2] = {1.f - dz, dz};
-      const float* c = gw + (rx * W::E + ry) * W::EZ + rz;
+      const float* c = gw + (rx * CIC_E + ry) * CIC_EZ + rz;
       float ax = 0.f, ay = 0.f, az = 0.f;
 #pragma unroll
       for (int cx = 0; cx < 2; ++cx)
@@ -210,7 +201,7 @@ __global__ void __launch_bounds__(CIC_THREADS, LPT2_CIC_MINB) k_cic_grad(CicGrad
         for (int cy = 0; cy < 2; ++cy)
 #pragma unroll
           for (int cz = 0; cz < 2; ++cz) {
-            const float gc = c[(cx * W::E + cy) * W::EZ + cz];
+            const float gc = c[(cx * CIC_E + cy) * CIC_EZ + cz];
             const float sx = cx ? 1.f : -1.f, sy = cy ? 1.f : -1.f, sz = cz ? 1.f : -1.f;
             ax = fmaf(gc * sx, wy[cy] * wz[cz], ax);
             ay = fmaf(gc * sy, wx[cx] * wz[cz], ay);
@@ -235,8 +226,8 @@ __global__ void __launch_bounds__(CIC_THREADS, LPT2_CIC_MINB) k_cic_grad(CicGrad
 
 template <int N>
 cudaError_t launch_cic_grad_n(const CicGradArgs& a, cudaStream_t s) {
-  cudaFuncSetAttribute(k_cic_grad<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, CicGather::SMEM);
-  return launch_overlapped(k_cic_grad<N>, (unsigned)((N / CIC_T) * (N / CIC_T) * (N / CIC_T)), CIC_THREADS, CicGather::SMEM, s, a);
+  cudaFuncSetAttribute(k_cic_grad<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, CIC_SMEM);
+  return launch_overlapped(k_cic_grad<N>, (unsigned)((N / CIC_T) * (N / CIC_T) * (N / CIC_T)), CIC_THREADS, CIC_SMEM, s, a);
 }
 
 cudaError_t launch_cic_grad(const CicGradArgs& a, cudaStream_t s) {
@@ -257,9 +248,9 @@ cudaError_t launch_cic_grad(const CicGradArgs& a, cudaStream_t s) {
 
 template <int N>
 cudaError_t launch_cic_n(const CicArgs& a, cudaStream_t s) {
-  cudaFuncSetAttribute(k_cic<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, CicDeposit::SMEM);
+  cudaFuncSetAttribute(k_cic<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, CIC_SMEM);
   const dim3 blocks((unsigned)((N / CIC_T) * (N / CIC_T) * (N / CIC_T)), a.g.batch);
-  return launch_overlapped(k_cic<N>, blocks, CIC_THREADS, CicDeposit::SMEM, s, a);
+  return launch_overlapped(k_cic<N>, blocks, CIC_THREADS, CIC_SMEM, s, a);
 }
 
 cudaError_t launch_cic(const CicArgs& a, cudaStream_t s) {
