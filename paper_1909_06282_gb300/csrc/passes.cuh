@@ -1265,6 +1265,13 @@ __device__ __forceinline__ float warp_sum(float x) {
   return x;
 }
 
+// Sum of the N (a power of two) values row[(j + rot) & 31], j = first .. first + N - 1, by a tree:
+// each value passes through log2(N) roundings, not up to N - 1 as in a chain.
+template <int N> __host__ __device__ __forceinline__ float tree_sum(const float* row, int rot, int first = 0) {
+  if constexpr (N == 1) return row[(first + rot) & 31];
+  else return tree_sum<N / 2>(row, rot, first) + tree_sum<N / 2>(row, rot, first + N / 2);
+}
+
 // Shell of |n|^2 = n2 by the thresholds (ns for n2 >= (N/2)^2): a float estimate of floor(2 ns |n| /
 // N), off by at most one, corrected by integer comparisons.
 __device__ __forceinline__ int shell_below(int n2, const int* thr, int ns, float n) {
@@ -1419,11 +1426,11 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[XCfg<N, MODE>
     // V |delta|^2 / N^6 of its modes to a column of its own in the exchange buffer, which is free
     // after the transform: [warp][shell][lane], no two lanes in one bank, no atomics, and no
     // assumption on how many shells neighbouring modes span.  It holds 2 RMAX shells; more take
-    // several rounds.  Then a thread per (shell, warp) sums the 32 lanes, and FP64 sums the
+    // several rounds.  Then a thread per (shell, warp) sums the 32 lanes by a tree, and FP64 sums the
     // warps (a fixed tree over NWARP lanes, spread over the CTA's warps: a conversion or addition
     // holds an FP64 unit for 64 cycles).  The shell of a mode is a float estimate of floor(2 ns |n| /
-    // N), off by at most one, corrected against integer thresholds.  At most 32 x RMAX values per
-    // shell and warp in FP32 (relative error below 4e-5 even when every rounding goes one way).
+    // N), off by at most one, corrected against integer thresholds.  A value passes through at most
+    // RMAX + 5 FP32 additions (relative error below 21 x 2^-24 even when every rounding goes one way).
     // Measured (against a warp's two reductions for its patch's shells and a warp sum for each):
     // x_pk at 512^3 329 -> 250 us (240 with the middle radix on shuffles), 96 batched instances 948 -> 700, 48 shells at 192^3 61 -> 48, 64^3
     // 12.3 -> 8.1 us.
@@ -1459,11 +1466,7 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[XCfg<N, MODE>
       for (int i0 = 0; i0 < S * NWARP; i0 += C::XT) {
         const int i = i0 + threadIdx.x, b = i / NWARP, wi = i % NWARP;
         float lanes = 0.f;
-        if (b < S && b0 + b < ns) {
-          const float* row = hist + (wi * S + b) * 32;
-#pragma unroll
-          for (int j = 0; j < 32; ++j) lanes += row[(j + lane) & 31];
-        }
+        if (b < S && b0 + b < ns) lanes = tree_sum<32>(hist + (wi * S + b) * 32, lane);
         double acc = (double)lanes;
 #pragma unroll
         for (int o = NWARP / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
