@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(CIC_THREADS, LPT2_CIC_MINB) k_cic(CicArgs a) {
     const int i = p / (CIC_T * CIC_T), j = (p / CIC_T) % CIC_T, l = p % CIC_T;
     const size_t e = ((size_t)(x0 + i) * N + (y0 + j)) * N + (z0 + l);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) u[k][c] = __ldg(a.pos + c * n3 + e);
+    for (int c = 0; c < 3; ++c) u[k][c] = a.pos[c * n3 + e];
   }
   for (int i = threadIdx.x; i < CIC_E * CIC_E * CIC_QZ; i += blockDim.x)
     reinterpret_cast<uint4*>(win)[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(CIC_THREADS, LPT2_CIC_MINB) k_cic_grad(CicGrad
     const int i = p / (CIC_T * CIC_T), j = (p / CIC_T) % CIC_T, l = p % CIC_T;
     const size_t e = ((size_t)(x0 + i) * N + (y0 + j)) * N + (z0 + l);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) u[k][c] = __ldg(a.pos + c * n3 + e);
+    for (int c = 0; c < 3; ++c) u[k][c] = a.pos[c * n3 + e];
   }
   // group q = (wx * CIC_E + wy) * CIC_QZ + qz, advanced by the CTA size without divisions
   constexpr int SQZ = CIC_THREADS % CIC_QZ, SR = CIC_THREADS / CIC_QZ;
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(CIC_THREADS, LPT2_CIC_MINB) k_cic_grad(CicGrad
       gy = wrap_cell<N>(gy);
       gz = wrap_cell<N>(gz);
     }
-    reinterpret_cast<float4*>(gw)[q] = __ldg(reinterpret_cast<const float4*>(a.grho + ((size_t)gx * N + gy) * N + gz));
+    reinterpret_cast<float4*>(gw)[q] = *reinterpret_cast<const float4*>(a.grho + ((size_t)gx * N + gy) * N + gz);
   }
   __syncthreads();
   const float ic = a.g.inv_cell;
@@ -181,6 +181,11 @@ __global__ void __launch_bounds__(CIC_THREADS, LPT2_CIC_MINB) k_cic_grad(CicGrad
     const int p = threadIdx.x + k * CIC_THREADS;
     const int i = p / (CIC_T * CIC_T), j = (p / CIC_T) % CIC_T, l = p % CIC_T;
     const size_t e = ((size_t)(x0 + i) * N + (y0 + j)) * N + (z0 + l);
+    float gp[3];   // read before the gather, whose latency covers this one's
+    if (a.gpos) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) gp[c] = a.gpos[c * n3 + e];
+    }
     const float ux = wrapN<N>(u[k][0] * ic), uy = wrapN<N>(u[k][1] * ic), uz = wrapN<N>(u[k][2] * ic);
     const float fx = floorf(ux), fy = floorf(uy), fz = floorf(uz);
     int rx = (int)fx - ox, ry = (int)fy - oy, rz = (int)fz - oz;
@@ -214,9 +219,9 @@ __global__ void __launch_bounds__(CIC_THREADS, LPT2_CIC_MINB) k_cic_grad(CicGrad
       cic_gather_grad<N>(a.grho, a.pos, e, n3, ic, gxv, gyv, gzv);
     }
     if (a.gpos) {
-      gxv += __ldg(a.gpos + e);
-      gyv += __ldg(a.gpos + n3 + e);
-      gzv += __ldg(a.gpos + 2 * n3 + e);
+      gxv += gp[0];
+      gyv += gp[1];
+      gzv += gp[2];
     }
     a.gx[e] = gxv;
     a.gy[e] = gyv;
@@ -389,7 +394,7 @@ cudaError_t launch_shell_geometry(int n, double box, int n_shells, double* ksum,
 // (lane, b) = (tid / ns, tid % ns) sums rows lane, lane + L, ... of shell b (L = 256 / ns lanes; a
 // warp reads consecutive shells of a row, i.e. contiguous doubles), then the lanes are summed in
 // order into scratch[instance][g][b].
-__global__ void k_pk_rows(const double* __restrict__ part, int n_blocks, int ns, int rows, double* __restrict__ scratch) {
+__global__ void k_pk_rows(const double* part, int n_blocks, int ns, int rows, double* scratch) {
   grid_sync();
   const int g = blockIdx.x, inst = blockIdx.y;
   part += (size_t)inst * n_blocks * ns;
@@ -412,7 +417,7 @@ __global__ void k_pk_rows(const double* __restrict__ part, int n_blocks, int ns,
 // P(k) of an instance from n_rows rows of sums: as k_pk_rows over all rows, the lanes summed by a
 // fixed tree, divided by the shell's mode count.
 constexpr int kPkThreads = 1024;
-__global__ void __launch_bounds__(kPkThreads) k_pk_finalize_p(const double* __restrict__ sums, int n_rows, int ns,
+__global__ void __launch_bounds__(kPkThreads) k_pk_finalize_p(const double* sums, int n_rows, int ns,
                                                               const double* ksum, const unsigned long long* count,
                                                               double* pk, double* kmean, int64_t* nmodes) {
   __shared__ double sh[kPkThreads];

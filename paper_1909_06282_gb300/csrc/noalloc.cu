@@ -203,6 +203,8 @@ extern "C" int lpt2_cic_pk_noalloc(int n, double box, const float* pos, float* d
     if (e_ != cudaSuccess) return fail(LPT2_ECUDA, std::string(#expr ": ") + cudaGetErrorString(e_)); \
   } while (0)
 
+  // the passes read the table before their grid_sync(): the clear and the deposit, which wait for
+  // it, lie between
   noalloc_twiddles(n, tw, s);
   NA_CHECK(cudaGetLastError());
   NA_CHECK(launch_fill0(rho, n3, s));               // the deposit accumulates: start from zero

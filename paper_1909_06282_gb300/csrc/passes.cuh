@@ -172,15 +172,15 @@ __device__ __forceinline__ void z_store_pair_d(const float2 (&v)[Cfg<N>::RMAX], 
 // Z value at element n of the Hermitian extension of two half-spectrum rows,
 // each multiplied by (i k_z)^m first: Z = A + i B.
 template <int N>
-__device__ __forceinline__ float2 z_assemble(const float2* __restrict__ ra, const float2* __restrict__ rb,
+__device__ __forceinline__ float2 z_assemble(const float2* ra, const float2* rb,
                                              int n, float kf, int ma, int mb) {
   constexpr int H = N / 2;
   if (n == H) return make_float2(0.f, 0.f);
   const bool lo = n < H;
   const int m = lo ? n : N - n;
   const float kz = kf * (float)m;
-  float2 A = deriv(__ldg(ra + m), kz, ma);
-  float2 B = deriv(__ldg(rb + m), kz, mb);
+  float2 A = deriv(ra[m], kz, ma);
+  float2 B = deriv(rb[m], kz, mb);
   if (!lo) { A = cconj(A); B = cconj(B); }
   return make_float2(A.x - B.y, A.y + B.x);
 }
@@ -196,18 +196,20 @@ template <int N, int SRC> constexpr int zr2c_smem() {
 #define LPT2_ZNOISE_MINB 3   // resident noise-pass CTAs per SM asked: 80 registers (it is issue bound)
 #endif
 template <int N, int SRC>
-__global__ void __launch_bounds__(PassCfg<N>::ZT, SRC == Z_NOISE ? LPT2_ZNOISE_MINB : LPT2_Z_MINB)
+__global__ void __launch_bounds__(PassCfg<N>::ZT, SRC == Z_NOISE ? LPT2_ZNOISE_MINB
+                                         : SRC == Z_DENSITY && PassCfg<N>::ZT <= 256 ? 3 : LPT2_Z_MINB)
     k_z_r2c(ZR2CArgs a) {
   using C = PassCfg<N>;
   extern __shared__ __align__(16) float2 smem[];
   float2* s_tw = smem;
   float4* s_bm = reinterpret_cast<float4*>(reinterpret_cast<char*>(smem) + zr2c_tab_off<N>());
-  load_twiddles(s_tw, a.tw, N);
   if (SRC == Z_NOISE) {
+    load_twiddles(s_tw, a.tw, N);
     bm_load_table(s_bm, a.bm);
     __syncthreads();
+  } else {
+    grid_sync();
   }
-  if (SRC != Z_NOISE) grid_sync();
   const int p = threadIdx.x / C::TPP, t = threadIdx.x % C::TPP;
   const SmemRowT<kRowWarp<N>> sm{smem + N + p * SmemRow::words(N)};
   const int pair = blockIdx.x * C::ZP + p;
@@ -234,20 +236,23 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, SRC == Z_NOISE ? LPT2_ZNOISE_M
 #pragma unroll
     for (int r = 0; r < C::RMAX; ++r) {
       const int n = elem<N>(t, r);
-      float fa, fb;
-      fa = __ldg(a.in + (size_t)rowa * N + n);
-      fb = __ldg(a.in + (size_t)rowb * N + n);
-      if (SRC == Z_DENSITY) {
-        // density contrast rho N^3 / N_p - 1 with one particle per cell.  Written from here it
-        // costs its own bytes only (a pass of its own re-read the density: 260 us at 512^3)
-        fa -= 1.0f;
-        fb -= 1.0f;
+      v[r] = make_float2(a.in[(size_t)rowa * N + n], a.in[(size_t)rowb * N + n]);
+    }
+    load_twiddles(s_tw, a.tw, N);   // behind the row's loads: one latency for both
+    if (SRC == Z_DENSITY) {
+      // density contrast rho N^3 / N_p - 1 with one particle per cell.  Written from here it
+      // costs its own bytes only (a pass of its own re-read the density: 260 us at 512^3); after
+      // all the loads, which could not pass a store
+#pragma unroll
+      for (int r = 0; r < C::RMAX; ++r) {
+        const int n = elem<N>(t, r);
+        v[r].x -= 1.0f;
+        v[r].y -= 1.0f;
         if (a.contrast) {
-          a.contrast[(size_t)rowa * N + n] = fa;
-          a.contrast[(size_t)rowb * N + n] = fb;
+          a.contrast[(size_t)rowa * N + n] = v[r].x;
+          a.contrast[(size_t)rowb * N + n] = v[r].y;
         }
       }
-      v[r] = make_float2(fa, fb);
     }
   }
   if (SRC == Z_NOISE) grid_sync();   // the draws need nothing of the earlier kernels
@@ -261,7 +266,6 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_c2r(ZC2RArgs 
   using C = PassCfg<N>;
   extern __shared__ float2 smem[];
   float2* s_tw = smem;
-  load_twiddles(s_tw, a.tw, N);
   grid_sync();
   const int p = threadIdx.x / C::TPP, t = threadIdx.x % C::TPP;
   const SmemRowT<kRowWarp<N>> sm{smem + N + p * SmemRow::words(N)};
@@ -276,14 +280,21 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_c2r(ZC2RArgs 
   float2 v[C::RMAX];
 #pragma unroll
   for (int r = 0; r < C::RMAX; ++r) v[r] = z_assemble<N>(ra, rb, elem<N>(t, r), 0.f, 0, 0);
+  load_twiddles(s_tw, a.tw, N);   // behind the rows' loads: one latency for both
   __syncthreads();
   fft<N, true>(v, t, sm, s_tw);
+  if (a.add_in) {   // all loads before the stores
+#pragma unroll
+    for (int r = 0; r < C::RMAX; ++r) {
+      const int n = elem<N>(t, r);
+      v[r] = cadd(v[r], make_float2(a.add_in[(size_t)rowa * N + n], a.add_in[(size_t)rowb * N + n]));
+    }
+  }
 #pragma unroll
   for (int r = 0; r < C::RMAX; ++r) {
     const int n = elem<N>(t, r);
-    const size_t ea = (size_t)rowa * N + n, eb = (size_t)rowb * N + n;
-    a.out[ea] = a.add_in ? v[r].x + __ldg(a.add_in + ea) : v[r].x;
-    a.out[eb] = a.add_in ? v[r].y + __ldg(a.add_in + eb) : v[r].y;
+    a.out[(size_t)rowa * N + n] = v[r].x;
+    a.out[(size_t)rowb * N + n] = v[r].y;
   }
 }
 
@@ -809,12 +820,12 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_split_cta(ZFi
 // dL/drho at the 8 cells of each particle into dL/dx (= dL/dPsi), then forward
 // z transforms with conj z-derivatives: (g_x, g_y) of each row, g_z of both rows.
 template <int N>
-__device__ __forceinline__ void cic_gather_grad(const float* __restrict__ g, const float* __restrict__ pos,
+__device__ __forceinline__ void cic_gather_grad(const float* g, const float* pos,
                                                 size_t e, size_t n3, float inv_cell, float& gx, float& gy,
                                                 float& gz) {
-  const float ux = wrapN<N>(__ldg(pos + e) * inv_cell);
-  const float uy = wrapN<N>(__ldg(pos + n3 + e) * inv_cell);
-  const float uz = wrapN<N>(__ldg(pos + 2 * n3 + e) * inv_cell);
+  const float ux = wrapN<N>(pos[e] * inv_cell);
+  const float uy = wrapN<N>(pos[n3 + e] * inv_cell);
+  const float uz = wrapN<N>(pos[2 * n3 + e] * inv_cell);
   const float fx = floorf(ux), fy = floorf(uy), fz = floorf(uz);
   const float dx = ux - fx, dy = uy - fy, dz = uz - fz;
   const int ix = wrap_idx<N>((int)fx), iy = wrap_idx<N>((int)fy), iz = wrap_idx<N>((int)fz);
@@ -828,7 +839,7 @@ __device__ __forceinline__ void cic_gather_grad(const float* __restrict__ g, con
     for (int oy = 0; oy < 2; ++oy)
 #pragma unroll
       for (int oz = 0; oz < 2; ++oz) {
-        const float gc = __ldg(g + ((size_t)cx[ox] * N + cy[oy]) * N + cz[oz]);
+        const float gc = g[((size_t)cx[ox] * N + cy[oy]) * N + cz[oz]];
         const float sx = ox ? 1.f : -1.f, sy = oy ? 1.f : -1.f, sz = oz ? 1.f : -1.f;
         ax = fmaf(gc * sx, wy[oy] * wz[oz], ax);
         ay = fmaf(gc * sy, wx[ox] * wz[oz], ay);
@@ -900,7 +911,7 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_adj_source(ZA
 #pragma unroll
       for (int r = 0; r < C::RMAX; ++r) {
         const int iz = elem<N>(t, r);
-        const float ga = __ldg(g0 + iz), gb = __ldg(g0 + N + iz);
+        const float ga = g0[iz], gb = g0[N + iz];
         v[r] = f < 3 ? make_float2(ga * (T0[r] - v[r].x), gb * (T1[r] - v[r].y))
                      : make_float2(-2.f * ga * v[r].x, -2.f * gb * v[r].y);
       }
@@ -997,14 +1008,14 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_adj_source_ct
 #pragma unroll
       for (int r = 0; r < C::RMAX; ++r) {
         const int iz = elem<N>(t, r);
-        const float ga = __ldg(g0 + iz), gb = __ldg(g0 + N + iz);
+        const float ga = g0[iz], gb = g0[N + iz];
         v[r] = make_float2(ga * (T0[r] - v[r].x), gb * (T1[r] - v[r].y));
       }
     } else {
 #pragma unroll
       for (int r = 0; r < C::RMAX; ++r) {
         const int iz = elem<N>(t, r);
-        const float ga = __ldg(g0 + iz), gb = __ldg(g0 + N + iz);
+        const float ga = g0[iz], gb = g0[N + iz];
         v[r] = make_float2(-2.f * ga * v[r].x, -2.f * gb * v[r].y);
       }
     }
@@ -2114,6 +2125,12 @@ template <int N, int MODE> cudaError_t launch_x_m(const XArgs& a, cudaStream_t s
   constexpr bool has_split = MODE == X_DELTA || MODE == X_SOURCE;
   auto k = has_split && a.split ? k_x<N, MODE, has_split> : k_x<N, MODE, false>;
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if constexpr (MODE == X_PKADJ) {
+    // not overlapped: it gathers the shell weights, which the kernel before it writes, on the
+    // read-only path (32 plain loads between the branches of shell_of spill 112 bytes a thread)
+    k<<<dim3(C::H / C::W, N, a.g.batch), C::XT, smem, s>>>(a);
+    return cudaGetLastError();
+  }
   return launch_overlapped(k, dim3(C::H / C::W, N, a.g.batch), C::XT, smem, s, a);
 }
 template <int N> cudaError_t launch_x_t(const XArgs& a, cudaStream_t s) {

@@ -17,7 +17,11 @@ namespace lpt2 {
 
 // Start of a kernel launched with launch_overlapped (passes.h): waits until the stream's earlier
 // kernels have completed and their writes are visible.  Before it a kernel touches only shared
-// memory and tables that the plan wrote once (twiddles, Box-Muller).  No kernel signals its
+// memory and tables that were complete when the kernel before it started: the plan's (twiddles,
+// Box-Muller, seeds), or twiddles written on the same stream with at least one overlapped kernel,
+// which waits in every thread, in between (lpt2_cic_pk_noalloc).  After it, what the previous
+// kernel wrote is read with plain loads: __ldg and const __restrict__ promise data that does not
+// change while the kernel lives, and let the compiler move the load above the wait.  No kernel signals its
 // dependents early (griddepcontrol.launch_dependents): the next kernel's CTAs then start when the
 // last of this one's have exited, which hides the launch and the set-up (64^3 102 -> 78 us a
 // step).  Signalling at the start costs more than it hides: CTAs that start on an SM still

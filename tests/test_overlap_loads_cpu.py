@@ -1,0 +1,41 @@
+"""Kernels that start before the stream's previous kernel has ended (grid_sync() in their body) must
+read what that kernel writes with plain loads: the read-only path (__ldg, const __restrict__) is for
+data that does not change while the kernel lives, and the compiler may move such a load above the
+wait.  On that path may be only the tables that set-up calls wrote several kernels before (twiddles,
+Box-Muller, multipliers, the sqrt(P) field), and the shell weights of X_PKADJ, whose launch is not
+overlapped."""
+import os
+import re
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_1909_06282_gb300", "csrc")
+TABLES = {"g_tab", "a.mt0", "a.mt1", "mp", "a.scf", "sp"}
+
+
+def sources():
+    return {f: open(os.path.join(CSRC, f)).read() for f in sorted(os.listdir(CSRC)) if f.endswith((".cu", ".cuh"))}
+
+
+def test_read_only_loads_are_of_tables():
+    src = sources()
+    seen = set()
+    for text in src.values():
+        seen |= {m.group(1) for m in re.finditer(r"__ldg\(\s*(?:reinterpret_cast<[^>]*>\()?([\w.]+)", text)}
+    assert seen <= TABLES | {"a.shell_w"}
+    # the weights are read in X_PKADJ only, and its launch is an ordinary one
+    p = src["passes.cuh"]
+    assert p.count("__ldg(a.shell_w") == 1
+    launch = p[p.index("cudaError_t launch_x_m("):p.index("cudaError_t launch_x_t(")]
+    assert re.search(r"if constexpr \(MODE == X_PKADJ\) \{[^}]*k<<<[^}]*return cudaGetLastError\(\);\s*\}", launch)
+
+
+def test_overlapped_kernels_take_no_restricted_inputs():
+    for f, text in sources().items():
+        for m in re.finditer(r"__global__[^;{]*\{", text):
+            end = text.find("\n}\n", m.start())
+            if "grid_sync()" in text[m.start():end]:
+                assert "__restrict__" not in m.group(0), (f, m.group(0))
+    # functions inlined into them: restricted inputs are the tables
+    for f in ("passes.cuh", "fft_core.cuh", "boxmuller.cuh"):
+        for name in re.findall(r"const \w+\s*\*\s*__restrict__ (\w+)", sources()[f]):
+            assert name in {"tw", "g_tw", "g_tab"}, (f, name)
