@@ -1049,10 +1049,6 @@ int displace_prefix(lpt2_plan_t p, const FwdSlots& f, const float* noise, bool s
   x.cosmo = p->cosmo_dev;
   x.mt0 = p->mt0;
   x.mt1 = p->mt1;
-  x.d1f = p->tabf;
-  x.d2f = p->tabf + p->nk;
-  x.t1f = p->tabf + 2 * p->nk;
-  x.t2f = p->tabf + 3 * p->nk;
   LAUNCH(p, "x_delta", (split ? 28.0 : 22.0) * V3(p), x_pass(n, x, p->stream));   // + the sqrt(P) field
 
   // 2. y inverse with y derivatives: the six phi_ij (+ Psi1)
@@ -1098,11 +1094,9 @@ int displace_prefix(lpt2_plan_t p, const FwdSlots& f, const float* noise, bool s
 }
 
 // Steps of one output scale factor, whose D1(k, a), D2(k, a) enter through the
-// multiplier tables mt0 and the growth tables tabf: S(k) -> phi2 (+ phi1 D1),
-// Psi, positions, CIC density (slots A and D are read, not written).
+// multiplier tables mt0: S(k) -> phi2 (+ phi1 D1), Psi, positions, CIC density (slots A and D are read, not written).
 int displace_suffix(lpt2_plan_t p, const FwdSlots& f, bool split, float* psi1, float* psi2, float* pos,
-                    float2* s_keep, const float4* mt0, const float* tabf,
-                    float* pos_scratch = nullptr) {
+                    float2* s_keep, const float4* mt0, float* pos_scratch = nullptr) {
   const int n = p->n;
   const Geo g = make_geo(p);
   float* rho = rho_group(p);
@@ -1122,10 +1116,6 @@ int displace_suffix(lpt2_plan_t p, const FwdSlots& f, bool split, float* psi1, f
   xs.out[1] = f.X[1];
   xs.cosmo = p->cosmo_dev;
   xs.mt0 = mt0;
-  xs.d1f = tabf;
-  xs.d2f = tabf + p->nk;
-  xs.t1f = tabf + 2 * p->nk;
-  xs.t2f = tabf + 3 * p->nk;
   LAUNCH(p, "x_source", (split ? 16.0 : 20.0) * V3(p), x_pass(n, xs, p->stream));   // + the cleared density
 
   // 5. y inverse: (x0 y0), (x0 y1), (x1 y0)
@@ -1174,7 +1164,7 @@ int displace_impl(lpt2_plan_t p, const float* noise, float* psi1, float* psi2, f
   const FwdSlots f = fwd_slots(p);
   int rc = displace_prefix(p, f, noise, split);
   if (rc) return rc;
-  rc = displace_suffix(p, f, split, psi1, psi2, pos, s_keep, p->mt0, p->tabf, pos_scratch);
+  rc = displace_suffix(p, f, split, psi1, psi2, pos, s_keep, p->mt0, pos_scratch);
   if (rc) return rc;
   if (dk) {
     const size_t cells = (size_t)p->n * p->n * p->n * p->cur_batch;
@@ -1361,8 +1351,7 @@ int lpt2_displace_outputs(lpt2_plan_t p, const float* noise, float* pos, double*
   if (rc) return rc;
   const size_t n3 = (size_t)p->n * p->n * p->n;
   for (int j = 0; j < p->n_out_a; ++j) {
-    rc = displace_suffix(p, f, false, nullptr, nullptr, pos ? pos + j * 3 * n3 : nullptr, nullptr,
-                         out_mt0(p, j), out_tabf(p, j));
+    rc = displace_suffix(p, f, false, nullptr, nullptr, pos ? pos + j * 3 * n3 : nullptr, nullptr, out_mt0(p, j));
     if (rc) return rc;
     // the density spectrum goes to a slot the suffix does not use (A and D stay intact)
     rc = cic_pk_group(p, 0, nullptr, nullptr, pk + (size_t)j * n_shells, j == 0 ? k_mean : nullptr,
@@ -1650,10 +1639,6 @@ int lpt2_source_ratio(lpt2_plan_t p, const float* noise, int n_bins, double* mea
     x.cosmo = p->cosmo_dev;
     x.mt0 = p->mt0;
     x.mt1 = p->mt1;
-    x.d1f = p->tabf;
-    x.d2f = p->tabf + p->nk;
-    x.t1f = p->tabf + 2 * p->nk;
-    x.t2f = p->tabf + 3 * p->nk;
     LAUNCH(p, "x_delta", 22.0 * V3(p), x_pass(n, x, p->stream));   // + the sqrt(P) field
   }
   // one real field: IDFT[(i k)^ord g(|k|) delta0(k)]
@@ -1962,10 +1947,6 @@ int lpt2_displace_vjp(lpt2_plan_t p, const float* noise, const float* g_pos, con
   xs.cosmo = p->cosmo_dev;
   xs.mt0 = p->mt0;
   xs.mt1 = p->mt1;
-  xs.d1f = p->tabf;
-  xs.d2f = p->tabf + p->nk;
-  xs.t1f = p->tabf + 2 * p->nk;
-  xs.t2f = p->tabf + 3 * p->nk;
   xs.theta_part = thp;
   LAUNCH(p, "x_adj_source", 28.0 * V3(p), x_pass(n, xs, p->stream));
   YArgs yh = yi;

@@ -41,10 +41,6 @@ template <int N> struct PassCfg {
   static constexpr int XT = TPP * W;                                  // y/x CTA threads
   static constexpr int ZSMEM = (N + ZP * SmemRow::words(N)) * 8;
   static constexpr int XSMEM = (N + N * W) * 8;
-  // resident x-pass CTAs per SM asked of the compiler: caps a thread at 128 registers for
-  // every CTA size (at 256 threads the multi-output modes would otherwise take 184 and
-  // halve the warps per SM)
-  static constexpr int XMINB = XT >= 512 ? 1 : 512 / XT;
 };
 
 // y passes: their own pencils per CTA (the y tile rows are 2 KB apart, the x tile rows a
@@ -93,7 +89,8 @@ template <int N, int MODE> struct XCfg {
   static constexpr bool PAIR =
       MODE == X_PKP || MODE == X_PKI || MODE == X_ADJ_SOURCE || MODE == X_ADJ_DELTA;
   static constexpr int XSMEM = (N + N * W) * 8;
-  // resident CTAs per SM asked of the compiler: a cap of 128 registers, or 64 for the
+  // resident CTAs per SM asked of the compiler: a cap of 128 registers (at 256 threads the
+  // multi-output modes would otherwise take 184 and halve the warps per SM), or 64 for the
   // one-transform shell sums (twice the CTAs)
   static constexpr int CAP = MODE == X_PK || MODE == X_PKP ? 1024 : 512;
   static constexpr int MINB = XT >= CAP ? 1 : CAP / XT;

@@ -179,10 +179,6 @@ struct XArgs {
   const float2* hpsi_in;  // X_ADJ_DELTA: h_Psi(k)
   float2* out[5];         // x-inverse outputs
   const DevCosmo* cosmo;
-  const float* d1f;       // float growth tables [nk]
-  const float* d2f;
-  const float* t1f;       // float d/dln|fR0| tables [nk]
-  const float* t2f;
   double* pk_part;        // X_PK: per-block partials [blocks][3][n_shells]
   int n_shells;
   const float* shell_w;   // X_PKADJ: weight per shell
@@ -258,7 +254,6 @@ LPT2_DECLARE_LAUNCHERS(1024)
 // Size-independent kernels (misc.cu / growth.cu).
 cudaError_t launch_cic(const CicArgs&, cudaStream_t);   // grid y = a.g.batch
 cudaError_t launch_fill0(float* p, size_t n, cudaStream_t);
-cudaError_t launch_contrast(const float* rho, float* out, size_t n, cudaStream_t);
 cudaError_t launch_pk_finalize(const double* part, int n_blocks, int n_shells, double* pk,
                                double* k_mean, int64_t* n_modes, cudaStream_t, int batch = 1);
 // Mode count and sum of |k| per shell (0 < |n| < N/2, half spectrum kz < N/2, kz > 0
