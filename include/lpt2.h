@@ -161,8 +161,8 @@ int lpt2_set_workspace(lpt2_plan_t plan, void* dev_ptr, size_t bytes);
  * default) and their derivatives with respect to ln|f_R0| (Eq. d1, Eq. full-d2 at
  * the variant's triangle, T1: k1 = k2 = k/sqrt2, theta = 90 deg; D2 sign such
  * that GR gives -3/7 D1^2), recomputed
- * on the plan's stream by the batched FP64 RK4 kernel (one thread per
- * (instance, k)) and copied into the caller's device arrays double[n_inst][n_k]
+ * on the plan's stream by the batched FP64 RK4 kernel (a lane per second-order
+ * chain of an (instance, k)) and copied into the caller's device arrays double[n_inst][n_k]
  * (each pointer may be NULL). */
 int lpt2_growth_tables(lpt2_plan_t plan, double* d1, double* d2,
                        double* dd1_dlogf, double* dd2_dlogf);

@@ -28,8 +28,8 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
 // The radix butterflies add with padd / psub (packed.cuh).  A packed add has the arithmetic rate
 // of two scalar adds but takes one issue slot instead of two (measured: 0.53 against 1.04
 // instructions per cycle and scheduler), and the passes with several transforms per field are
-// bound by issue and shared-memory slots: z_source at 512^3 1141 -> 1071 us, z_final 636 -> 617
-// us, x_pkadj 367 -> 341 us.  Products stay scalar: a packed complex product needs swapped or
+// bound by issue and shared-memory slots: z_source at 512^3 1141 -> 1071 us, z_final 636 -> 617.
+// (Its aligned register pairs cost x_delta and x_source at 512 spills of 132 and 68 bytes.)  Products stay scalar: a packed complex product needs swapped or
 // doubled operands, whose moves cost what it saves.
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
 __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
@@ -39,13 +39,12 @@ __device__ __forceinline__ float2 mul_mi(float2 a) { return make_float2(a.y, -a.
 // ------------------------------------------------------------ radix schedules
 // V = 0: radix sequences with the same radix first and last (so that stage-0 input and
 // last-stage output share one element pattern); every radix divides RMAX.
-// V = 1 (where it exists): twice the values per thread and two stages, so one shared-memory
-// exchange per transform instead of two, half the twiddle loads and half the threads per
-// pencil: for passes that hold one array of values (registers).  fft() brings the outputs
-// back into the input's pattern (a renaming of registers).  N = 128 in all passes instead of 8-2-8 was
-// slower where passes follow one another without a pause: the batch of 96 mixed grids 16.69 ms, against
-// 15.50 with 8-2-8 and 15.40 with 16-8 in the y passes, the plain x passes, the source and the shell sums
-// only (five output times 445, 421 and 409 us).
+// V = 1 (32, 128, 512): twice the values per thread and two stages, so one shared-memory exchange
+// per transform instead of two, half the twiddle loads and half the threads per pencil.  fft()
+// brings the outputs back into the input's pattern (a renaming of registers).
+// Rule (YCfg, XCfg): passes that hold one array of values, where the registers allow it.  The z
+// passes, x_delta, the adjoint x passes and the summing y passes keep V = 0: 16-8 in all passes at
+// 128 costs the batch of 96 mixed grids 16.7 ms a call, 8-2-8 in all 15.5, by the rule 15.4.
 template <int N, int V = 0> struct Cfg;
 template <> struct Cfg<96>   { static constexpr int NS = 3, RMAX = 12; static __host__ __device__ constexpr int rad(int s) { return s == 1 ? 6 : 4; } };
 template <> struct Cfg<192>  { static constexpr int NS = 3, RMAX = 12; static __host__ __device__ constexpr int rad(int s) { return s == 1 ? 12 : 4; } };
@@ -195,11 +194,12 @@ template <int R, bool INV> struct Dft {   // even R: split into even and odd hal
 // butterfly are the same register of threads t and t + TPP / 2.  Where those are lanes of one warp
 // (partner(): the lane mask, 0 where they are not), the middle stage can run on shuffles: one exchange
 // through shared memory per transform instead of two, which is what bounds the z passes (70 % of
-// their cycles) and whose CTA barriers the x passes wait at.  512^3: z_source 1099 -> 1043 us,
-// z_adj_source 1766 -> 1672, x_adj_delta 833 -> 769, x_adj_source 874 -> 857, x_pk 251 -> 240, z_c2r 208 ->
-// 198; 64 batched 32^3 grids: z_source 27.8 -> 22.7, z_final 20.4 -> 17.8.  Not where the 32 values in
-// flight spill (x_delta 740 -> 863, x_source 702 -> 723, the y passes that sum 1065 -> 1141), nor in
-// z_final at 512, whose independent warps miss the instruction cache (499 -> 512).
+// their cycles) and whose CTA barriers the x passes wait at.
+// Rule: z passes of 32, 128 and 512 (512^3: z_source 1099 -> 1043 us, z_adj_source 1766 -> 1672) and,
+// at 512, the shell sums and the adjoint x passes (x_pk 251 -> 240, x_adj_delta 833 -> 769).  Not
+// where they spill more than the pass does without them (x_delta, 132 bytes a thread as it stands,
+// 740 -> 863 us; x_source 702 -> 723; the summing y passes 1065 -> 1141), nor in z_final at
+// 512, whose independent warps miss the instruction cache (499 -> 512).
 template <int N, int V> inline constexpr bool kPaired =
     Cfg<N, V>::NS == 3 && Cfg<N, V>::rad(1) == 2 && Cfg<N, V>::RMAX == Cfg<N, V>::rad(0);
 

@@ -48,13 +48,13 @@ template <int N> struct PassCfg {
 // the build default; the launcher also has WY = 8 and 16 compiled, which a plan's tile
 // schedule (Geo::ytile) selects per grid-size group.
 //
-// N = 512, one array of values (Y_ONE, Y_MULTI): bound by DRAM, whose rows want 128-byte
-// segments, so 16 kz per CTA; with 16 values per thread that CTA has 512 threads that
-// wait for one another (y_phi 1399 us), with 32 values 256 threads and one exchange instead
-// of two: y_phi 1067 -> 930 us, y_psi 537 -> 463, y_fwd 215 -> 184 against 8 kz and 16
-// values.  N = 32 (8-4 instead of 4-2-4): 64 batched grids y_phi 19.1 -> 16.4 us, x_pk 13.1 -> 10.5, the
-// call 108.5 -> 104.7.  N = 128 (16-8): five output times 414 -> 409 us a call.  Two CTAs per SM at 512: a third fits in registers (80), but its tile takes the L1 the loads in
-// flight need (y_phi 1098 us).  Y_SUM keeps an accumulator beside the values: 8 kz, 16 values.
+// Rule: passes that hold one array of values (Y_ONE, Y_MULTI) take the two-stage transform (V = 1)
+// where N has one; Y_SUM, with an accumulator beside the values, the three-stage one.
+// N = 512 is bound by DRAM, whose rows want 128-byte segments: 16 kz per CTA, which with V = 1 has 256
+// threads (y_phi 930 us; 8 kz and V = 0 1067; 16 kz and V = 0, 512 threads that wait for one another,
+// 1399).  Two CTAs per SM: a third fits in registers (80), but its tile takes the L1 that the loads in
+// flight need (y_phi 1098).
+// N = 32: y_phi of 64 batched grids 19.1 -> 16.4 us.  N = 128: five output times 414 -> 409 us a call.
 enum YKind { Y_MULTI = 0, Y_SUM = 1, Y_ONE = 2 };
 template <int N, int KIND, int WY = 0> struct YCfg {
   static constexpr int H = N / 2;
@@ -70,11 +70,11 @@ template <int N, int KIND, int WY = 0> struct YCfg {
   static_assert(H % W == 0, "a CTA's kz block must tile the half spectrum");
 };
 
-// x passes: the tile of a mode.  V = 1 as in the y passes (N = 512, modes that hold one array of
-// values): 16 kz and 32 values per thread, x_fwd 275 -> 185 us, x_inv 284 -> 182, x_pkadj 343 ->
-// 334.  Not the shell sums there: they want the resident warps that 64 registers allow (250 us against
-// 275 with 32 values).  N = 128 (16 values): x_pk of five output times 63 -> 53 us, x_source 80 -> 74.
-// N = 32 (4 threads a pencil): where 8 pencils or more make whole warps.
+// x passes: the tile of a mode.  V = 1 in the modes that hold one array of values: at 512 the plain
+// ones, with 16 kz (x_fwd 275 -> 185 us, x_pkadj 343 -> 334), but not the shell sums, which want the
+// resident warps that 64 registers allow (250 us against 275); at 128 also the shell sums (63 -> 53 us
+// for five output times) and the source (80 -> 74); at 32 the shell sums (4 threads a pencil: where 8
+// pencils or more make whole warps; 64 batched grids 13.1 -> 10.5 us).
 template <int N, int MODE> struct XCfg {
   static constexpr bool PLAIN = MODE == X_FWD || MODE == X_INV || MODE == X_PKADJ || MODE == X_MUL;
   static constexpr bool SHELLS = MODE == X_PKP || MODE == X_PKI;
@@ -308,13 +308,12 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_c2r(ZC2RArgs 
 // g, g + G, ...) and synchronises with nobody: while one group waits for a copy or an exchange
 // the others issue, and the next tile's first copies fly during this one's last transforms.
 //
-// Which: warps that run apart fetch different instructions, so the group form pays where its
-// code is short.  The total form of z_final (one transform body) at every N: 512^3 622 -> 516
-// us, 256^3 82 -> 72, 96 batched instances 1605 -> 1307.  The others (several bodies) up to N =
-// 192, where a pencil's transform is short: z_source 2859 -> 2435 us (the 96 instances), split
-// z_final at 128^3 31.1 -> 26.6, z_adj_source at 128^3 52 -> 47; from N = 256 on the CTA form:
-// z_source 123 against 141 us at 256^3 and 1096 against 1416 at 512^3 (where the loop state also
-// spills), split z_final 156 against 171 at 256^3, z_adj_source 261 against 272.
+// Rule: warps that run apart fetch different instructions, so the group form pays where its code is
+// short.  The total form of z_final (one transform body) takes it at every N (512^3 622 -> 516 us, 96
+// batched instances 1605 -> 1307); z_source, the split z_final and z_adj_source (several bodies) up to
+// N = 192 (z_source of the batch 2859 -> 2435 us; at 192 the other two are level), above it the CTA
+// form (z_source 123 against 141 us at 256^3, 1096 against 1416 at 512^3, where the loop state also
+// spills; both before the middle radix went to shuffles: 1044 at 512^3 now).
 #ifndef LPT2_ZS_STAGES
 #define LPT2_ZS_STAGES 2
 #endif
@@ -1034,9 +1033,9 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_adj_source_ct
 // paired-row form transforms 7.5 pencils per row and reads the diagonal fields twice).
 // Tiles as in the field-pair layout: a ring stage holds the two fields of a pencil for the
 // CTA's eight rows, each row in its warp's padded region, used in place as the exchange row.  The
-// rows of g_S come with them: read from global memory where they are used, behind a
-// transform, they cost 250 us (512^3: 2005 -> 1754; 1672 with the middle radix on shuffles).  One tile per CTA: a persistent walk needs
-// registers that spill (2654 us).
+// rows of g_S come with them: read from global memory where they are used, behind a transform, they
+// cost 250 us of 2005 at 512^3.  One tile per CTA: a persistent walk needs registers that spill (2654
+// us).  1665 us now.
 #ifndef LPT2_ZADJ_FIELD_PAIRS
 #define LPT2_ZADJ_FIELD_PAIRS 1
 #endif
@@ -1439,9 +1438,8 @@ __device__ __forceinline__ void x_tile(const XArgs& a, float2 (&v)[XCfg<N, MODE>
     // holds an FP64 unit for 64 cycles).  The shell of a mode is a float estimate of floor(2 ns |n| /
     // N), off by at most one, corrected against integer thresholds.  A value passes through at most
     // RMAX + 5 FP32 additions (relative error below 21 x 2^-24 even when every rounding goes one way).
-    // Measured (against a warp's two reductions for its patch's shells and a warp sum for each):
-    // x_pk at 512^3 329 -> 250 us (240 with the middle radix on shuffles), 96 batched instances 948 -> 700, 48 shells at 192^3 61 -> 48, 64^3
-    // 12.3 -> 8.1 us.
+    // x_pk at 512^3 240 us, 48 shells at 192^3 48, 64^3 8 (by reductions over the warp's patch of modes
+    // for each of its shells: 329, 61, 12).
     const float pnorm = a.g.box * a.g.box * a.g.box * a.g.inv_n3 * a.g.inv_n3;
     const int ns = a.n_shells;
     const int* s_thr = reinterpret_cast<const int*>(s_acc);   // [ns + 1]: smallest |n|^2 in shell b or above
