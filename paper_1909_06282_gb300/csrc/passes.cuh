@@ -1004,14 +1004,14 @@ __global__ void __launch_bounds__(PassCfg<N>::ZT, LPT2_Z_MINB) k_z_adj_source_ct
 #pragma unroll
       for (int r = 0; r < C::RMAX; ++r) {
         const int iz = elem<N>(t, r);
-        const float ga = g0[iz], gb = g0[N + iz];
+        const float ga = __ldg(g0 + iz), gb = __ldg(g0 + N + iz);
         v[r] = make_float2(ga * (T0[r] - v[r].x), gb * (T1[r] - v[r].y));
       }
     } else {
 #pragma unroll
       for (int r = 0; r < C::RMAX; ++r) {
         const int iz = elem<N>(t, r);
-        const float ga = g0[iz], gb = g0[N + iz];
+        const float ga = __ldg(g0 + iz), gb = __ldg(g0 + N + iz);
         v[r] = make_float2(-2.f * ga * v[r].x, -2.f * gb * v[r].y);
       }
     }
@@ -2015,10 +2015,14 @@ template <int N, class K, class A> cudaError_t launch_zgrp(K k, const A& a, cuda
   const cudaError_t e = persistent_grid(k, PassCfg<N>::ZT, Q::SMEM, Q::TILES * a.g.batch, Q::GROUPS, &grid);
   return e != cudaSuccess ? e : launch_overlapped(k, grid, PassCfg<N>::ZT, Q::SMEM, s, a);
 }
-template <int N, class K, class A> cudaError_t launch_zcta(K k, const A& a, cudaStream_t s) {
+template <int N, class K, class A> cudaError_t launch_zcta(K k, const A& a, cudaStream_t s, bool overlap = true) {
   using Q = ZSrcCfg<N>;
   LPT2_CHECK_BATCH(a);
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Q::SMEM);
+  if (!overlap) {
+    k<<<dim3(N * N / Q::ROWS, 1, a.g.batch), PassCfg<N>::ZT, Q::SMEM, s>>>(a);
+    return cudaGetLastError();
+  }
   return launch_overlapped(k, dim3(N * N / Q::ROWS, 1, a.g.batch), PassCfg<N>::ZT, Q::SMEM, s, a);
 }
 template <int N> cudaError_t launch_z_source_t(const ZSourceArgs& a, cudaStream_t s) {
@@ -2039,7 +2043,9 @@ template <int N> cudaError_t launch_z_adj_source_t(const ZAdjSourceArgs& a, cuda
   } else if constexpr (zgroups<N>()) {
     return launch_zgrp<N>(k_z_adj_source<N>, a, s);
   } else {
-    return launch_zcta<N>(k_z_adj_source_cta<N>, a, s);
+    // not overlapped: it reads g_S, which the kernel before it writes, on the read-only path, so that
+    // the compiler may place the reads before the transforms (256^3: 260 us; plain loads 288)
+    return launch_zcta<N>(k_z_adj_source_cta<N>, a, s, false);
   }
 }
 template <int N, int KIND, int WYA> cudaError_t launch_y_k(const YArgs& a, cudaStream_t s) {

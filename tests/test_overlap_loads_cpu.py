@@ -2,8 +2,8 @@
 read what that kernel writes with plain loads: the read-only path (__ldg, const __restrict__) is for
 data that does not change while the kernel lives, and the compiler may move such a load above the
 wait.  On that path may be only the tables that set-up calls wrote several kernels before (twiddles,
-Box-Muller, multipliers, the sqrt(P) field), and the shell weights of X_PKADJ, whose launch is not
-overlapped."""
+Box-Muller, multipliers, the sqrt(P) field), and the inputs of kernels whose launch is not overlapped:
+the shell weights of X_PKADJ and g_S (g0) of k_z_adj_source_cta."""
 import os
 import re
 
@@ -21,12 +21,16 @@ def test_read_only_loads_are_of_tables():
     seen = set()
     for text in src.values():
         seen |= {m.group(1) for m in re.finditer(r"__ldg\(\s*(?:reinterpret_cast<[^>]*>\()?([\w.]+)", text)}
-    assert seen <= TABLES | {"a.shell_w"}
+    assert seen <= TABLES | {"a.shell_w", "g0"}
     # the weights are read in X_PKADJ only, and its launch is an ordinary one
     p = src["passes.cuh"]
     assert p.count("__ldg(a.shell_w") == 1
     launch = p[p.index("cudaError_t launch_x_m("):p.index("cudaError_t launch_x_t(")]
     assert re.search(r"if constexpr \(MODE == X_PKADJ\) \{[^}]*k<<<[^}]*return cudaGetLastError\(\);\s*\}", launch)
+    cta = p[p.index("k_z_adj_source_cta(ZAdjSourceArgs a)"):p.index("k_z_adj_source_fp(ZAdjSourceArgs a)")]
+    assert p.count("__ldg(g0") == cta.count("__ldg(g0")
+    assert p.count("(k_z_adj_source_cta<N>, a, s, false)") == p.count("k_z_adj_source_cta<N>")
+    assert re.search(r"if \(!overlap\) \{[^}]*k<<<[^}]*return cudaGetLastError\(\);\s*\}", p)
 
 
 def test_overlapped_kernels_take_no_restricted_inputs():
