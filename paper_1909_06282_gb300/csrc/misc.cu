@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(CIC_THREADS, LPT2_CIC_MINB) k_cic_grad(CicGrad
     const int i = p / (CIC_T * CIC_T), j = (p / CIC_T) % CIC_T, l = p % CIC_T;
     const size_t e = ((size_t)(x0 + i) * N + (y0 + j)) * N + (z0 + l);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) u[k][c] = a.pos[c * n3 + e];
+    for (int c = 0; c < 3; ++c) u[k][c] = __ldg(a.pos + c * n3 + e);
   }
   // group q = (wx * CIC_E + wy) * CIC_QZ + qz, advanced by the CTA size without divisions
   constexpr int SQZ = CIC_THREADS % CIC_QZ, SR = CIC_THREADS / CIC_QZ;
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(CIC_THREADS, LPT2_CIC_MINB) k_cic_grad(CicGrad
       gy = wrap_cell<N>(gy);
       gz = wrap_cell<N>(gz);
     }
-    reinterpret_cast<float4*>(gw)[q] = *reinterpret_cast<const float4*>(a.grho + ((size_t)gx * N + gy) * N + gz);
+    reinterpret_cast<float4*>(gw)[q] = __ldg(reinterpret_cast<const float4*>(a.grho + ((size_t)gx * N + gy) * N + gz));
   }
   __syncthreads();
   const float ic = a.g.inv_cell;
@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(CIC_THREADS, LPT2_CIC_MINB) k_cic_grad(CicGrad
     float gp[3];   // read before the gather, whose latency covers this one's
     if (a.gpos) {
 #pragma unroll
-      for (int c = 0; c < 3; ++c) gp[c] = a.gpos[c * n3 + e];
+      for (int c = 0; c < 3; ++c) gp[c] = __ldg(a.gpos + c * n3 + e);
     }
     const float ux = wrapN<N>(u[k][0] * ic), uy = wrapN<N>(u[k][1] * ic), uz = wrapN<N>(u[k][2] * ic);
     const float fx = floorf(ux), fy = floorf(uy), fz = floorf(uz);
@@ -232,7 +232,11 @@ __global__ void __launch_bounds__(CIC_THREADS, LPT2_CIC_MINB) k_cic_grad(CicGrad
 template <int N>
 cudaError_t launch_cic_grad_n(const CicGradArgs& a, cudaStream_t s) {
   cudaFuncSetAttribute(k_cic_grad<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, CIC_SMEM);
-  return launch_overlapped(k_cic_grad<N>, (unsigned)((N / CIC_T) * (N / CIC_T) * (N / CIC_T)), CIC_THREADS, CIC_SMEM, s, a);
+  // not overlapped: the density cotangent, which the kernel before it writes, is read on the read-only
+  // path, from where the gathers of particles beyond the window may move above the stores of others
+  // (512^3 1279 us, 1466 with g_pos; plain loads 1389, 1570)
+  k_cic_grad<N><<<(unsigned)((N / CIC_T) * (N / CIC_T) * (N / CIC_T)), CIC_THREADS, CIC_SMEM, s>>>(a);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_cic_grad(const CicGradArgs& a, cudaStream_t s) {

@@ -819,9 +819,9 @@ template <int N>
 __device__ __forceinline__ void cic_gather_grad(const float* g, const float* pos,
                                                 size_t e, size_t n3, float inv_cell, float& gx, float& gy,
                                                 float& gz) {
-  const float ux = wrapN<N>(pos[e] * inv_cell);
-  const float uy = wrapN<N>(pos[n3 + e] * inv_cell);
-  const float uz = wrapN<N>(pos[2 * n3 + e] * inv_cell);
+  const float ux = wrapN<N>(__ldg(pos + e) * inv_cell);
+  const float uy = wrapN<N>(__ldg(pos + n3 + e) * inv_cell);
+  const float uz = wrapN<N>(__ldg(pos + 2 * n3 + e) * inv_cell);
   const float fx = floorf(ux), fy = floorf(uy), fz = floorf(uz);
   const float dx = ux - fx, dy = uy - fy, dz = uz - fz;
   const int ix = wrap_idx<N>((int)fx), iy = wrap_idx<N>((int)fy), iz = wrap_idx<N>((int)fz);
@@ -835,7 +835,7 @@ __device__ __forceinline__ void cic_gather_grad(const float* g, const float* pos
     for (int oy = 0; oy < 2; ++oy)
 #pragma unroll
       for (int oz = 0; oz < 2; ++oz) {
-        const float gc = g[((size_t)cx[ox] * N + cy[oy]) * N + cz[oz]];
+        const float gc = __ldg(g + ((size_t)cx[ox] * N + cy[oy]) * N + cz[oz]);
         const float sx = ox ? 1.f : -1.f, sy = oy ? 1.f : -1.f, sz = oz ? 1.f : -1.f;
         ax = fmaf(gc * sx, wy[oy] * wz[oz], ax);
         ay = fmaf(gc * sy, wx[ox] * wz[oz], ay);

@@ -3,7 +3,7 @@ read what that kernel writes with plain loads: the read-only path (__ldg, const 
 data that does not change while the kernel lives, and the compiler may move such a load above the
 wait.  On that path may be only the tables that set-up calls wrote several kernels before (twiddles,
 Box-Muller, multipliers, the sqrt(P) field), and the inputs of kernels whose launch is not overlapped:
-the shell weights of X_PKADJ and g_S (g0) of k_z_adj_source_cta."""
+the shell weights of X_PKADJ, g_S (g0) of k_z_adj_source_cta, and all of k_cic_grad's."""
 import os
 import re
 
@@ -18,6 +18,13 @@ def sources():
 
 def test_read_only_loads_are_of_tables():
     src = sources()
+    # k_cic_grad and the gather that only it calls: an ordinary launch
+    p, m = src["passes.cuh"], src["misc.cu"]
+    assert m.count("cic_gather_grad<N>(") == 1 and "cic_gather_grad<N>(" not in p
+    grad = m[m.index("k_cic_grad(CicGradArgs a)"):m.index("cudaError_t launch_cic_grad_n(")]
+    gather = p[p.index("void cic_gather_grad("):p.index("// Transpose of k_z_source.")]
+    assert "cic_gather_grad<N>(" in grad and m.count("k_cic_grad<N><<<") == 1 and "launch_overlapped(k_cic_grad" not in m
+    src["misc.cu"], src["passes.cuh"] = m.replace(grad, ""), p.replace(gather, "")
     seen = set()
     for text in src.values():
         seen |= {m.group(1) for m in re.finditer(r"__ldg\(\s*(?:reinterpret_cast<[^>]*>\()?([\w.]+)", text)}
