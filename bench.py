@@ -133,12 +133,12 @@ class ClockSampler:
 # Source: profiles/kernels_256.md.  A kernel changed since its capture must be removed here
 # (its traffic is then reported as null).
 TRAFFIC_512 = {
-    "z_source": (402.749 + 52.055) * 1e6 * 8,
-    "cic": (270.239 + 45.127) * 1e6 * 8,
-    "y_phi": (204.904 + 345.829) * 1e6 * 8,
-    "x_delta": (100.718 + 224.513) * 1e6 * 8,   # k_x_tma<256, 0, 1> (sqrt(P) field form)
-    "x_source": (135.136 + 150.306) * 1e6 * 8,
-    "z_final": (201.364 + 148.753) * 1e6 * 8,
+    "z_source": (402.751 + 51.289) * 1e6 * 8,
+    "cic": (270.259 + 45.335) * 1e6 * 8,
+    "y_phi": (204.794 + 346.230) * 1e6 * 8,
+    "x_delta": (100.718 + 224.306) * 1e6 * 8,   # k_x_tma<256, 0, 1> (sqrt(P) field form)
+    "x_source": (135.137 + 150.081) * 1e6 * 8,
+    "z_final": (201.364 + 148.379) * 1e6 * 8,
 }
 
 
